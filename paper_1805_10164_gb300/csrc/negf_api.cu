@@ -654,6 +654,27 @@ uint64_t wave_bytes(const Wave& w, int prec) {
   return w.tab * 8 + (w.wt + w.l1w) * wsz + w.start * cb + 8ull * w.rows + 8ull * w.edge;
 }
 
+// Tasks per wave of negf_run when the caller leaves it open: up to eight waves (so that walks
+// overlap the next wave's build), but none so small that its block columns leave SMs idle.  A
+// task's block columns are counted against what the device holds at once (per SM two columns
+// of W > 32: one CTA of a column pair; eight of 16 < W <= 32: four CTAs; about 96 of W <= 16:
+// one-warp CTAs of up to three columns), and a wave gets at least four such fillings, so that
+// its last, partly empty round is a small share.  Measured (GB300, ms per call, an eighth of the
+// tasks per wave against one wave): W=64 x L=100, 8 energies 28.5 -> 11.1, 32 energies
+// 29.7 -> 21.1; W=40 x L=50, 16 tasks 28.0 -> 12.8; W=32 x L=100, 32 energies 12.9 -> 8.4;
+// W=10 x L=50, 64 energies 2.50 -> 1.78 (FP64 13.9 -> 6.6).  Batches whose eighths fill the
+// device several times over keep them: 1280 uneven tasks 271 (eighths) against 276 (one wave).
+int default_per_wave(const Plan& P, int sm_count) {
+  const int nt = (int)P.tasks.size();
+  double fill = 0.0;
+  for (const TaskDesc& d : P.tasks) {
+    const double at_once = (double)sm_count * (d.W > 32 ? 2 : d.W > 16 ? 8 : 96);
+    fill += (d.L + 2) / at_once;
+  }
+  const int waves = std::max(1, std::min(8, (int)(fill / 4.0)));
+  return std::max(1, (nt + waves - 1) / waves);
+}
+
 // Buffers shared by every wave of a batch.
 struct Persist {
   TaskDesc* d_tasks = nullptr;       // global descriptors (current assembly)
@@ -1068,7 +1089,7 @@ negf_status negf_run(negf_ctx ctx, const negf_wire* wires, int32_t n_wires,
     cudaMemGetInfo(&free_b, &total_b);
     budget = free_b / 2;
   }
-  const int per_wave = r.tasks_per_wave > 0 ? r.tasks_per_wave : std::max(1, (nt + 7) / 8);
+  const int per_wave = r.tasks_per_wave > 0 ? r.tasks_per_wave : default_per_wave(P, ctx->sm_count);
   std::vector<uint64_t> task_bytes(nt);
   for (int k = 0; k < nt; ++k) task_bytes[k] = wave_bytes(make_wave(P, k, k + 1), prec);
   std::vector<Wave> waves;
