@@ -5,9 +5,11 @@
 // row needs is produced once per (wire, energy) task:
 //   * lead_modes_kernel   - eigen self-energies Sigma_m and Gamma_m of the lead strips
 //                           (Sec. II.A lead self-energies; Sec. III.A model)
+//   * lead_block_kernel   - Phi diag(Sigma_m) Phi^T, the leads' self-energy on the sites
 //   * rgf_sweep_*_kernel  - left- and right-connected blocks g^L_k, g^R_k (one warp per task
 //                           and direction in registers for complex64 W <= 16, one CTA
-//                           otherwise; the sweep is a serial chain of W x W inversions)
+//                           otherwise, k_rgf_wide.cu for complex64; the sweep is a serial chain
+//                           of W x W inversions)
 //   * diag_*_kernel       - per slice m: G_mm by one more inversion; for the boundary slices
 //                           also G Phi, the A of every row (for the sum-rule check), the mode
 //                           weights of Eq. lead_out_probability and c_p = Tr[Gamma_p A]
@@ -17,8 +19,8 @@
 //                           emitted directly as Step 6' weights (Eq. draw_i_simult and the lead
 //                           probability of Step 6'); the two injection columns propagate G Phi
 //                           for the rows of Steps 4-5.
-// W x W block inversions are Gauss-Jordan: in registers by one warp for complex64 W <= 16, in
-// shared memory by one CTA otherwise; partial pivoting except on slices where every site
+// W x W block inversions are Gauss-Jordan: in registers by one warp for complex64 W <= 16, by
+// one CTA otherwise (gj.cuh, gj_blocked.cuh); partial pivoting except on slices where every site
 // dephases (see gj_rows).  All of it runs in the precision of the tables: complex128 for
 // NEGF_FP64, complex64 for NEGF_FP32; the lead self-energies, whose square roots are singular
 // at the sub-band edges, are FP64 in both and rounded once.
@@ -83,9 +85,36 @@ __global__ void lead_modes_kernel(const TaskDesc* __restrict__ tasks, int n_task
   }
 }
 
-// ---- CTA-wide inversions (any W <= 64; complex128, and complex64 above W = 16) -------------
-// cta_gj: the slice block sits in shared memory and is inverted in place by Gauss-Jordan (no
-// augmented identity):
+// The lead block Phi diag(sigma) Phi^T of every task (both leads alike), summed in FP64 and
+// rounded to the blocks' precision, into the last slice's slot of g^L (the left-connected block
+// of slice L - 1 is never needed).  One thread per entry a >= b, mirrored.  The sum takes W
+// dependent FP64 steps per entry; formed inside every sweep and boundary diagonal block, one
+// CTA at a time on the narrow FP64 pipe, it cost 0.2 ms of latency per kernel at W = 64.
+constexpr int kLeadBlockThreads = 64;
+
+template <typename C>
+__global__ void __launch_bounds__(kLeadBlockThreads) lead_block_kernel(
+    const TaskDesc* __restrict__ tasks, int chunks, const double* __restrict__ phig,
+    const cd* __restrict__ sig, C* __restrict__ gL) {
+  const TaskDesc& d = tasks[blockIdx.x / chunks];
+  const int W = d.W;
+  const int e = (blockIdx.x % chunks) * kLeadBlockThreads + threadIdx.x;
+  if (e >= W * (W + 1) / 2) return;
+  int a = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+  while (a * (a + 1) / 2 > e) --a;
+  while ((a + 1) * (a + 2) / 2 <= e) ++a;
+  const int b = e - a * (a + 1) / 2;
+  const double* phi = phig + d.phi_off;
+  const cd* sg = sig + d.lead_off;
+  cd acc = mk(0.0, 0.0);
+  for (int m = 0; m < W; ++m) acc = acc + (phi[a * W + m] * phi[b * W + m]) * sg[m];
+  C* lb = gL + d.g_off + (uint64_t)(d.L - 1) * W * W;
+  lb[a * W + b] = lb[b * W + a] = to_c(acc, C{});
+}
+
+// ---- CTA-wide complex128 inversions (any W <= 64) ------------------------------------------
+// cta_gj (gj.cuh): the slice block sits in shared memory and is inverted in place by
+// Gauss-Jordan (no augmented identity):
 //   pivot k:  a_kk <- 1/a_kk;  a_kj <- a_kj / a_kk;  a_ik <- -a_ik / a_kk;
 //             a_ij <- a_ij - (a_ik / a_kk) a_kj            (i, j != k)
 // with two barriers per pivot: the pivot row (1/a_kk formed once, in a_kk's slot) and the
@@ -94,11 +123,10 @@ __global__ void lead_modes_kernel(const TaskDesc* __restrict__ tasks, int n_task
 // ... (R = threads / W), so that a warp touches consecutive entries of one row.  On a
 // slice where every site dephases no pivot search is needed (see gj_rows); otherwise rows are
 // interchanged by partial pivoting and the inverse's columns unscrambled at the end.  The
-// diagonal blocks use it, and the sweeps on slices with an undephased site.
+// diagonal blocks use it, and every sweep on slices with an undephased site.
 //
-// The complex64 sweeps above W = 16 (rgf_sweep_cta_kernel) run it on the block in shared
-// memory with 1024 threads.  The complex128 sweeps (rgf_sweep_rows_kernel) keep the block in
-// registers instead: thread t owns column j = t mod W of rows g, g + RG, g + 2 RG, ...
+// The sweeps (rgf_sweep_rows_kernel) keep the block in registers instead: thread t owns column
+// j = t mod W of rows g, g + RG, g + 2 RG, ...
 // (g = t / W, RG = ceil(W / RPT) row groups of at most RPT rows), and a pivot costs one
 // barrier: the owners of row k publish it, the owners of column k publish that column, and the
 // owner of a_kk publishes 1/a_kk, into one of two buffers (alternating with k, so that the next
@@ -107,16 +135,14 @@ __global__ void lead_modes_kernel(const TaskDesc* __restrict__ tasks, int n_task
 // once per pivot instead of once per thread.  The next slice's matrix E - H - Sigma_s - t^2 g_k
 // is formed in the same registers while g_k is stored.
 constexpr int kSweepThreads = 256;       // diagonal blocks: many CTAs
-constexpr int kSweepCtaThreads = 1024;   // complex64 sweeps: few serial chains, one CTA per SM
 constexpr int kSweepRowsThreads = 256;   // complex128 sweeps
 constexpr int kSweepRegMaxW = 16;        // complex64 sweeps up to this width: one warp each
 
 template <typename C>
 __host__ __device__ inline size_t sweep_rows_bytes(int W) {
-  // A W x W | pivot rows 2 x 64 | pivot columns 2 x 64 | 1/pivot 2 (complex) | phi W x W
-  // double | perm 64, flag (int)
-  return sizeof(C) * (size_t)(W * W + 4 * 64 + 2) + sizeof(double) * (size_t)(W * W) +
-         sizeof(int) * (size_t)(64 + 2);
+  // A W x W | pivot rows 2 x 64 | pivot columns 2 x 64 | 1/pivot 2 (complex) | perm 64, flag
+  // (int)
+  return sizeof(C) * (size_t)(W * W + 4 * 64 + 2) + sizeof(int) * (size_t)(64 + 2);
 }
 
 // In-place inverse of the register-held block (see above; no pivot search: the caller takes
@@ -178,9 +204,7 @@ __device__ bool gj_regcols(C (&a)[RPT], int W, int RG, int g, int j, bool own, C
 
 template <typename C, int RPT>
 __device__ __forceinline__ void sweep_rows_body(const TaskDesc& d, int dir,
-                                               const double* __restrict__ wire,
-                                               const double* __restrict__ phig,
-                                               const cd* __restrict__ sig, C* gL, C* gR,
+                                               const double* __restrict__ wire, C* gL, C* gR,
                                                int32_t* err, unsigned char* smem_raw) {
   using R = typename Real<C>::T;
   const int W = d.W, L = d.L, WW = W * W;
@@ -192,26 +216,21 @@ __device__ __forceinline__ void sweep_rows_body(const TaskDesc& d, int dir,
   C* rowk = A + WW;
   C* fcol = rowk + 2 * 64;
   C* sinv = fcol + 2 * 64;
-  double* phi = reinterpret_cast<double*>(sinv + 2);
-  int* perm = reinterpret_cast<int*>(phi + WW);
+  int* perm = reinterpret_cast<int*>(sinv + 2);
   int* flag = perm + 64;
   const double* onsite = wire + d.onsite_off;
   const double* eta = onsite + d.n;
-  const cd* sg = sig + d.lead_off;
-  for (int idx = tid; idx < WW; idx += nth) phi[idx] = phig[d.phi_off + idx];
-  __syncthreads();
-  // first slice of the sweep: E - H - Sigma_s - Phi diag(sigma) Phi^T (the lead block in FP64)
+  // first slice of the sweep: E - H - Sigma_s - the lead block
+  const C* lb = gL + d.g_off + (uint64_t)(L - 1) * WW;
   const int kf = dir == 0 ? 0 : L - 1;
   C a[RPT];
 #pragma unroll
   for (int m = 0; m < RPT; ++m) {
     const int i = g + RG * m;
     a[m] = mkc(0.0, 0.0, C{});
-    if (own && i < W) {
-      cd acc = mk(0.0, 0.0);
-      for (int q = 0; q < W; ++q) acc = acc + (phi[i * W + q] * phi[j * W + q]) * sg[q];
-      a[m] = slice_entry<C>(i, j, kf, W, d.E, d.t, onsite, eta, slice_block(d, onsite)) - to_c(acc, C{});
-    }
+    if (own && i < W)
+      a[m] = slice_entry<C>(i, j, kf, W, d.E, d.t, onsite, eta, slice_block(d, onsite)) -
+             lb[i * W + j];
   }
   C* out = dir == 0 ? gL : gR;
   const R tt = (R)(d.t * d.t);
@@ -257,8 +276,8 @@ __device__ __forceinline__ void sweep_rows_body(const TaskDesc& d, int dir,
 }
 
 __global__ void __launch_bounds__(kSweepRowsThreads) rgf_sweep_rows_kernel(
-    const TaskDesc* __restrict__ tasks, int n_tasks, const double* __restrict__ wire,
-    const double* __restrict__ phig, const cd* __restrict__ sig, cd* gL, cd* gR, int32_t* err) {
+    const TaskDesc* __restrict__ tasks, int n_tasks, const double* __restrict__ wire, cd* gL,
+    cd* gR, int32_t* err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int job = blockIdx.x;
   if (job >= 2 * n_tasks) return;
@@ -268,79 +287,11 @@ __global__ void __launch_bounds__(kSweepRowsThreads) rgf_sweep_rows_kernel(
   // rows per thread: W <= 16 -> 4, W <= 32 -> 8, W <= 64 -> 16 (at most 4 row groups, so that
   // kSweepRowsThreads = 256 threads cover every width)
   if (d.W <= 16)
-    sweep_rows_body<cd, 4>(d, dir, wire, phig, sig, gL, gR, err, smem_raw);
+    sweep_rows_body<cd, 4>(d, dir, wire, gL, gR, err, smem_raw);
   else if (d.W <= 32)
-    sweep_rows_body<cd, 8>(d, dir, wire, phig, sig, gL, gR, err, smem_raw);
+    sweep_rows_body<cd, 8>(d, dir, wire, gL, gR, err, smem_raw);
   else
-    sweep_rows_body<cd, 16>(d, dir, wire, phig, sig, gL, gR, err, smem_raw);
-}
-
-template <typename C>
-__host__ __device__ inline size_t sweep_smem_bytes(int W) {
-  // A W x W | pivot row W | multipliers W (complex) | phi W x W double | perm W, flag (int)
-  return sizeof(C) * (size_t)(W * W + 2 * W) + sizeof(double) * (size_t)(W * W) +
-         sizeof(int) * (size_t)(W + 2);
-}
-
-// complex64 sweeps of width min_W .. 64 with the block in shared memory (cta_gj)
-__global__ void __launch_bounds__(kSweepCtaThreads) rgf_sweep_cta_kernel(
-    const TaskDesc* __restrict__ tasks, int n_tasks, const double* __restrict__ wire,
-    const double* __restrict__ phig, const cd* __restrict__ sig, cf* gL, cf* gR, int32_t* err,
-    int min_W) {
-  using C = cf;
-  using R = float;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int job = blockIdx.x;
-  if (job >= 2 * n_tasks) return;
-  const TaskDesc d = tasks[job >> 1];
-  const int dir = job & 1;
-  const int W = d.W, L = d.L, WW = W * W;
-  const int tid = threadIdx.x, nth = blockDim.x;
-  if (L < 2 || W > 64 || W < min_W) return;       // narrower tasks: rgf_sweep_reg_kernel
-  C* A = reinterpret_cast<C*>(smem_raw);
-  C* rowk = A + WW;
-  C* fcol = rowk + W;
-  double* phi = reinterpret_cast<double*>(fcol + W);
-  int* perm = reinterpret_cast<int*>(phi + WW);
-  int* flag = perm + W;
-  const double* onsite = wire + d.onsite_off;
-  const double* eta = onsite + d.n;
-  const cd* sg = sig + d.lead_off;
-  for (int idx = tid; idx < WW; idx += nth) phi[idx] = phig[d.phi_off + idx];
-  __syncthreads();
-  // first slice of the sweep: E - H - Sigma_s - Phi diag(sigma) Phi^T (the lead block in FP64)
-  const int kf = dir == 0 ? 0 : L - 1;
-  for (int idx = tid; idx < WW; idx += nth) {
-    const int a = idx / W, b = idx - a * W;
-    cd acc = mk(0.0, 0.0);
-    for (int m = 0; m < W; ++m) acc = acc + (phi[a * W + m] * phi[b * W + m]) * sg[m];
-    A[idx] = slice_entry<C>(a, b, kf, W, d.E, d.t, onsite, eta, slice_block(d, onsite)) - to_c(acc, C{});
-  }
-  C* out = dir == 0 ? gL : gR;
-  const R tt = (R)(d.t * d.t);
-  for (int s = 0; s < L - 1; ++s) {
-    const int k = dir == 0 ? s : L - 1 - s;
-    const bool deph = __syncthreads_and(tid >= W || eta[k * W + tid] > 0.0);
-    if (!cta_gj(A, rowk, fcol, perm, flag, W, !deph)) {
-      if (tid == 0) atomicOr(err, ERR_SINGULAR);
-      return;
-    }
-    // store g_k; build the next slice in place: E - H - Sigma_s - t^2 g_k
-    C* dst = out + d.g_off + (uint64_t)k * WW;
-    const bool more = s + 1 < L - 1;
-    const int kn = dir == 0 ? s + 1 : L - 2 - s;
-    bool bad = false;
-    for (int idx = tid; idx < WW; idx += nth) {
-      const C v = A[idx];
-      dst[idx] = v;
-      bad |= !finite_c(v);
-      if (more) {
-        const int a = idx / W, b = idx - a * W;
-        A[idx] = slice_entry<C>(a, b, kn, W, d.E, d.t, onsite, eta, slice_block(d, onsite)) - tt * v;
-      }
-    }
-    if (__syncthreads_or(bad) && tid == 0) atomicOr(err, ERR_NONFINITE);
-  }
+    sweep_rows_body<cd, 16>(d, dir, wire, gL, gR, err, smem_raw);
 }
 
 // ---- register-resident variants for complex64 blocks with W <= 16 ------------------------
@@ -521,25 +472,18 @@ __device__ void build_col(cf (&a)[W], double E, double t, double onsite_j, doubl
   }
 }
 
-// row (= column, the block is symmetric) j of the lead block Phi diag(sig) Phi^T (lanes j < W)
-template <int MAXW>
-__device__ void lead_col(const double* phi, const cd* sig, int W, cf (&x)[MAXW]) {
+// column (lane < W) of the lead block at lb; other lanes get zeros
+template <int W>
+__device__ __forceinline__ void lead_col(const cf* lb, cf (&x)[W]) {
   const int j = threadIdx.x & 31;
 #pragma unroll
-  for (int i = 0; i < MAXW; ++i) {
-    cd acc = mk(0.0, 0.0);
-    if (i < W && j < W)
-      for (int m = 0; m < W; ++m) acc = acc + (phi[i * W + m] * phi[j * W + m]) * sig[m];
-    x[i] = cf{(float)acc.x, (float)acc.y};
-  }
+  for (int i = 0; i < W; ++i) x[i] = j < W ? lb[i * W + j] : cf{0.f, 0.f};
 }
 
 // One sweep (task d, direction dir) with W == MAXW known at compile time.
 template <int MAXW>
 __device__ __forceinline__ void sweep_reg_body(const TaskDesc& d, int dir,
-                                               const double* __restrict__ wire,
-                                               const double* __restrict__ phig,
-                                               const cd* __restrict__ sig, cf* gL, cf* gR,
+                                               const double* __restrict__ wire, cf* gL, cf* gR,
                                                int32_t* err, cf* srow) {
   constexpr int W = MAXW;
   const int L = d.L;
@@ -548,7 +492,7 @@ __device__ __forceinline__ void sweep_reg_body(const TaskDesc& d, int dir,
   const double* eta = onsite + d.n;
   const float ttf = (float)(d.t * d.t);     // FP32 on the serial path (FP64 is slow here)
   cf x[MAXW], a[MAXW];
-  lead_col<MAXW>(phig + d.phi_off, sig + d.lead_off, W, x);   // column j of the lead block
+  lead_col<W>(gL + d.g_off + (uint64_t)(L - 1) * W * W, x);
   cf* out = dir == 0 ? gL : gR;
   const int jc = lane < W ? lane : 0;
   // the next slice's onsite energy and dephasing are fetched one step ahead
@@ -616,15 +560,14 @@ struct SweepReg {
 
 // One warp per (task, direction), tasks of width W <= kSweepRegMaxW.
 __global__ void rgf_sweep_reg_kernel(const TaskDesc* __restrict__ tasks, int n_tasks,
-                                     const double* __restrict__ wire,
-                                     const double* __restrict__ phig, const cd* __restrict__ sig,
-                                     cf* gL, cf* gR, int32_t* err) {
+                                     const double* __restrict__ wire, cf* gL, cf* gR,
+                                     int32_t* err) {
   const int job = blockIdx.x;
   if (job >= 2 * n_tasks) return;
   __shared__ __align__(16) cf s_row[34];
   const TaskDesc d = tasks[job >> 1];
   if (d.L < 2) return;
-  by_width<SweepReg>(d.W, d, job & 1, wire, phig, sig, gL, gR, err, s_row);
+  by_width<SweepReg>(d.W, d, job & 1, wire, gL, gR, err, s_row);
 }
 
 // last task whose first job index (`first(t)`) is <= job
@@ -638,31 +581,30 @@ __device__ __forceinline__ int find_task(int n_tasks, uint32_t job, F first) {
   return lo;
 }
 
-// CTA-wide diagonal blocks (any W <= 64): one CTA of kSweepThreads threads per (task, y); same
-// outputs as diag_kernel, with the inversion of cta_gj.
-template <typename C>
+// CTA-wide complex128 diagonal blocks: one CTA of kSweepThreads threads per (task, y); same
+// outputs as diag_reg_kernel, with the inversion of cta_gj.
 __host__ __device__ inline size_t diag_cta_bytes(int W) {
-  // A, S (lead block, then start block) W x W | pivot row, multipliers W (complex) | phi W x W
-  // double | mode weights W double | perm W, flag (int)
-  return sizeof(C) * (size_t)(2 * W * W + 2 * W) + sizeof(double) * (size_t)(W * W + W) +
+  // A, S (start block) W x W | pivot row, multipliers W (complex) | phi W x W double | mode
+  // weights W double | perm W, flag (int)
+  return sizeof(cd) * (size_t)(2 * W * W + 2 * W) + sizeof(double) * (size_t)(W * W + W) +
          sizeof(int) * (size_t)(W + 2);
 }
 
-template <typename C>
 __global__ void __launch_bounds__(kSweepThreads) diag_cta_kernel(
     const TaskDesc* __restrict__ tasks, int n_tasks, uint32_t n_jobs,
-    const double* __restrict__ wire, const double* __restrict__ phig, const cd* __restrict__ sig,
-    const double* __restrict__ gam, const C* __restrict__ gL, const C* __restrict__ gR,
-    C* __restrict__ start, double* __restrict__ rowsum, double* __restrict__ mode_w,
-    double* __restrict__ cvals, int32_t* err, int min_W) {
-  using R = typename Real<C>::T;
+    const double* __restrict__ wire, const double* __restrict__ phig,
+    const double* __restrict__ gam, const cd* __restrict__ gL, const cd* __restrict__ gR,
+    cd* __restrict__ start, double* __restrict__ rowsum, double* __restrict__ mode_w,
+    double* __restrict__ cvals, int32_t* err) {
+  using C = cd;
+  using R = double;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const uint32_t job = blockIdx.x;
   if (job >= n_jobs) return;
   const int task = find_task(n_tasks, job, [&](int t) { return tasks[t].col_base; });
   const TaskDesc d = tasks[task];
   const int W = d.W, L = d.L, n = d.n, WW = W * W;
-  if (W > 64 || W < min_W) return;                // narrower tasks: diag_reg_kernel
+  if (W > 64) return;
   const int tid = threadIdx.x, nth = blockDim.x;
   const int y = (int)(job - d.col_base);
   const bool inj = y >= L;
@@ -681,25 +623,15 @@ __global__ void __launch_bounds__(kSweepThreads) diag_cta_kernel(
   const R tt = (R)(d.t * d.t);
   const bool lead_l = m0 == 0, lead_r = m0 == L - 1;
   for (int idx = tid; idx < WW; idx += nth) phi[idx] = phig[d.phi_off + idx];
-  __syncthreads();
-  if (lead_l || lead_r) {
-    const cd* sg = sig + d.lead_off;
-    for (int idx = tid; idx < WW; idx += nth) {
-      const int a = idx / W, b = idx - a * W;
-      cd acc = mk(0.0, 0.0);
-      for (int m = 0; m < W; ++m) acc = acc + (phi[a * W + m] * phi[b * W + m]) * sg[m];
-      S[idx] = to_c(acc, C{});
-    }
-  }
-  __syncthreads();
   // A = E - H - Sigma_s - (lead block or t^2 g^L_{m-1}) - (lead block or t^2 g^R_{m+1})
+  const C* lb = gL + d.g_off + (uint64_t)(L - 1) * WW;
   const C* gl = lead_l ? nullptr : gL + d.g_off + (uint64_t)(m0 - 1) * WW;
   const C* gr = lead_r ? nullptr : gR + d.g_off + (uint64_t)(m0 + 1) * WW;
   for (int idx = tid; idx < WW; idx += nth) {
     const int a = idx / W, b = idx - a * W;
     C v = slice_entry<C>(a, b, m0, W, d.E, d.t, onsite, eta, slice_block(d, onsite));
-    v = v - (gl ? tt * gl[idx] : S[idx]);
-    v = v - (gr ? tt * gr[idx] : S[idx]);
+    v = v - (gl ? tt * gl[idx] : lb[idx]);
+    v = v - (gr ? tt * gr[idx] : lb[idx]);
     A[idx] = v;
   }
   const bool deph = __syncthreads_and(tid >= W || eta[m0 * W + tid] > 0.0);
@@ -753,7 +685,6 @@ template <int MAXW>
 __device__ __forceinline__ void diag_reg_body(const TaskDesc& d, int task, uint32_t job,
                                               const double* __restrict__ wire,
                                               const double* __restrict__ phig,
-                                              const cd* __restrict__ sig,
                                               const double* __restrict__ gam,
                                               const cf* __restrict__ gL,
                                               const cf* __restrict__ gR, cf* __restrict__ start,
@@ -776,7 +707,7 @@ __device__ __forceinline__ void diag_reg_body(const TaskDesc& d, int task, uint3
   cf x[MAXW], a[MAXW];
   const bool lead_l = m0 == 0, lead_r = m0 == L - 1;
   if (lead_l || lead_r) {
-    lead_col<MAXW>(phig + d.phi_off, sig + d.lead_off, W, x);
+    lead_col<W>(gL + d.g_off + (uint64_t)(L - 1) * W * W, x);
     if (lead_l && lead_r) {
 #pragma unroll
       for (int i = 0; i < MAXW; ++i) x[i] = 2.f * x[i];
@@ -859,12 +790,12 @@ struct DiagReg {
 };
 
 // Register-resident diagonal blocks (complex64, W <= 16), one warp per column job; same outputs
-// as diag_kernel.  Shared memory per warp: G (W x W complex64), phi (W x W double), the mode
+// as diag_cta_kernel.  Shared memory per warp: G (W x W complex64), phi (W x W double), the mode
 // weights.
 __global__ void diag_reg_kernel(const TaskDesc* __restrict__ tasks, int n_tasks, uint32_t n_jobs,
                                 const double* __restrict__ wire, const double* __restrict__ phig,
-                                const cd* __restrict__ sig, const double* __restrict__ gam,
-                                const cf* __restrict__ gL, const cf* __restrict__ gR,
+                                const double* __restrict__ gam, const cf* __restrict__ gL,
+                                const cf* __restrict__ gR,
                                 cf* __restrict__ start, double* __restrict__ rowsum,
                                 double* __restrict__ mode_w, double* __restrict__ cvals,
                                 int32_t* err) {
@@ -877,7 +808,7 @@ __global__ void diag_reg_kernel(const TaskDesc* __restrict__ tasks, int n_tasks,
   if (job >= n_jobs) return;
   const int task = find_task(n_tasks, job, [&](int t) { return tasks[t].col_base; });
   const TaskDesc d = tasks[task];
-  by_width<DiagReg>(d.W, d, task, job, wire, phig, sig, gam, gL, gR, start, rowsum, mode_w,
+  by_width<DiagReg>(d.W, d, task, job, wire, phig, gam, gL, gR, start, rowsum, mode_w,
                     cvals, err, s_G[warp], s_phi[warp], s_mw[warp], s_row[warp]);
 }
 
@@ -1019,46 +950,34 @@ int chain_max(int max_W) {
 }
 
 template <typename C>
-cudaError_t sweep_impl(const TaskDesc* d_tasks, int n_tasks, int max_W, const double* d_wire,
-                       const double* d_phi, const cd* d_sig, C* d_gL, C* d_gR, int32_t* d_err,
-                       cudaStream_t s);
+cudaError_t lead_blocks(const TaskDesc* d_tasks, int n_tasks, int max_W, const double* d_phi,
+                        const cd* d_sig, C* d_gL, cudaStream_t s) {
+  const int chunks = (max_W * (max_W + 1) / 2 + kLeadBlockThreads - 1) / kLeadBlockThreads;
+  lead_block_kernel<C><<<(unsigned)(n_tasks * chunks), kLeadBlockThreads, 0, s>>>(
+      d_tasks, chunks, d_phi, d_sig, d_gL);
+  return cudaGetLastError();
+}
 
-template <>
-cudaError_t sweep_impl<cf>(const TaskDesc* d_tasks, int n_tasks, int max_W,
-                           const double* d_wire, const double* d_phi, const cd* d_sig, cf* d_gL,
-                           cf* d_gR, int32_t* d_err, cudaStream_t s);
-
-template <>
-cudaError_t sweep_impl<cd>(const TaskDesc* d_tasks, int n_tasks, int max_W,
-                           const double* d_wire, const double* d_phi, const cd* d_sig, cd* d_gL,
-                           cd* d_gR, int32_t* d_err, cudaStream_t s) {
+cudaError_t sweep_fp64(const TaskDesc* d_tasks, int n_tasks, int max_W, const double* d_wire,
+                       cd* d_gL, cd* d_gR, int32_t* d_err, cudaStream_t s) {
   // one CTA per sweep: each sweep is a serial chain of W x W inversions, spread one per SM
   const size_t smem = sweep_rows_bytes<cd>(max_W);
   cudaError_t e = cudaFuncSetAttribute(rgf_sweep_rows_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  rgf_sweep_rows_kernel<<<2 * n_tasks, kSweepRowsThreads, smem, s>>>(
-      d_tasks, n_tasks, d_wire, d_phi, d_sig, d_gL, d_gR, d_err);
+  rgf_sweep_rows_kernel<<<2 * n_tasks, kSweepRowsThreads, smem, s>>>(d_tasks, n_tasks, d_wire,
+                                                                     d_gL, d_gR, d_err);
   return cudaGetLastError();
 }
 
-template <>
-cudaError_t sweep_impl<cf>(const TaskDesc* d_tasks, int n_tasks, int max_W,
-                           const double* d_wire, const double* d_phi, const cd* d_sig, cf* d_gL,
-                           cf* d_gR, int32_t* d_err, cudaStream_t s) {
-  // one warp per sweep for the tasks of width <= 32 (it skips wider ones), a CTA per sweep for
+cudaError_t sweep_fp32(const TaskDesc* d_tasks, int n_tasks, int max_W, const double* d_wire,
+                       cf* d_gL, cf* d_gR, int32_t* d_err, cudaStream_t s) {
+  // one warp per sweep for the tasks of width <= 16 (it skips wider ones), a CTA per sweep for
   // the rest
-  rgf_sweep_reg_kernel<<<2 * n_tasks, 32, 0, s>>>(d_tasks, n_tasks, d_wire, d_phi, d_sig, d_gL,
-                                                  d_gR, d_err);
+  rgf_sweep_reg_kernel<<<2 * n_tasks, 32, 0, s>>>(d_tasks, n_tasks, d_wire, d_gL, d_gR, d_err);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || max_W <= kSweepRegMaxW) return e;
-  const size_t smem = sweep_smem_bytes<cf>(max_W);
-  e = cudaFuncSetAttribute(rgf_sweep_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-  if (e != cudaSuccess) return e;
-  rgf_sweep_cta_kernel<<<2 * n_tasks, kSweepCtaThreads, smem, s>>>(
-      d_tasks, n_tasks, d_wire, d_phi, d_sig, d_gL, d_gR, d_err, kSweepRegMaxW + 1);
-  return cudaGetLastError();
+  return launch_rgf_sweep_wide(d_tasks, n_tasks, max_W, d_wire, d_gL, d_gR, d_err, s);
 }
 
 template <typename C>
@@ -1077,20 +996,22 @@ cudaError_t columns_impl(const TaskDesc* d_tasks, int n_tasks, uint32_t n_cols, 
     const cf* gl = reinterpret_cast<const cf*>(d_gL);
     const cf* gr = reinterpret_cast<const cf*>(d_gR);
     cf* st = reinterpret_cast<cf*>(d_start);
-    diag_reg_kernel<<<blocks, 32 * warps, 0, s>>>(d_tasks, n_tasks, n_cols, d_wire, d_phi, d_sig,
-                                                  d_gam, gl, gr, st, d_rowsum, d_mode_w, d_c,
-                                                  d_err);
+    diag_reg_kernel<<<blocks, 32 * warps, 0, s>>>(d_tasks, n_tasks, n_cols, d_wire, d_phi, d_gam,
+                                                  gl, gr, st, d_rowsum, d_mode_w, d_c, d_err);
     cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && max_W > 16)
+      e = launch_diag_wide(d_tasks, n_tasks, n_cols, max_W, d_wire, d_phi, d_gam, gl, gr, st,
+                           d_rowsum, d_mode_w, d_c, d_err, s);
     if (e != cudaSuccess) return e;
-  }
-  if (sizeof(C) != sizeof(cf) || max_W > 16) {
-    const size_t smem = diag_cta_bytes<C>(max_W);
-    cudaError_t e = cudaFuncSetAttribute(diag_cta_kernel<C>,
+  } else {
+    const size_t smem = diag_cta_bytes(max_W);
+    cudaError_t e = cudaFuncSetAttribute(diag_cta_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    diag_cta_kernel<C><<<n_cols, kSweepThreads, smem, s>>>(
-        d_tasks, n_tasks, n_cols, d_wire, d_phi, d_sig, d_gam, d_gL, d_gR, d_start, d_rowsum,
-        d_mode_w, d_c, d_err, sizeof(C) == sizeof(cf) ? 17 : 1);
+    diag_cta_kernel<<<n_cols, kSweepThreads, smem, s>>>(
+        d_tasks, n_tasks, n_cols, d_wire, d_phi, d_gam, reinterpret_cast<const cd*>(d_gL),
+        reinterpret_cast<const cd*>(d_gR), reinterpret_cast<cd*>(d_start), d_rowsum, d_mode_w,
+        d_c, d_err);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -1132,11 +1053,17 @@ cudaError_t launch_rgf_sweep(const TaskDesc* d_tasks, int n_tasks, int max_W, in
                              const double* d_wire, const double* d_phi, const cd* d_sig,
                              void* d_gL, void* d_gR, int32_t* d_err, cudaStream_t s) {
   if (n_tasks == 0) return cudaSuccess;
-  if (precision == NEGF_FP64)
-    return sweep_impl<cd>(d_tasks, n_tasks, max_W, d_wire, d_phi, d_sig,
-                          static_cast<cd*>(d_gL), static_cast<cd*>(d_gR), d_err, s);
-  return sweep_impl<cf>(d_tasks, n_tasks, max_W, d_wire, d_phi, d_sig, static_cast<cf*>(d_gL),
-                        static_cast<cf*>(d_gR), d_err, s);
+  cudaError_t e;
+  if (precision == NEGF_FP64) {
+    e = lead_blocks(d_tasks, n_tasks, max_W, d_phi, d_sig, static_cast<cd*>(d_gL), s);
+    return e != cudaSuccess ? e
+                            : sweep_fp64(d_tasks, n_tasks, max_W, d_wire, static_cast<cd*>(d_gL),
+                                         static_cast<cd*>(d_gR), d_err, s);
+  }
+  e = lead_blocks(d_tasks, n_tasks, max_W, d_phi, d_sig, static_cast<cf*>(d_gL), s);
+  return e != cudaSuccess ? e
+                          : sweep_fp32(d_tasks, n_tasks, max_W, d_wire, static_cast<cf*>(d_gL),
+                                       static_cast<cf*>(d_gR), d_err, s);
 }
 
 cudaError_t launch_block_columns(const TaskDesc* d_tasks, int n_tasks, uint32_t n_cols,

@@ -111,12 +111,22 @@ cudaError_t launch_lead_modes(const TaskDesc* d_tasks, int n_tasks, int max_W,
                               const double* d_wire, double* d_phi, float* d_phi32,
                               float* d_eta32, cd* d_sig, double* d_gam, int32_t* d_err,
                               cudaStream_t s);
+// RGF sweeps of every task, after the lead blocks (the last slice's slot of g^L holds the task's
+// lead block Phi diag(sigma) Phi^T, which the diagonal blocks read too).
 // RGF blocks, start blocks: complex128 [..] for NEGF_FP64, complex64 for NEGF_FP32 (the lead
 // self-energies stay FP64 in both).  block_bytes() gives the element size.
 inline size_t block_bytes(int precision) { return precision == NEGF_FP64 ? 16 : 8; }
 cudaError_t launch_rgf_sweep(const TaskDesc* d_tasks, int n_tasks, int max_W, int precision,
                              const double* d_wire, const double* d_phi, const cd* d_sig,
                              void* d_gL, void* d_gR, int32_t* d_err, cudaStream_t s);
+// Complex64 sweeps and diagonal blocks of the tasks wider than 16 sites (k_rgf_wide.cu).
+cudaError_t launch_rgf_sweep_wide(const TaskDesc* d_tasks, int n_tasks, int max_W,
+                                  const double* d_wire, cf* d_gL, cf* d_gR, int32_t* d_err,
+                                  cudaStream_t s);
+cudaError_t launch_diag_wide(const TaskDesc* d_tasks, int n_tasks, uint32_t n_cols, int max_W,
+                             const double* d_wire, const double* d_phi, const double* d_gam,
+                             const cf* d_gL, const cf* d_gR, cf* d_start, double* d_rowsum,
+                             double* d_mode_w, double* d_c, int32_t* d_err, cudaStream_t s);
 // Diagonal blocks (start blocks, A per row, mode weights, c_p) then the block-column chains
 // emitting the weights.  n_cols = sum over tasks of L + 2.  On return rowsum holds A of every
 // table row and c_p in the two mode-row slots; the alias build replaces them by the row sums.
