@@ -3,11 +3,20 @@
 // G_{k,m} = -t g^R_k G_{k-1,m} towards slice L - 1, each block emitted as the Step 6' weights
 // w_{(m,b),(k,a)} = eta_{k,a} |G_{k,m}[a][b]|^2 of the column's W rows (Eq. draw_i_simult) and,
 // at the boundary slices, the lead weights <psi_b|Gamma|psi_b> = sum_nu Gamma_nu
-// |(Phi^T G_{k,m})_{nu b}|^2.  Same weights as chain_kernel (one warp per column), computed
-// by 512 threads with the two columns side by side: X_k [64][128] = (-t g_k) [64][64] X_{k+1}
-// in shared memory, FP32 fused multiply-adds, each thread a 4 x 4 block of outputs (four warps
-// per scheduler to hide the shared-memory and dependency latencies).
+// |(Phi^T G_{k,m})_{nu b}|^2.  Same weights as chain_kernel (one warp per column), the two
+// columns side by side: X_k [64][128] = (-t g_k) [64][64] X_{k+1} in shared memory.
 //
+// What bounds it: the FP32 multiply-add pipe (64 x 64 x 128 complex products a step, 16,384
+// cycles of an SM's 128 lanes).  One set of warps that first multiplies and then emits left that
+// pipe idle for half of a step, so the CTA's 16 warps have two roles:
+//   * warps 0..7 multiply.  A lane holds 8 x 4 outputs as (re, im) pairs and uses the paired
+//     multiply-add (fma.rn.f32x2), which does not raise the pipe's rate but takes half the
+//     issue slots, so that the other warps' instructions fit between.  (-t g) lies in shared
+//     memory with every value twice, (x, x, y, y), so that a pair operand is one half of a
+//     16-byte load; X's swapped pair (-im, re) is made in registers, twice per eight uses;
+//   * warps 8..15 emit the block of the step before meanwhile, and bring in the next g.
+// X is overwritten in place between two barriers at the end of a step, together with |X|^2
+// (FP32, N below), from which the emitting warps form every weight.
 // W = 64 uses the symmetry G = G^T (H real symmetric, every self-energy a complex symmetric
 // matrix), which halves the products: only the chains towards slice 0 run (and the one of the
 // lead-L injection column towards slice L - 1).  A block G_{k,m} (k < m) of site column m gives
@@ -25,6 +34,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "level2.cuh"
 #include "negf_internal.cuh"
 
@@ -34,16 +45,74 @@ namespace {
 constexpr int kW = 64;
 constexpr int kN = 2 * kW;                    // two columns side by side
 constexpr int kThreads = 512;
-constexpr int kWtPitch = kW + 1;              // padded row of the weight staging
-// Gs, the X ping-pong pair, the weights staging and (level-2 blocks built in the kernel) the
-// staging of the transposed rows' weights
-constexpr size_t kSmem = sizeof(cf) * (kW * kW + 2 * kW * kN) + 2 * sizeof(float) * kN * kWtPitch;
+constexpr int kMul = 256;                     // threads of the multiplying warps
+constexpr int kNPitch = kN + 1;               // row pitch of N
 constexpr int kB2 = 8 + kW;                   // level-2 block of a 64-site slice: guide + octets
+constexpr int kSP = kB2 + 4;                  // its pitch in the staging: 16-byte aligned, and
+                                              // eight blocks start on different banks
+// X, two g blocks (doubled values), N
+constexpr size_t kSmem = sizeof(cf) * kW * kN + 2 * sizeof(float4) * kW * kW +
+                         sizeof(float) * kW * kNPitch;
 
 // eta |G|^2 with every rounding explicit, so that the weight of a (row, site) pair has the same
 // bits wherever it is formed (stored weights, or a level-2 block built in the kernel)
-__device__ __forceinline__ float wsq(float e, cf v) {
-  return __fmul_rn(e, __fadd_rn(__fmul_rn(v.x, v.x), __fmul_rn(v.y, v.y)));
+__device__ __forceinline__ float nsq(cf v) {
+  return __fadd_rn(__fmul_rn(v.x, v.x), __fmul_rn(v.y, v.y));
+}
+
+typedef unsigned long long f2;                // two floats: a register pair
+__device__ __forceinline__ f2 pack2(float lo, float hi) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ ulonglong2 lds2(const void* p) {
+  return *reinterpret_cast<const ulonglong2*>(p);
+}
+
+// Element (a, b') of N.  The column is permuted within groups of 32 so that the emitting
+// lanes, eight rows (or columns) by four chunks of 16, read 32 different banks either way.
+__device__ __forceinline__ int n_at(int a, int bp) {
+  return a * kNPitch + (bp ^ (((bp >> 5) & 1) << 3) ^ (((a >> 4) & 3) << 3));
+}
+// Element (a, c) of the doubled -t g: the lanes that write a row and those that read a column
+// take different banks.
+__device__ __forceinline__ int g_at(int a, int c) { return c * kW + (a ^ (c & 7)); }
+
+// shared -> global copy of `bytes` (a multiple of 16, both ends 16-byte aligned) by the TMA
+// engine, in the calling thread's bulk group
+__device__ __forceinline__ void bulk_store(void* gmem, const void* smem, unsigned bytes) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(gmem), "r"(sa),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;\n" ::: "memory"); }
+template <int kPending>
+__device__ __forceinline__ void bulk_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;\n" ::"n"(kPending) : "memory");
+}
+__device__ __forceinline__ void fence_async_shared() {
+  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+}
+// the emitting warps' own barrier
+__device__ __forceinline__ void emit_sync() {
+  asm volatile("bar.sync 1, %0;\n" ::"n"(kThreads - kMul) : "memory");
+}
+
+// the whole CTA, the two roles from their own code
+__device__ __forceinline__ void step_sync() {
+  asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory");
 }
 
 __global__ void __launch_bounds__(kThreads, 1) chain_cta_kernel(
@@ -53,13 +122,13 @@ __global__ void __launch_bounds__(kThreads, 1) chain_cta_kernel(
     const cf* __restrict__ start, float* __restrict__ weights, uint64_t* __restrict__ tab,
     int32_t* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char smem[];
-  cf* Gs = reinterpret_cast<cf*>(smem);                    // [a][c]; also Phi at the edges
-  cf* Xa = Gs + kW * kW;                                   // [c][b'] ping
-  cf* Xb = Xa + kW * kN;                                   // [c][b'] pong
-  float* Wt = reinterpret_cast<float*>(Xb + kW * kN);      // [b'][a] weights staging
-  float* Wt2 = Wt + kN * kWtPitch;                         // fused: transposed rows [r][b]
+  cf* X = reinterpret_cast<cf*>(smem);                     // [c][b']
+  float4* G0 = reinterpret_cast<float4*>(X + kW * kN);     // two (-t g) blocks, g_at
+  float* N = reinterpret_cast<float*>(G0 + 2 * kW * kW);   // |X|^2, n_at
 
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const bool mul = tid < kMul;
+  const int ew = (tid - kMul) >> 5;                        // emitting warp 0..7
   const TcJob job = jobs[blockIdx.x];
   const TaskDesc d = tasks[job.task];
   const int L = d.L, n = d.n, K = d.K;
@@ -77,243 +146,94 @@ __global__ void __launch_bounds__(kThreads, 1) chain_cta_kernel(
   auto row_of = [&](int y, int b) -> uint64_t {
     return y < L ? (uint64_t)y * kW + b : (uint64_t)n + (uint64_t)(y - L) * kW + b;
   };
-  // fused: the level-2 blocks of a step, one per pair of adjacent threads (block bi = tid / 2,
-  // half h = tid % 2: the block's weights wrow[0..63], the pair's `have`, row and slice), their
-  // thresholds in registers (level2_fp32_pair); staged in shared memory 128 at a time (the two
-  // weight stagings, free once read) and written block by block, 18 lanes per 288-byte block,
-  // so that the stores stay contiguous
-  uint64_t* blk_row = reinterpret_cast<uint64_t*>(Gs);     // Gs is free outside the product
-  int* blk_slice = reinterpret_cast<int*>(blk_row + kN);
-  auto put_blocks = [&](bool have, uint64_t row, int slice, const float* wrow) {
-    const int h = tid & 1, bi = tid >> 1;
-    uint32_t c[32];
+  // Fused: the level-2 blocks of 64 rows (row0 + r) towards `slice` from 64 weights each,
+  // e(i) N(r, i); emitting warp ew builds rows 8 ew .. 8 ew + 7, lane (q, r) chunk q of row
+  // 8 ew + r, stages the blocks in stg (this warp's) and sends each off as one bulk copy.
+  auto put_blocks = [&](uint32_t* stg, const float* e, uint64_t row0, int slice, auto norm) {
+    const int q = lane >> 3, r = lane & 7;
+    float w[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      w[i] = __fmul_rn(__ldg(e + 16 * q + i), norm(8 * ew + r, 16 * q + i));
+    uint32_t c[16];
     float tot = 0.f;
-    const bool ok = level2_fp32_pair([&](int a) { return wrow[32 * h + a]; }, h, c, &tot);
-    if (have) bad |= !ok;
-    __syncthreads();                                       // every weight row has been read
-    // 2 x 128 x 65 >= 128 x 76 words; pitch 76 (not 72): 16-byte stores of neighbouring
-    // blocks start on different bank groups
-    constexpr int kSP = kB2 + 4;
-    uint32_t* stage = reinterpret_cast<uint32_t*>(Wt);
-    for (int half = 0; half < 2; ++half) {
-      const int b = bi & (kN - 1);
-      if ((bi >> 7) == half) {
-        if (h == 0) {
-          blk_row[b] = have ? row : ~0ull;
-          blk_slice[b] = slice;
-          if (have) l1[row * (L + 2) + slice] = tot;
-        }
-        if (have) {
-          uint32_t* dst = stage + b * kSP;
-          // guide: the last threshold of octets 0..6 (octet 7's is 2^31); lane h holds octets
-          // 4h .. 4h + 3
-          *reinterpret_cast<uint4*>(dst + 4 * h) =
-              make_uint4(c[7], c[15], c[23], h == 0 ? c[31] : kCdfOne);
+    bad |= !level2_fp32_quad(w, q, c, &tot);
+    const uint64_t row = row0 + 8 * ew + r;
+    if (q == 3) c[15] = kCdfOne;                           // the slice's last threshold
+    uint32_t* dst = stg + r * kSP;
+    *reinterpret_cast<uint2*>(dst + 2 * q) = make_uint2(c[7], c[15]);
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
-            *reinterpret_cast<uint4*>(dst + 8 + 32 * h + 4 * i) =
-                make_uint4(c[4 * i], c[4 * i + 1], c[4 * i + 2],
-                           (h == 1 && i == 7) ? kCdfOne : c[4 * i + 3]);
-        }
-      }
-      __syncthreads();
-      for (int i = tid; i < kN * (kB2 / 4); i += kThreads) {
-        const int bb = i / (kB2 / 4), q = i - bb * (kB2 / 4);
-        const uint64_t r = blk_row[bb];
-        if (r != ~0ull)
-          *reinterpret_cast<uint4*>(l2 + (r * L + blk_slice[bb]) * kB2 + 4 * q) =
-              *reinterpret_cast<const uint4*>(stage + bb * kSP + 4 * q);
-      }
-      __syncthreads();
+    for (int i = 0; i < 4; ++i)
+      *reinterpret_cast<uint4*>(dst + 8 + 16 * q + 4 * i) =
+          make_uint4(c[4 * i], c[4 * i + 1], c[4 * i + 2], c[4 * i + 3]);
+    fence_async_shared();
+    __syncwarp();
+    if (q == 0) {
+      l1[row * (L + 2) + slice] = tot;
+      bulk_store(l2 + (row * L + slice) * kB2, dst, kB2 * 4);
+      bulk_commit();
     }
   };
-  // start block of column slot col into X[:, col*64 .. col*64+63]
-  auto load_start = [&](cf* X, int col) {
-    const cf* st = start + d.start_off + (uint64_t)ys[col] * kW * kW;
-    for (int i = tid; i < kW * kW; i += kThreads) {
-      const int c = i / kW, b = i % kW;
-      X[c * kN + col * kW + b] = st[i];
-    }
-  };
-  // weights of slice k for the columns in `mask` from X (and lead weights at a boundary slice);
-  // fused, also the level-2 blocks of the rows (k, a) towards the site columns in `tmask`
-  // (their slice ys[col], weights eta_{y,b} |G_{k,y}[a][b]|^2): one block per thread, the
-  // columns' rows on threads 0..127 and the transposed rows on 128..255
-  auto emit = [&](const cf* X, int k, unsigned mask, unsigned tmask) {
-    for (int i = tid; i < kN * kW; i += kThreads) {
-      const int r = i % kN, a = i / kN;                    // r consecutive across threads
-      Wt[r * kWtPitch + a] = wsq(eta[k * kW + a], X[a * kN + r]);
-    }
-    if (tmask) {
-      for (int i = tid; i < kN * kW; i += kThreads) {
-        const int r = i / kW, b = i % kW, col = r / kW;
-        if (tmask & (1u << col))
-          Wt2[r * kWtPitch + b] = wsq(eta[ys[col] * kW + b], X[(r % kW) * kN + col * kW + b]);
+  // Emit slice k from N (and X), by the emitting warps: the weights of the columns in `mask`,
+  // and of the rows (k, a) towards the site columns in `tmask` (their slice ys[col], weights
+  // eta_{y,b} |G_{k,y}[a][b]|^2).  stage: shared memory free during the call (39 KB).
+  auto emit = [&](int k, unsigned mask, unsigned tmask, uint32_t* stage) {
+    uint32_t* stg = stage + ew * 2 * 8 * kSP;
+    int pass = 0;
+    auto turn = [&]() {
+      // two staging areas in turn: the copies of the one before last have been read
+      uint32_t* s = stg + (pass & 1) * 8 * kSP;
+      if (pass >= 2) {
+        if (lane < 8) bulk_wait_read<1>();
+        __syncwarp();
       }
-    }
-    __syncthreads();
-    if (!fused) {
-      for (int i = tid; i < kN * kW; i += kThreads) {
-        const int a = i % kW, r = i / kW;                  // a consecutive: coalesced rows
-        const int col = r / kW;
-        if (mask & (1u << col))
-          wt[row_of(ys[col], r % kW) * K + (uint64_t)k * kW + a] = Wt[r * kWtPitch + a];
-      }
-    } else {
-      // every thread takes part (the stores go through barriers): pairs 0..127 a row of the
-      // columns, 128..255 a transposed row
-      const int bi = tid >> 1;
-      bool have;
-      uint64_t row;
-      int slice;
-      const float* wrow;
-      if (bi < kN) {
-        have = mask & (1u << (bi / kW));
-        row = have ? row_of(ys[bi / kW], bi % kW) : 0;
-        slice = k;
-        wrow = Wt + bi * kWtPitch;
+      ++pass;
+      return s;
+    };
+#pragma unroll
+    for (int col = 0; col < 2; ++col) {
+      if (!(mask & (1u << col))) continue;
+      if (fused) {
+        put_blocks(turn(), eta + k * kW, row_of(ys[col], 0), k,
+                   [&](int r, int a) { return N[n_at(a, col * kW + r)]; });
       } else {
-        const int r = bi - kN, col = r / kW;
-        have = tmask & (1u << col);
-        row = (uint64_t)k * kW + r % kW;
-        slice = have ? ys[col] : 0;
-        wrow = Wt2 + r * kWtPitch;
-      }
-      put_blocks(have, row, slice, wrow);
-    }
-    if (k == 0 || k == L - 1) {
-      // lead weights: Phi (FP32) staged in Gs (free outside the product)
-      float* phis = reinterpret_cast<float*>(Gs);
-      float* gams = phis + kW * kW;
-      __syncthreads();
-      for (int i = tid; i < kW * kW; i += kThreads) phis[i] = phi32[d.phi_off + i];
-      for (int i = tid; i < kW; i += kThreads) gams[i] = (float)gam[d.lead_off + i];
-      __syncthreads();
-      const int r = tid % kN, h = tid / kN;                // four quarters of the modes
-      float part = 0.f;
-      for (int nu = h * 16; nu < h * 16 + 16; ++nu) {
-        float zr = 0.f, zi = 0.f;
-        for (int a = 0; a < kW; ++a) {
-          const float p = phis[a * kW + nu];
-          const cf v = X[a * kN + r];
-          zr += p * v.x;
-          zi += p * v.y;
-        }
-        part += gams[nu] * (zr * zr + zi * zi);
-      }
-      Wt[r * kWtPitch + h] = part;                         // staging is free again
-      __syncthreads();
-      if (h == 0) {
-        const int col = r / kW;
-        if (mask & (1u << col)) {
-          const float lw = (Wt[r * kWtPitch] + Wt[r * kWtPitch + 1]) +
-                           (Wt[r * kWtPitch + 2] + Wt[r * kWtPitch + 3]);
-          const uint64_t row = row_of(ys[col], r % kW);
-          if (fused) {
-            if (k == 0) l1[row * (L + 2) + L] = lw;
-            if (k == L - 1) l1[row * (L + 2) + L + 1] = lw;
-          } else {
-            if (k == 0) wt[row * K + n] = lw;
-            if (k == L - 1) wt[row * K + n + 1] = lw;
-          }
+        for (int r = ew; r < kW; r += 8) {
+          float* dst = wt + row_of(ys[col], r) * K + (uint64_t)k * kW;
+#pragma unroll
+          for (int a = lane; a < kW; a += 32)
+            dst[a] = __fmul_rn(__ldg(eta + k * kW + a), N[n_at(a, col * kW + r)]);
         }
       }
     }
-    __syncthreads();
-  };
-
-  unsigned have = 0;
-  for (int col = 0; col < 2; ++col)
-    if (ys[col] >= 0) have |= 1u << col;
-  // direction 0 emits every column's start slice
-  if (dir == 0) {
+#pragma unroll
     for (int col = 0; col < 2; ++col) {
-      if (!(have & (1u << col))) continue;
-      load_start(Xa, col);
-      __syncthreads();
-      emit(Xa, m0_of(ys[col]), 1u << col, 0u);
-    }
-  }
-  const int m0a = m0_of(job.y0), m0b = job.y1 >= 0 ? m0_of(job.y1) : m0a;
-  const int k_first = dir == 0 ? max(m0a, m0b) - 1 : min(m0a, m0b) + 1;
-  const int k_end = dir == 0 ? -1 : L;
-  const int kstep = dir == 0 ? -1 : 1;
-  cf* Xc = Xa;
-  cf* Xn = Xb;
-  const int ty = tid / 32, tx = tid % 32;                  // outputs a = ty + 16i, b' = tx + 32j
-  // this thread's share of the next step's g block, fetched while the current step multiplies
-  constexpr int kGPer = kW * kW / kThreads;
-  cf gnext[kGPer];
-  auto fetch = [&](int k) {
-    const cf* gk = gsrc + (uint64_t)k * kW * kW;
+      if (!(tmask & (1u << col))) continue;
+      const float* em = eta + ys[col] * kW;
+      if (fused) {
+        put_blocks(turn(), em, (uint64_t)k * kW, ys[col],
+                   [&](int a, int b) { return N[n_at(a, col * kW + b)]; });
+      } else {
+        for (int a = ew; a < kW; a += 8) {
+          float* dst = wt + (uint64_t)(k * kW + a) * K + (uint64_t)ys[col] * kW;
 #pragma unroll
-    for (int q = 0; q < kGPer; ++q) gnext[q] = gk[tid + q * kThreads];
-  };
-  if (k_first != k_end) fetch(k_first);
-  for (int k = k_first; k != k_end; k += kstep) {
-    unsigned active = 0;
-    for (int col = 0; col < 2; ++col) {
-      if (!(have & (1u << col))) continue;
-      const int m0 = m0_of(ys[col]);
-      if (dir == 0 ? k < m0 : k > m0) active |= 1u << col;
-      if (dir == 0 ? k == m0 - 1 : k == m0 + 1) load_start(Xc, col);
-    }
-#pragma unroll
-    for (int q = 0; q < kGPer; ++q) Gs[tid + q * kThreads] = cf{mt * gnext[q].x, mt * gnext[q].y};
-    __syncthreads();
-    if (k + kstep != k_end) fetch(k + kstep);
-    float accr[4][4], acci[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) accr[i][j] = acci[i][j] = 0.f;
-#pragma unroll 4
-    for (int c = 0; c < kW; ++c) {
-      cf g[4], x[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) g[i] = Gs[(ty + 16 * i) * kW + c];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) x[j] = Xc[c * kN + tx + 32 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          accr[i][j] = fmaf(g[i].x, x[j].x, accr[i][j]);
-          accr[i][j] = fmaf(-g[i].y, x[j].y, accr[i][j]);
-          acci[i][j] = fmaf(g[i].x, x[j].y, acci[i][j]);
-          acci[i][j] = fmaf(g[i].y, x[j].x, acci[i][j]);
+          for (int b = lane; b < kW; b += 32)
+            dst[b] = __fmul_rn(__ldg(em + b), N[n_at(a, col * kW + b)]);
         }
+      }
     }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) Xn[(ty + 16 * i) * kN + tx + 32 * j] = cf{accr[i][j], acci[i][j]};
-    __syncthreads();
-    unsigned tmask = 0;                                    // fused: transposed rows' blocks
-    if (dir == 0 && fused)
-      for (int col = 0; col < 2; ++col)
-        if ((active & (1u << col)) && ys[col] < L) tmask |= 1u << col;
-    if (active) emit(Xn, k, active, tmask);
     if (dir == 0) {
+#pragma unroll
       for (int col = 0; col < 2; ++col) {
-        if (!(active & (1u << col))) continue;
-        const int y = ys[col];
-        if (y < L && !fused) {
-          // rows (k, a) towards the column's start slice m = y: eta_{m,b} |G_{k,m}[a][b]|^2
-          const float* em = eta + y * kW;
-          float* dst = wt + (uint64_t)k * kW * K + (uint64_t)y * kW;
-          for (int i = tid; i < kW * kW; i += kThreads) {
-            const int a = i / kW, b = i % kW;               // b consecutive: coalesced rows
-            dst[(uint64_t)a * K + b] = wsq(em[b], Xn[a * kN + col * kW + b]);
-          }
-        } else if (y == L + 1) {
-          // lead-R weights of the rows of slice k from (G Phi_R)_k: eight threads per row
-          const int a = tid >> 3, q = tid & 7;
+        // lead-R weights of the rows of slice k from (G Phi_R)_k: eight threads per row
+        if (!(mask & (1u << col)) || ys[col] != L + 1 || k == L - 1) continue;
+        const int te = tid - kMul, q = te & 7;
+        for (int a = te >> 3; a < kW; a += (kThreads - kMul) / 8) {
           float part = 0.f;
-#pragma unroll 4
+#pragma unroll
           for (int nu = q * 8; nu < q * 8 + 8; ++nu) {
-            const cf v = Xn[a * kN + col * kW + nu];
-            part += (float)gam[d.lead_off + nu] * (v.x * v.x + v.y * v.y);
+            const cf v = X[a * kN + col * kW + nu];
+            part = __fmaf_rn((float)gam[d.lead_off + nu],
+                             __fmaf_rn(v.x, v.x, __fmul_rn(v.y, v.y)), part);
           }
           part += __shfl_xor_sync(0xffffffffu, part, 1);
           part += __shfl_xor_sync(0xffffffffu, part, 2);
@@ -325,10 +245,176 @@ __global__ void __launch_bounds__(kThreads, 1) chain_cta_kernel(
         }
       }
     }
-    cf* tmp = Xc;
-    Xc = Xn;
-    Xn = tmp;
+    if (lane < 8) bulk_wait_read<0>();
+    __syncwarp();
+  };
+  // Lead weights of the columns in `mask` from X at a boundary slice k, by the whole CTA; Phi
+  // (FP32) and the partial sums take the first g block, which no product needs any more (or
+  // yet).  Synchronised before and after.
+  auto lead_weights = [&](int k, unsigned mask) {
+    float* phis = reinterpret_cast<float*>(G0);
+    float* gams = phis + kW * kW;
+    float* parts = gams + kW;
+    for (int i = tid; i < kW * kW; i += kThreads) phis[i] = phi32[d.phi_off + i];
+    for (int i = tid; i < kW; i += kThreads) gams[i] = (float)gam[d.lead_off + i];
+    __syncthreads();
+    const int r = tid % kN, h = tid / kN;                  // four quarters of the modes
+    float part = 0.f;
+    for (int nu = h * 16; nu < h * 16 + 16; ++nu) {
+      float zr = 0.f, zi = 0.f;
+      for (int a = 0; a < kW; ++a) {
+        const float p = phis[a * kW + nu];
+        const cf v = X[a * kN + r];
+        zr = __fmaf_rn(p, v.x, zr);
+        zi = __fmaf_rn(p, v.y, zi);
+      }
+      part = __fmaf_rn(gams[nu], __fmaf_rn(zr, zr, __fmul_rn(zi, zi)), part);
+    }
+    parts[h * kN + r] = part;
+    __syncthreads();
+    if (h == 0) {
+      const int col = r / kW;
+      if (mask & (1u << col)) {
+        const float lw = (parts[r] + parts[kN + r]) + (parts[2 * kN + r] + parts[3 * kN + r]);
+        const uint64_t row = row_of(ys[col], r % kW);
+        if (fused) {
+          if (k == 0) l1[row * (L + 2) + L] = lw;
+          if (k == L - 1) l1[row * (L + 2) + L + 1] = lw;
+        } else {
+          if (k == 0) wt[row * K + n] = lw;
+          if (k == L - 1) wt[row * K + n + 1] = lw;
+        }
+      }
+    }
+    __syncthreads();
+  };
+  // start block of column slot col into X[:, col*64 .. col*64+63]
+  auto load_start = [&](int col) {
+    const cf* st = start + d.start_off + (uint64_t)ys[col] * kW * kW;
+    for (int i = tid; i < kW * kW; i += kThreads)
+      X[(i / kW) * kN + col * kW + i % kW] = st[i];
+  };
+
+  unsigned have = 0;
+  for (int col = 0; col < 2; ++col)
+    if (ys[col] >= 0) have |= 1u << col;
+  // direction 0 emits every column's start slice
+  if (dir == 0) {
+    for (int col = 0; col < 2; ++col) {
+      if (!(have & (1u << col))) continue;
+      const int m0 = m0_of(ys[col]);
+      load_start(col);
+      __syncthreads();
+      for (int i = tid; i < kW * kW; i += kThreads) {
+        const int a = i / kW, b = col * kW + i % kW;
+        N[n_at(a, b)] = nsq(X[a * kN + b]);
+      }
+      __syncthreads();
+      if (m0 == 0 || m0 == L - 1) lead_weights(m0, 1u << col);
+      if (!mul) emit(m0, 1u << col, 0u, reinterpret_cast<uint32_t*>(G0));
+      __syncthreads();
+    }
   }
+  const int m0a = m0_of(job.y0), m0b = job.y1 >= 0 ? m0_of(job.y1) : m0a;
+  const int k_first = dir == 0 ? max(m0a, m0b) - 1 : min(m0a, m0b) + 1;
+  const int k_end = dir == 0 ? -1 : L;
+  const int kstep = dir == 0 ? -1 : 1;
+  // -t g_k, doubled, into G (threads t0, t0 + nt, ...)
+  auto put_g = [&](int k, float4* G, int t0, auto nt) {
+    constexpr int kPer = kW * kW / decltype(nt)::value;
+    const cf* gk = gsrc + (uint64_t)k * kW * kW;
+    cf v[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) v[q] = gk[t0 + q * decltype(nt)::value];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int i = t0 + q * decltype(nt)::value;
+      const float gx = mt * v[q].x, gy = mt * v[q].y;
+      G[g_at(i / kW, i % kW)] = make_float4(gx, gx, gy, gy);
+    }
+  };
+  if (k_first != k_end) put_g(k_first, G0, tid, std::integral_constant<int, kThreads>());
+  // multiplying lane: rows a = 32 wa + ty + 4 i, columns b' = 32 wb + 2 tx + 16 h (+ 1)
+  const int ty = lane >> 3, tx = lane & 7, mw = tid >> 5;
+  const int wa = mw & 1, wb = (mw >> 1) & 3;
+  int k_prev = -1, buf = 0;
+  unsigned act_prev = 0, t_prev = 0;
+  for (int k = k_first; k != k_end; k += kstep) {
+    unsigned active = 0;
+    for (int col = 0; col < 2; ++col) {
+      if (!(have & (1u << col))) continue;
+      const int m0 = m0_of(ys[col]);
+      if (dir == 0 ? k < m0 : k > m0) active |= 1u << col;
+      if (dir == 0 ? k == m0 - 1 : k == m0 + 1) load_start(col);
+    }
+    if (active != act_prev) __syncthreads();               // a column has joined
+    if (mul) {
+      const float4* G = G0 + buf * kW * kW + 32 * wa;
+      const cf* Xl = X + 32 * wb + 2 * tx;
+      f2 acc[8][4];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+#pragma unroll 1
+      for (int c0 = 0; c0 < kW; c0 += 8) {
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+          const int c = c0 + s;
+          const ulonglong2 xa = lds2(Xl + c * kN), xb = lds2(Xl + c * kN + 16);
+          const f2 x[4] = {xa.x, xa.y, xb.x, xb.y};
+          f2 xs[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float2 v = unpack2(x[j]);
+            xs[j] = pack2(-v.y, v.x);
+          }
+          const float4* Gc = G + c * kW + (ty ^ (s & 3));
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const ulonglong2 g = lds2(Gc + ((4 * i) ^ (s & 4)));
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = fma2(g.x, x[j], acc[i][j]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = fma2(g.y, xs[j], acc[i][j]);
+          }
+        }
+      }
+      step_sync();                                         // X and N have been read
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int a = 32 * wa + ty + 4 * i;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int b = 32 * wb + 2 * tx + 16 * h;
+          *reinterpret_cast<ulonglong2*>(X + a * kN + b) =
+              make_ulonglong2(acc[i][2 * h], acc[i][2 * h + 1]);
+          const float2 u = unpack2(acc[i][2 * h]), v = unpack2(acc[i][2 * h + 1]);
+          N[n_at(a, b)] = nsq(cf{u.x, u.y});
+          N[n_at(a, b + 1)] = nsq(cf{v.x, v.y});
+        }
+      }
+    } else {
+      float4* Gn = G0 + (buf ^ 1) * kW * kW;
+      if (k_prev >= 0) {
+        emit(k_prev, act_prev, t_prev, reinterpret_cast<uint32_t*>(Gn));
+        emit_sync();                                       // the staging has been read
+      }
+      if (k + kstep != k_end)
+        put_g(k + kstep, Gn, tid - kMul, std::integral_constant<int, kThreads - kMul>());
+      step_sync();
+    }
+    __syncthreads();
+    if (k == 0 || k == L - 1) lead_weights(k, active);     // the last step of its direction
+    k_prev = k;
+    act_prev = active;
+    t_prev = 0;
+    if (dir == 0)
+      for (int col = 0; col < 2; ++col)
+        if ((active & (1u << col)) && ys[col] < L) t_prev |= 1u << col;
+    buf ^= 1;
+  }
+  if (!mul && k_prev >= 0) emit(k_prev, act_prev, t_prev, reinterpret_cast<uint32_t*>(G0));
   if (__syncthreads_or(bad) && tid == 0) atomicOr(err, ERR_NONFINITE);
 }
 
