@@ -374,33 +374,52 @@ __global__ void grad_diag_kernel(TaskDesc d, const C* __restrict__ G, const C* _
 }
 
 // ---- dI/dtheta per wire: sum over the wire's tasks (fixed order) of
-// seed_w * w_E (f_p - f_q) dT/dtheta.  One thread per (wire, site).
+// seed_w * w_E (f_p - f_q) dT/dtheta.  One CTA per (wire, 256 sites), one thread per site; the
+// tasks' factors, two FP64 hyperbolic tangents each, are formed once per CTA, a task per thread
+// (formed by every site's thread on one CTA per wire they took 0.58 ms on the W=16 x L=100,
+// 16-energy gradient; @@ ms now).
 __device__ __forceinline__ double fermi_b(double E, double mu, double kT) {
   return 0.5 * (1.0 - tanh(0.5 * (E - mu) / kT));
 }
 
-__global__ void grad_sum_kernel(const TaskDesc* __restrict__ tasks, int n_wires,
-                                const int32_t* __restrict__ wire_task0,
-                                const uint64_t* __restrict__ task_site_off,
-                                const uint64_t* __restrict__ wire_site_off,
-                                const double* __restrict__ dT_V, const double* __restrict__ dT_E,
-                                const double* __restrict__ seed, double mu_p, double mu_q,
-                                double kT, double* __restrict__ out_V, double* __restrict__ out_E) {
-  const int w = blockIdx.x;
-  if (w >= n_wires) return;
-  const int t0 = wire_task0[w], t1 = wire_task0[w + 1];
-  if (t0 == t1) return;
-  const int n = tasks[t0].n;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    double aV = 0.0, aE = 0.0;
-    for (int t = t0; t < t1; ++t) {
-      const TaskDesc& d = tasks[t];
-      const double wd = seed[w] * d.w_E * (fermi_b(d.E, mu_p, kT) - fermi_b(d.E, mu_q, kT));
-      aV += wd * dT_V[task_site_off[t] + k];
-      aE += wd * dT_E[task_site_off[t] + k];
+constexpr int kGradSumThreads = 256;
+
+__global__ void __launch_bounds__(kGradSumThreads) grad_sum_kernel(
+    const TaskDesc* __restrict__ tasks, int n_wires, const int32_t* __restrict__ wire_task0,
+    const uint64_t* __restrict__ task_site_off, const uint64_t* __restrict__ wire_site_off,
+    const double* __restrict__ dT_V, const double* __restrict__ dT_E,
+    const double* __restrict__ seed, double mu_p, double mu_q, double kT,
+    double* __restrict__ out_V, double* __restrict__ out_E) {
+  __shared__ double s_wd[kGradSumThreads];
+  __shared__ uint64_t s_off[kGradSumThreads];
+  for (int w = blockIdx.y; w < n_wires; w += gridDim.y) {
+    const int t0 = wire_task0[w], t1 = wire_task0[w + 1];
+    if (t0 == t1) continue;
+    const int n = tasks[t0].n;
+    for (int k0 = blockIdx.x * blockDim.x; k0 < n; k0 += gridDim.x * blockDim.x) {
+      const int k = k0 + threadIdx.x;
+      double aV = 0.0, aE = 0.0;
+      for (int tb = t0; tb < t1; tb += kGradSumThreads) {
+        const int nb = min(kGradSumThreads, t1 - tb);
+        __syncthreads();
+        if ((int)threadIdx.x < nb) {
+          const TaskDesc& d = tasks[tb + threadIdx.x];
+          s_wd[threadIdx.x] =
+              seed[w] * d.w_E * (fermi_b(d.E, mu_p, kT) - fermi_b(d.E, mu_q, kT));
+          s_off[threadIdx.x] = task_site_off[tb + threadIdx.x];
+        }
+        __syncthreads();
+        if (k < n)
+          for (int t = 0; t < nb; ++t) {
+            aV += s_wd[t] * dT_V[s_off[t] + k];
+            aE += s_wd[t] * dT_E[s_off[t] + k];
+          }
+      }
+      if (k < n) {
+        out_V[wire_site_off[w] + k] = aV;
+        out_E[wire_site_off[w] + k] = aE;
+      }
     }
-    out_V[wire_site_off[w] + k] = aV;
-    out_E[wire_site_off[w] + k] = aE;
   }
 }
 
@@ -485,7 +504,9 @@ cudaError_t launch_grad_sum(const TaskDesc* d_tasks, int n_wires, const int32_t*
                             double mu_p, double mu_q, double kT, double* out_V, double* out_E,
                             cudaStream_t s) {
   if (n_wires == 0) return cudaSuccess;
-  grad_sum_kernel<<<n_wires, 256, 0, s>>>(d_tasks, n_wires, d_wire_task0, d_task_site_off,
+  // wires on the grid's y (at most 65535 at a time), chunks of 256 sites on x
+  const dim3 grid(16, n_wires < 65535 ? n_wires : 65535);
+  grad_sum_kernel<<<grid, kGradSumThreads, 0, s>>>(d_tasks, n_wires, d_wire_task0, d_task_site_off,
                                           d_wire_site_off, dT_V, dT_E, d_seed, mu_p, mu_q, kT,
                                           out_V, out_E);
   return cudaGetLastError();
