@@ -9,14 +9,17 @@
 // transition from the current row: slot c = (x*K)>>32, keep c if y < thr[c] else alias[c].
 // Columns n and n+1 are the leads: drawing one ends the walk, and the sample's estimator is
 // X_pq = Tr[Gamma_p A] delta_rq (Eq. elast_lin_xpq), tallied as counts per absorbing lead.
-// A lane carries one or two walkers at a time (kSlots; with two, the dependent gathers of the
-// two walks are in flight together, which pays when the gathers miss L2).  When a walk ends
+// A lane carries one or two walkers at a time (kSlots).  An iteration takes every slot through
+// the same stages - Philox block, first gather, second gather, (two-level tables) third - with
+// each stage's loads of all slots issued before the first of them is used, so that the dependent
+// gathers of a lane's walks are in flight together.  When a walk ends
 // the lane starts the next walker of its own run of consecutive walker indices (32 per lane)
 // with no warp coordination; once enough lanes of a warp have an idle slot and an empty run,
 // one lane claims a new range for all of them from a global counter.  Every loop iteration
 // consumes one whole Philox block per walker (two draws: the injection and the first
 // transition for a new walker, two transitions afterwards), so the generator runs
-// warp-uniformly.  Each lane counts its outcomes for its current task (shared by its slots) in
+// warp-uniformly; the injection takes the same instructions as a transition, from another row.
+// Each lane counts its outcomes for its current task (shared by its slots) in
 // registers and adds them to the block's shared tally when it moves to another task; the block
 // adds its tally to global memory once.
 #include <cuda_runtime.h>
@@ -102,8 +105,17 @@ __device__ __forceinline__ uint32_t two_level_draw(const uint64_t* __restrict__ 
 }
 
 // kTwo: the launch may hold two-level tasks (one-level launches compile without that path).
+// CTAs per SM (registers): the two-level stages hold a guide or octet of each slot, and spilling
+// them costs more than the lost occupancy (32 energies x 1e6 walkers, two slots: W=24 x L=150
+// 4.14 ms at four CTAs, 3.30 at three; slot after slot, as before, 4.09; W=12 x L=190 5.05, 4.07
+// and 4.66).  One-level walks of tables in L2 (W=10 x L=50, 64 energies) want occupancy: 1.00 ms
+// with one slot at five CTAs, 1.05 with two at four (1.07 before).
+constexpr int walk_ctas(bool score, bool two, int slots) {
+  return score ? 3 : (two ? 5 : 6) - slots;
+}
+
 template <bool kTrace, bool kScore, int kSlotsReq, bool kTwo>
-__global__ void __launch_bounds__(kThreads, kScore ? 3 : (kSlotsReq == 2 ? 4 : 5)) walk_kernel(
+__global__ void __launch_bounds__(kThreads, walk_ctas(kScore, kTwo, kSlotsReq)) walk_kernel(
     const TaskDesc* __restrict__ tasks, int task0, int n_tasks, uint32_t id_base,
     const uint64_t* __restrict__ tab, const uint64_t* __restrict__ mode_tab,
     const double* __restrict__ cvals, int start_lead, PhiloxKey key, uint64_t walkers_per_task,
@@ -127,13 +139,12 @@ __global__ void __launch_bounds__(kThreads, kScore ? 3 : (kSlotsReq == 2 ? 4 : 5
   const unsigned lt_mask = (1u << lane) - 1u;
   const unsigned long long total = (unsigned long long)n_tasks * walkers_per_task;
 
-  // kSlots walkers per lane (registers), so that their dependent gathers overlap; b = next
-  // Philox block (draws 2b, 2b + 1)
+  // kSlots walkers per lane (registers); b = next Philox block (draws 2b, 2b + 1)
   constexpr int kSlots = kSlotsReq;
   bool has[kSlots];
-  unsigned long long g[kSlots];
+  unsigned long long g[kTrace ? kSlots : 1];
   uint32_t row[kSlots], b[kSlots], steps[kSlots], wid_lo[kSlots], wid_hi[kSlots];
-  uint32_t inj[kSlots];                                  // kScore: the injection mode
+  uint32_t inj[kScore ? kSlots : 1];                     // the injection mode
   // kScore: the column drawn at transition st (1-based) of the lane's walker in slot sl
   uint32_t ext[kScore ? kSlots * kPathExt : 1];
   auto record = [&](int sl, uint32_t st, uint32_t j) {
@@ -145,11 +156,12 @@ __global__ void __launch_bounds__(kThreads, kScore ? 3 : (kSlotsReq == 2 ? 4 : 5
 #pragma unroll
   for (int sl = 0; sl < kSlots; ++sl) {
     has[sl] = false;
-    g[sl] = 0;
-    row[sl] = b[sl] = steps[sl] = wid_lo[sl] = wid_hi[sl] = inj[sl] = 0;
+    row[sl] = b[sl] = steps[sl] = wid_lo[sl] = wid_hi[sl] = 0;
   }
-  // this lane's run of walker indices [r_next, r_end)
-  unsigned long long r_next = 0, r_end = 0;
+  // this lane's run: the next walker's index, how many are left, how many of those belong to
+  // the cached task
+  unsigned long long r_next = 0;
+  uint32_t r_left = 0, t_left = 0;
   // cached task (shared by the slots): index window [t_first, t_first + walkers_per_task)
   int tl = -1;
   unsigned long long t_first = 0;
@@ -169,34 +181,39 @@ __global__ void __launch_bounds__(kThreads, kScore ? 3 : (kSlotsReq == 2 ? 4 : 5
     // slot takes a walker of another task only when the other slots are idle
 #pragma unroll
     for (int sl = 0; sl < kSlots; ++sl) {
-      while (!has[sl] && r_next < r_end) {
-        const unsigned long long gn = r_next;
-        if (tl < 0 || gn - t_first >= walkers_per_task) {
+      while (!has[sl] && r_left) {
+        if (t_left == 0) {
           bool others = false;
 #pragma unroll
           for (int o = 0; o < kSlots; ++o)
             if (o != sl) others |= has[o];
-          if (others) break;
-          if (tl >= 0) flush_lane(s_tally, tl, a);
-          tl = (int)(gn / walkers_per_task);
-          t_first = (unsigned long long)tl * walkers_per_task;
-          const TaskDesc& d = tasks[task0 + tl];
-          task_id = id_base + (uint32_t)(task0 + tl);
-          K = (uint32_t)d.K;
-          n = (uint32_t)d.n;
-          W = (uint32_t)d.W;
-          inj_row0 = (uint32_t)(d.n + start_lead * d.W);
-          t_wt_off = d.wt_off;
-          t_mode_off = d.mode_off + start_lead * d.W;
-          trow = tab + d.tab_off;
-          two = kTwo && d.layout == NEGF_LAYOUT_TWO_LEVEL;
-          L = (uint32_t)d.L;
-          B2 = (uint32_t)level2_words(d.W);
-          l1row = tab + d.l1_off;
-          mrow = mode_tab + d.mode_off + start_lead * d.W;
-          t_open = cvals[2 * (task0 + tl) + start_lead] > 0.0;
+          if (tl < 0 || r_next - t_first >= walkers_per_task) {
+            if (others) break;
+            if (tl >= 0) flush_lane(s_tally, tl, a);
+            tl = (int)(r_next / walkers_per_task);
+            t_first = (unsigned long long)tl * walkers_per_task;
+            const TaskDesc& d = tasks[task0 + tl];
+            task_id = id_base + (uint32_t)(task0 + tl);
+            K = (uint32_t)d.K;
+            n = (uint32_t)d.n;
+            W = (uint32_t)d.W;
+            inj_row0 = (uint32_t)(d.n + start_lead * d.W);
+            t_wt_off = d.wt_off;
+            t_mode_off = d.mode_off + start_lead * d.W;
+            trow = tab + d.tab_off;
+            two = kTwo && d.layout == NEGF_LAYOUT_TWO_LEVEL;
+            L = (uint32_t)d.L;
+            B2 = (uint32_t)level2_words(d.W);
+            l1row = tab + d.l1_off;
+            mrow = mode_tab + d.mode_off + start_lead * d.W;
+            t_open = cvals[2 * (task0 + tl) + start_lead] > 0.0;
+          }
+          const unsigned long long in_task = walkers_per_task - (r_next - t_first);
+          t_left = in_task < r_left ? (uint32_t)in_task : r_left;
         }
-        ++r_next;
+        const unsigned long long gn = r_next++;
+        --r_left;
+        --t_left;
         if (!t_open) {
           // no open channel in the start lead: nothing to inject (T = 0 exactly)
           a[0] += 1u;
@@ -204,7 +221,7 @@ __global__ void __launch_bounds__(kThreads, kScore ? 3 : (kSlotsReq == 2 ? 4 : 5
           continue;
         }
         const uint64_t w = id_offset + (gn - t_first);
-        g[sl] = gn;
+        if (kTrace) g[sl] = gn;
         wid_lo[sl] = (uint32_t)w;
         wid_hi[sl] = (uint32_t)(w >> 32);
         b[sl] = 0;
@@ -220,7 +237,7 @@ __global__ void __launch_bounds__(kThreads, kScore ? 3 : (kSlotsReq == 2 ? 4 : 5
     }
     // ---- claim new runs once enough lanes have an idle slot and an empty run (or none has
     // work left)
-    const unsigned dry = __ballot_sync(FULL, idle && r_next >= r_end);
+    const unsigned dry = __ballot_sync(FULL, idle && r_left == 0);
     if (dry && !no_more && (__popc(dry) >= kClaimMin || dry == FULL)) {
       unsigned long long base = 0;
       if (lane == 0) base = atomicAdd(counter, (unsigned long long)__popc(dry) * kRun);
@@ -230,7 +247,8 @@ __global__ void __launch_bounds__(kThreads, kScore ? 3 : (kSlotsReq == 2 ? 4 : 5
       } else if (dry & (1u << lane)) {
         const unsigned long long lo = base + (unsigned long long)__popc(dry & lt_mask) * kRun;
         r_next = lo < total ? lo : total;
-        r_end = lo + kRun < total ? lo + kRun : total;
+        r_left = total - r_next < kRun ? (uint32_t)(total - r_next) : kRun;
+        t_left = 0;
       }
       continue;      // start the new walkers first
     }
@@ -239,64 +257,112 @@ __global__ void __launch_bounds__(kThreads, kScore ? 3 : (kSlotsReq == 2 ? 4 : 5
     if (kSlots == 1 ? dry == FULL : !__any_sync(FULL, busy)) break;
     if (!busy) continue;
 
-    // ---- per walking slot one Philox block = two draws.  Block 0: the injection draw (Step 4)
-    // then the first transition; later blocks: two Step 6' transitions.
+    // ---- one Philox block per walking slot: block 0 is the injection draw (Step 4) and, with
+    // one-level tables, the first transition; later blocks are one (two-level) or two Step 6'
+    // transitions.  outcome -3: continue, 0/1: absorbed at L/R, -2: truncated
+    int outcome[kSlots];
+    uint4 r[kSlots];
+#pragma unroll
+    for (int sl = 0; sl < kSlots; ++sl) {
+      outcome[sl] = -3;
+      r[sl] = philox4x32_10(make_uint4(b[sl], wid_lo[sl], wid_hi[sl], task_id), key);
+    }
+    // the first gather: the mode row, or the walk's (level-1) row
+    const bool lane_two = kTwo && two;
+    const uint32_t K1 = lane_two ? L + 2 : K;
+    const uint64_t* rows1 = lane_two ? l1row : trow;
+    uint32_t c1[kSlots];
+    uint64_t e1[kSlots];
+#pragma unroll
+    for (int sl = 0; sl < kSlots; ++sl) {
+      const bool first = b[sl] == 0;
+      c1[sl] = __umulhi(r[sl].x, first ? W : K1);
+      const uint64_t* src = first ? mrow : rows1 + (uint64_t)row[sl] * K1;
+      e1[sl] = has[sl] ? __ldg(src + c1[sl]) : 0ull;
+    }
+    // a transition to j: ends the walk at a lead or at the cap
+    auto moved = [&](int sl, uint32_t j) {
+      ++steps[sl];
+      record(sl, steps[sl], j);
+      if (j >= n) outcome[sl] = (int)(j - n);
+      else if (steps[sl] >= max_steps) outcome[sl] = -2;
+      else row[sl] = j;
+    };
+    if (!lane_two) {
+      uint64_t e2[kSlots];
+      uint32_t c2[kSlots];
+#pragma unroll
+      for (int sl = 0; sl < kSlots; ++sl) {
+        const uint32_t j = r[sl].y < (uint32_t)e1[sl] ? c1[sl] : (uint32_t)(e1[sl] >> 32);
+        if (b[sl] == 0) {
+          if (kScore) inj[sl] = j;
+          row[sl] = inj_row0 + j;
+        } else {
+          moved(sl, j);
+        }
+        c2[sl] = __umulhi(r[sl].z, K);
+        e2[sl] = has[sl] && outcome[sl] == -3 ? __ldg(trow + (uint64_t)row[sl] * K + c2[sl]) : 0ull;
+      }
+#pragma unroll
+      for (int sl = 0; sl < kSlots; ++sl)
+        if (outcome[sl] == -3)
+          moved(sl, r[sl].w < (uint32_t)e2[sl] ? c2[sl] : (uint32_t)(e2[sl] >> 32));
+    } else {
+      // (x, y) drew the slice or lead, z draws the site: v = z >> 1 against the guide, then
+      // against the octet it points to
+      const uint4* blk[kSlots];
+      uint32_t k[kSlots], q[kSlots];
+      uint4 q0[kSlots], q1[kSlots];
+      bool site[kSlots];
+#pragma unroll
+      for (int sl = 0; sl < kSlots; ++sl) {
+        k[sl] = r[sl].y < (uint32_t)e1[sl] ? c1[sl] : (uint32_t)(e1[sl] >> 32);
+        site[sl] = has[sl] && b[sl] != 0 && k[sl] < L;
+        blk[sl] = reinterpret_cast<const uint4*>(trow) +
+                  (((uint64_t)row[sl] * L + (site[sl] ? k[sl] : 0u)) * B2 >> 2);
+        q0[sl] = q1[sl] = make_uint4(0u, 0u, 0u, 0u);
+        if (site[sl] && W > 8) {
+          q0[sl] = __ldg(blk[sl]);
+          q1[sl] = __ldg(blk[sl] + 1);
+        }
+      }
+#pragma unroll
+      for (int sl = 0; sl < kSlots; ++sl) {
+        const uint32_t v = r[sl].z >> 1;
+        q[sl] = 0;
+        if (W > 8) {
+          q[sl] = (q0[sl].x <= v) + (q0[sl].y <= v) + (q0[sl].z <= v) + (q0[sl].w <= v) +
+                  (q1[sl].x <= v) + (q1[sl].y <= v) + (q1[sl].z <= v) + (q1[sl].w <= v);
+          blk[sl] += 2 + 2 * q[sl];
+        }
+        if (site[sl]) {
+          q0[sl] = __ldg(blk[sl]);
+          q1[sl] = __ldg(blk[sl] + 1);
+        }
+      }
+#pragma unroll
+      for (int sl = 0; sl < kSlots; ++sl) {
+        const uint32_t v = r[sl].z >> 1;
+        if (b[sl] == 0) {
+          if (kScore) inj[sl] = k[sl];
+          row[sl] = inj_row0 + k[sl];
+        } else {
+          const uint32_t at = 8 * q[sl] + (q0[sl].x <= v) + (q0[sl].y <= v) + (q0[sl].z <= v) +
+                              (q0[sl].w <= v) + (q1[sl].x <= v) + (q1[sl].y <= v) +
+                              (q1[sl].z <= v) + (q1[sl].w <= v);
+          moved(sl, site[sl] ? k[sl] * W + at : n + (k[sl] - L));
+        }
+      }
+    }
 #pragma unroll
     for (int sl = 0; sl < kSlots; ++sl) {
       if (!has[sl]) continue;
-      const uint4 r = philox4x32_10(make_uint4(b[sl], wid_lo[sl], wid_hi[sl], task_id), key);
-      int outcome = -3;                // -3: continue, 0/1: absorbed at L/R, -2: truncated
-      if (kTwo && two) {
-        // two-level tables: block 0 is the injection draw alone; block b >= 1 is transition
-        // b, words (x, y) for the slice or lead (level 1, alias), z for the site in the slice
-        // (level 2: v = z >> 1 against the guide, then against the octet it points to)
-        if (b[sl] == 0) {
-          const uint32_t c = __umulhi(r.x, W);
-          const uint64_t e = __ldg(mrow + c);
-          inj[sl] = r.y < (uint32_t)e ? c : (uint32_t)(e >> 32);
-          row[sl] = inj_row0 + inj[sl];
-        } else {
-          const uint32_t j = two_level_draw(l1row, trow, row[sl], L, W, B2, r);
-          ++steps[sl];
-          record(sl, steps[sl], j);
-          if (j >= n) outcome = (int)(j - n);
-          else if (steps[sl] >= max_steps) outcome = -2;
-          else row[sl] = j;
-        }
-        ++b[sl];
-      } else {
-        if (b[sl] == 0) {
-          const uint32_t c = __umulhi(r.x, W);
-          const uint64_t e = __ldg(mrow + c);
-          inj[sl] = r.y < (uint32_t)e ? c : (uint32_t)(e >> 32);
-          row[sl] = inj_row0 + inj[sl];
-        } else {
-          const uint32_t c = __umulhi(r.x, K);
-          const uint64_t e = __ldg(trow + (uint64_t)row[sl] * K + c);
-          const uint32_t j = r.y < (uint32_t)e ? c : (uint32_t)(e >> 32);
-          ++steps[sl];
-          record(sl, steps[sl], j);
-          if (j >= n) outcome = (int)(j - n);
-          else if (steps[sl] >= max_steps) outcome = -2;
-          else row[sl] = j;
-        }
-        if (outcome == -3) {
-          const uint32_t c = __umulhi(r.z, K);
-          const uint64_t e = __ldg(trow + (uint64_t)row[sl] * K + c);
-          const uint32_t j = r.w < (uint32_t)e ? c : (uint32_t)(e >> 32);
-          ++steps[sl];
-          record(sl, steps[sl], j);
-          if (j >= n) outcome = (int)(j - n);
-          else if (steps[sl] >= max_steps) outcome = -2;
-          else row[sl] = j;
-        }
-        ++b[sl];
-      }
-      if (kScore && outcome >= 0 && steps[sl] <= (uint32_t)(kPath + kPathExt)) {
+      ++b[sl];
+      if (kScore && outcome[sl] >= 0 && steps[sl] <= (uint32_t)(kPath + kPathExt)) {
         // count the recorded transitions of the finished walk under its absorbing lead
-        unsigned long long* cnt = score.cnt + (size_t)outcome * score.stride + t_wt_off;
+        unsigned long long* cnt = score.cnt + (size_t)outcome[sl] * score.stride + t_wt_off;
         atomicAdd(score.mode_cnt +
-                      ((size_t)(blockIdx.x % kModeReplicas) * 2 + outcome) * score.mode_stride +
+                      ((size_t)(blockIdx.x % kModeReplicas) * 2 + outcome[sl]) * score.mode_stride +
                       t_mode_off + inj[sl],
                   1ull);
         uint32_t rrow = inj_row0 + inj[sl];
@@ -307,11 +373,11 @@ __global__ void __launch_bounds__(kThreads, kScore ? 3 : (kSlotsReq == 2 ? 4 : 5
           atomicAdd(cnt + (uint64_t)rrow * K + j, 1ull);
           rrow = j;
         }
-      } else if (kScore && outcome >= 0) {
+      } else if (kScore && outcome[sl] >= 0) {
         // a walk longer than the record: replay it and count its transitions
-        unsigned long long* cnt = score.cnt + (size_t)outcome * score.stride + t_wt_off;
+        unsigned long long* cnt = score.cnt + (size_t)outcome[sl] * score.stride + t_wt_off;
         unsigned long long* mcnt =
-            score.mode_cnt + ((size_t)(blockIdx.x % kModeReplicas) * 2 + outcome) * score.mode_stride +
+            score.mode_cnt + ((size_t)(blockIdx.x % kModeReplicas) * 2 + outcome[sl]) * score.mode_stride +
             t_mode_off;
         uint32_t rrow = 0;
         bool live = true;
@@ -357,13 +423,13 @@ __global__ void __launch_bounds__(kThreads, kScore ? 3 : (kSlotsReq == 2 ? 4 : 5
           }
         }
       }
-      if (outcome != -3) {
+      if (outcome[sl] != -3) {
         a[0] += 1u;
-        if (outcome == 0) a[1] += 1u;
-        else if (outcome == 1) a[2] += 1u;
+        if (outcome[sl] == 0) a[1] += 1u;
+        else if (outcome[sl] == 1) a[2] += 1u;
         else a[3] += 1u;
         a[4] += steps[sl];
-        if (kTrace) { trace_lead[g[sl]] = outcome; trace_steps[g[sl]] = steps[sl]; }
+        if (kTrace) { trace_lead[g[sl]] = outcome[sl]; trace_steps[g[sl]] = steps[sl]; }
         has[sl] = false;
         if (a[4] >= kFlushAt || a[0] >= kFlushAt) flush_lane(s_tally, tl, a);
       }
