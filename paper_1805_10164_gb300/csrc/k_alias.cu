@@ -38,21 +38,57 @@ __device__ __forceinline__ uint64_t pack(uint32_t thr, uint32_t alias) {
   return (uint64_t)thr | ((uint64_t)alias << 32);
 }
 
+// What bounds it: instructions, on few warps per SM (shared memory per warp).  A row passes
+// through its items three times to form the units (largest weight; integer weights and their
+// total; units and their sums), once to list lights and heavies, and once, over the list of
+// lights, to write the slots: a light's own, and those of the heavies whose excess ends within
+// its interval, so that no slot needs a search.  Measured, GB300, against six passes with a
+// search per slot: rows of 502 slots (W=10 x L=50, 64 energies) 0.300 -> 0.218 ms, of 1602
+// (W=16 x L=100, 16 energies, weights kept) 1.38 -> 0.65, of 2002 (W=40 x L=50, 16 tasks)
+// 2.03 -> 1.35, FP64 rows of 502 0.61 -> 0.54.
+//
 // Each lane owns a block of npl = ceil(K/32) consecutive items.  Per-item values live in shared
 // memory at slot (i / npl) * pitch + i % npl, with an odd pitch (npl or npl + 1) so that the 32
 // lanes walking their blocks in step touch 32 different banks.
 __host__ __device__ inline int alias_npl(int K) { return (K + 31) >> 5; }
 __host__ __device__ inline int alias_pitch(int K) { return alias_npl(K) | 1; }
-// Per-warp shared memory: s_u, s_c : u64 [32 pitch] | s_x : u32 [cap] | staging buffer for the
-// next row's weights (cap elements of `elem` bytes, or 64 FP64 mode weights), 16-byte aligned.
-__host__ __device__ inline size_t alias_stage_off(int cap) {
-  const size_t slots = (size_t)32 * alias_pitch(cap);
-  return (2 * slots * sizeof(uint64_t) + (size_t)cap * sizeof(uint32_t) + 15) & ~(size_t)15;
+// Per-warp shared memory: s_u, s_c : u64 [32 pitch] | the row's weights (32 pitch elements of
+// `elem` bytes, or 32 alias_pitch(64) FP64 mode weights) | s_x : u16 [cap]
+__host__ __device__ inline size_t alias_stage_bytes(int cap, int elem) {
+  const size_t row = (size_t)32 * alias_pitch(cap) * elem;
+  const size_t modes = (size_t)32 * alias_pitch(64) * sizeof(double);
+  return ((row > modes ? row : modes) + 15) & ~(size_t)15;
 }
 __host__ __device__ inline size_t alias_warp_bytes(int cap, int elem) {
-  const size_t stage = (size_t)cap * elem > 64 * sizeof(double) ? (size_t)cap * elem
-                                                                  : 64 * sizeof(double);
-  return alias_stage_off(cap) + ((stage + 15) & ~(size_t)15);
+  const size_t slots = (size_t)32 * alias_pitch(cap);
+  return 2 * slots * sizeof(uint64_t) + alias_stage_bytes(cap, elem) +
+         (((size_t)cap * sizeof(uint16_t) + 15) & ~(size_t)15);
+}
+// A warp's arrays in its shared memory
+struct AliasSmem {
+  uint64_t *u, *c;
+  unsigned char* stage;
+  uint16_t* x;
+  __device__ AliasSmem(unsigned char* base, int cap, int elem) {
+    u = reinterpret_cast<uint64_t*>(base);
+    c = u + (size_t)32 * alias_pitch(cap);
+    stage = reinterpret_cast<unsigned char*>(c + (size_t)32 * alias_pitch(cap));
+    x = reinterpret_cast<uint16_t*>(stage + alias_stage_bytes(cap, elem));
+  }
+};
+
+// f(i, slot) for the lane's items i = lane, lane + 32, ... of a K-item row
+template <typename F>
+__device__ __forceinline__ void alias_strided(int K, F f) {
+  const int lane = threadIdx.x & 31, npl = alias_npl(K), pitch = alias_pitch(K);
+  const int q32 = 32 / npl, r32 = 32 - q32 * npl;
+  int q = lane / npl, r = lane - q * npl;
+  for (int i = lane; i < K; i += 32) {
+    f(i, q * pitch + r);
+    q += q32;
+    r += r32;
+    if (r >= npl) { r -= npl; ++q; }
+  }
 }
 
 // Asynchronous global -> shared copies of 4 or 8 bytes (the weights of the next row).
@@ -68,70 +104,41 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 __device__ __forceinline__ uint32_t fixp(float w, int sh) { return small_fixp(w, sh); }
 __device__ __forceinline__ uint32_t fixp(double w, int sh) { return __double2uint_rz(ldexp(w, sh)); }
 
-// First index in [lo, hi) whose key is > x (pred gt) or >= x (pred ge); hi when none.  key(i) is
-// non-decreasing.  Starts with a gallop from lo, so that a cursor that moves little costs a few
-// loads.
-template <bool kStrict, typename Key>
-__device__ __forceinline__ int gallop_first(int lo, int hi, uint64_t x, Key key) {
-  auto past = [&](int i) { return kStrict ? key(i) > x : key(i) >= x; };
-  if (lo >= hi || past(lo)) return lo;
-  int step = 1;                                   // key(lo) fails the test
-  int a = lo;                                     // invariant: key(a) fails
-  while (a + step < hi && !past(a + step)) {
-    a += step;
-    step <<= 1;
-  }
-  int b = min(a + step, hi);                      // b == hi or key(b) passes
-  ++a;
-  while (a < b) {
-    const int mid = (a + b) >> 1;
-    if (past(mid)) b = mid; else a = mid + 1;
-  }
-  return a;
-}
-
-// Build one row.  w: the K weights, staged in shared memory; A: the value the row must sum to
-// (checked when check_A, to tol A + atol: a row whose spectral weight is at the rounding level
-// of G, such as an orbital no open channel reaches, carries only rounding noise); out: K
-// entries; rowsum_out: receives the row sum.  s_u, s_c:
-// 32 * alias_pitch(K) u64 each; s_x: K u32.  after_stage() is called by every lane once w has
-// been read (the caller reuses w's buffer for the next row).
+// Build one row.  sm.stage: the K weights, item i at its slot (alias_strided); A: the value the
+// row must sum to (checked when check_A, to tol A + atol: a row whose spectral weight is at the
+// rounding level of G, such as an orbital no open channel reaches, carries only rounding noise);
+// out: K entries; rowsum_out: receives the row sum.  after_stage() is called by every lane once
+// the weights have been read (the caller reuses the stage for the next row).
 template <typename R, typename After>
-__device__ void alias_row(const R* w, int K, double A, bool check_A, double tol, double atol,
-                          uint64_t* __restrict__ out, double* rowsum_out, uint64_t* s_u,
-                          uint64_t* s_c, uint32_t* s_x, int32_t* err, After after_stage) {
+__device__ void alias_row(const AliasSmem& sm, int K, double A, bool check_A, double tol,
+                          double atol, uint64_t* __restrict__ out, double* rowsum_out,
+                          int32_t* err, After after_stage) {
   const int lane = threadIdx.x & 31;
   const unsigned FULL = 0xffffffffu;
   const int npl = alias_npl(K), pitch = alias_pitch(K);
-  // slots of items lane, lane + 32, ...: (quotient, remainder) by npl, stepped by 32
-  const int q32 = 32 / npl, r32 = 32 - q32 * npl;
-  const int qlane = lane / npl, rlane = lane - qlane * npl;
   const int i0 = lane * npl;                                    // this lane's items [i0, i1)
   const int i1 = min(K, i0 + npl);
   const int mine = max(0, i1 - i0);
-  uint64_t* my_u = s_u + lane * pitch;
-  R* s_w = reinterpret_cast<R*>(s_c);
-  R* my_w = s_w + lane * pitch;
-  // pass 1 (coalesced): stage the row, largest weight; FP64 rows also take their FP64 sum here
-  // (lane-strided order, tree to lane 0)
+  uint64_t* my_u = sm.u + lane * pitch;
+  const R* w = reinterpret_cast<const R*>(sm.stage);
+  const R* my_w = w + lane * pitch;
+  // pass 1: largest weight; FP64 rows also take their FP64 sum here (lane-strided order, tree to
+  // lane 0)
   R wmax = 0;
   bool bad = false;
-  double part = 0.0;
-  for (int i = lane, q = qlane, rm = rlane; i < K; i += 32) {
-    const R v = w[i];
-    s_w[q * pitch + rm] = v;
-    q += q32;
-    rm += r32;
-    if (rm >= npl) { rm -= npl; ++q; }
-    bad |= !(v >= 0) || !isfinite(v);
-    if (v > wmax && isfinite(v)) wmax = v;
-    if (sizeof(R) == 8) part += (double)v;
+  for (int k = 0; k < mine; ++k) {
+    const R v = my_w[k];
+    const bool ok = v >= 0 && v < (R)INFINITY;
+    bad |= !ok;
+    if (ok && v > wmax) wmax = v;
   }
-  __syncwarp();
-  after_stage();
+  double part = 0.0;
+  if (sizeof(R) == 8) alias_strided(K, [&](int, int slot) { part += (double)w[slot]; });
   for (int off = 16; off > 0; off >>= 1) wmax = max(wmax, __shfl_xor_sync(FULL, wmax, off));
   if (__any_sync(FULL, bad) && lane == 0) atomicOr(err, ERR_NONFINITE);
   if (!(wmax > 0)) {
+    __syncwarp();
+    after_stage();
     if (lane == 0) *rowsum_out = 0.0;
     if (lane == 0 && check_A && A > 1e-300 && A > atol) atomicOr(err, ERR_ROWSUM);
     for (int i = lane; i < K; i += 32) out[i] = pack(0xffffffffu, (uint32_t)i);
@@ -141,15 +148,26 @@ __device__ void alias_row(const R* w, int K, double A, bool check_A, double tol,
   if (sizeof(R) == 4) frexpf((float)wmax, &ex);   // wmax = f 2^ex, f in [0.5, 1)
   else frexp((double)wmax, &ex);
   const int sh = 32 - ex;                          // wmax 2^sh in [2^31, 2^32)
-  // pass 2 (own block): integer weights m_i, T = sum m_i
-  uint64_t T = 0;
-  for (int k = 0; k < mine; ++k) {
+  auto unit = [&](int k) {
     const R v = my_w[k];
-    const uint32_t m = (v > 0 && isfinite(v)) ? fixp(v, sh) : 0u;
-    my_u[k] = m;
+    return v > 0 && v < (R)INFINITY ? fixp(v, sh) : 0u;
+  };
+  // pass 2: integer weights m_i, T = sum m_i, and the first index of the largest
+  uint64_t T = 0;
+  uint32_t mmax = 0;
+  int imax = 0x7fffffff;
+  for (int k = 0; k < mine; ++k) {
+    const uint32_t m = unit(k);
+    if (sizeof(R) == 8) my_u[k] = m;
     T += m;
+    if (m > mmax) { mmax = m; imax = i0 + k; }
   }
-  for (int off = 16; off > 0; off >>= 1) T += __shfl_xor_sync(FULL, T, off);
+  for (int off = 16; off > 0; off >>= 1) {
+    T += __shfl_xor_sync(FULL, T, off);
+    const uint32_t om = __shfl_xor_sync(FULL, mmax, off);
+    const int oi = __shfl_xor_sync(FULL, imax, off);
+    if (om > mmax || (om == mmax && oi < imax)) { mmax = om; imax = oi; }
+  }
   // row sum: FP64 weights are summed in FP64; FP32 weights use the exact fixed-point sum
   // (within K 2^-32 of the largest weight)
   if (sizeof(R) == 8)
@@ -162,36 +180,49 @@ __device__ void alias_row(const R* w, int K, double A, bool check_A, double tol,
     *rowsum_out = total;
     if (check_A && A > 1e-300 && fabs(total - A) > tol * A + atol) atomicOr(err, ERR_ROWSUM);
   }
-  // pass 3: u_i = floor(m_i K 2^32 / T) = (m_i K) (2^94 / T) / 2^62, with the 128-bit product
   rcp = __shfl_sync(FULL, rcp, 0);
-  const uint64_t target = (uint64_t)K << 32;
-  uint64_t usum = 0, umax = 0;
-  int imax = 0x7fffffff;
+  // pass 3: u_i = floor(m_i K 2^32 / T) = (m_i K) (2^94 / T) / 2^62, a 48 x 63-bit product in
+  // 32-bit limbs.  m_i <= T, so no unit count exceeds K 2^32; K 2^32 / T > 1 + 2^-33 exceeds the
+  // reciprocal's error, so u_i grows strictly with m_i and the largest m has the largest u.
+  // Lights (u < 2^32) carry deficits 2^32 - u, heavies excesses u - 2^32.
+  const uint32_t r0 = (uint32_t)rcp, r1 = (uint32_t)(rcp >> 32);
+  uint64_t usum = 0, dl = 0;
+  uint32_t cnt = 0;                               // lights | heavies << 16
   for (int k = 0; k < mine; ++k) {
-    const uint64_t q = my_u[k] * (uint64_t)K;
-    const uint64_t hi = __umul64hi(q, rcp), lo = q * rcp;
-    uint64_t u = (hi << 2) | (lo >> 62);
-    if (u > target) u = target;
+    const uint32_t m = sizeof(R) == 8 ? (uint32_t)my_u[k] : unit(k);
+    const uint64_t q = (uint64_t)m * (uint32_t)K;
+    const uint32_t q0 = (uint32_t)q, q1 = (uint32_t)(q >> 32);
+    const uint64_t p = (uint64_t)q0 * r1 + (((uint64_t)q0 * r0) >> 32);
+    const uint64_t s = (uint64_t)q1 * r0 + (uint32_t)p;
+    const uint64_t hi = (uint64_t)q1 * r1 + (p >> 32) + (s >> 32);
+    const uint64_t u = (hi << 2) | ((uint32_t)s >> 30);
     my_u[k] = u;
     usum += u;
-    if (u > umax) { umax = u; imax = i0 + k; }   // first index of the lane's maximum
+    const bool heavy = u >= kSlot;
+    cnt += heavy ? 1u << 16 : 1u;
+    dl += heavy ? 0u : (uint32_t)u;               // lights' units
   }
-  for (int off = 16; off > 0; off >>= 1) {
-    usum += __shfl_xor_sync(FULL, usum, off);
-    const uint64_t om = __shfl_xor_sync(FULL, umax, off);
-    const int oi = __shfl_xor_sync(FULL, imax, off);
-    if (om > umax || (om == umax && oi < imax)) { umax = om; imax = oi; }
+  __syncwarp();
+  after_stage();
+  const int nl_mine = (int)(cnt & 0xffffu), nh_mine = (int)(cnt >> 16);
+  uint64_t dh = usum - dl - ((uint64_t)nh_mine << 32);          // excesses
+  dl = ((uint64_t)nl_mine << 32) - dl;                            // deficits
+  for (int off = 16; off > 0; off >>= 1) usum += __shfl_xor_sync(FULL, usum, off);
+  if (i0 <= imax && imax < i1) {                  // the signed remainder goes to the largest item
+    const uint64_t rem = ((uint64_t)K << 32) - usum;
+    const uint64_t u0 = my_u[imax - i0], u1 = u0 + rem;
+    my_u[imax - i0] = u1;
+    if (u0 >= kSlot) {
+      dh += rem;
+    } else if (u1 >= kSlot) {
+      cnt += (1u << 16) - 1u;
+      dl -= kSlot - u0;
+      dh += u1 - kSlot;
+    } else {
+      dl -= rem;
+    }
   }
-  if (i0 <= imax && imax < i1) my_u[imax - i0] += target - usum;   // signed remainder
-  // pass 4: lights (u < 2^32) carry deficits 2^32 - u, heavies excesses u - 2^32; exclusive
-  // prefix over the lanes of counts and sums
-  uint32_t cnt = 0;                               // lights | heavies << 16
-  uint64_t dl = 0, dh = 0;
-  for (int k = 0; k < mine; ++k) {
-    const uint64_t u = my_u[k];
-    if (u >= kSlot) { cnt += 1u << 16; dh += u - kSlot; }
-    else { cnt += 1u; dl += kSlot - u; }
-  }
+  // exclusive prefix over the lanes of counts and sums
   uint32_t cx = cnt;
   uint64_t lx = dl, hx = dh;                      // inclusive scans
   for (int off = 1; off < 32; off <<= 1) {
@@ -204,68 +235,65 @@ __device__ void alias_row(const R* w, int K, double A, bool check_A, double tol,
   const int nl = (int)(ctot & 0xffffu), nh = (int)(ctot >> 16);
   int r = (int)((cx - cnt) & 0xffffu), j = (int)((cx - cnt) >> 16);   // first light / heavy
   uint64_t runl = lx - dl, runh = hx - dh;                             // of this lane
-  __syncwarp();                                   // s_w (in s_c) is dead from here
-  // pass 5: Lc_r (inclusive deficit prefix, light order) from the front of s_c, Ec_j (inclusive
+  // pass 4: Lc_r (inclusive deficit prefix, light order) from the front of s_c, Ec_j (inclusive
   // excess prefix, heavy order) from the back; s_x holds the item index of each
   for (int k = 0; k < mine; ++k) {
     const uint64_t u = my_u[k];
-    if (u >= kSlot) {
-      runh += u - kSlot;
-      s_c[K - 1 - j] = runh;
-      s_x[K - 1 - j] = (uint32_t)(i0 + k);
-      ++j;
-    } else {
-      runl += kSlot - u;
-      s_c[r] = runl;
-      s_x[r] = (uint32_t)(i0 + k);
-      ++r;
-    }
+    const bool heavy = u >= kSlot;
+    if (heavy) runh += u - kSlot;
+    else runl += kSlot - u;
+    const int at = heavy ? K - 1 - j : r;
+    sm.c[at] = heavy ? runh : runl;
+    sm.x[at] = (uint16_t)(i0 + k);
+    j += heavy;
+    r += !heavy;
   }
   __syncwarp();
-  if (nh == 0) {   // cannot happen when sum(u) == K 2^32; keep the row drawable anyway
+  if (nl == 0 || nh == 0) {   // every item holds one slot (nh == 0 cannot happen: the sum is K 2^32)
     for (int i = lane; i < K; i += 32) out[i] = pack(0xffffffffu, (uint32_t)i);
     return;
   }
-  auto Ec = [&](int jj) { return s_c[K - 1 - jj]; };
-  auto Lc = [&](int rr) { return s_c[rr]; };
-  // pass 6: entries, into s_u by item index (s_u is dead from here).  The lanes split the light
-  // list, then the heavy list, into contiguous ranges, each searched from a cursor that moves
-  // forward.
-  // Light r (start Lc_{r-1}, u_r = 2^32 - (Lc_r - Lc_{r-1})) aliases the heavy whose excess
-  // interval [Ec_{j-1}, Ec_j) contains its start.
+  auto Ec = [&](int jj) { return sm.c[K - 1 - jj]; };
+  auto Xh = [&](int jj) { return (uint32_t)sm.x[K - 1 - jj]; };
+  auto Lc = [&](int rr) { return sm.c[rr]; };
+  // pass 5: entries, into s_u by item index (s_u is dead from here).  The lanes split the list of
+  // lights into contiguous ranges.  Light r (start Lc_{r-1}, u_r = 2^32 - (Lc_r - Lc_{r-1}))
+  // aliases heavy j, the first whose excess interval [Ec_{j-1}, Ec_j) reaches past its start;
+  // the heavies (but the last) that end within (Lc_{r-1}, Lc_r] are consumed past their excess
+  // by this light: heavy j keeps 2^32 - (Lc_r - Ec_j) and aliases heavy j + 1.  Heavies without
+  // excess at the front of the list (Ec = 0) and the last heavy are full.
   {
     const int ra = (lane * nl) >> 5, rb = ((lane + 1) * nl) >> 5;
-    uint64_t st = ra == 0 ? 0ull : Lc(ra - 1);
-    int jc = 0;
-    for (int rr = ra; rr < rb; ++rr) {
-      const uint64_t Lr = Lc(rr);
-      jc = gallop_first<true>(jc, nh, st, Ec);          // first j with Ec_j > st
-      const int jj = jc < nh ? jc : nh - 1;
-      s_u[s_x[rr]] = pack((uint32_t)(kSlot - (Lr - st)), s_x[K - 1 - jj]);
-      st = Lr;
-    }
-  }
-  // Heavy j (not the last, Ec_j > 0) is consumed past its excess by the light interval
-  // (Lc_{r-1}, Lc_r] containing Ec_j: it keeps 2^32 - (Lc_r - Ec_j) and aliases heavy j + 1.
-  {
-    const int ja = (lane * nh) >> 5, jb = ((lane + 1) * nh) >> 5;
-    int rc = 0;
-    for (int jj = ja; jj < jb; ++jj) {
-      const uint32_t self = s_x[K - 1 - jj];
-      uint64_t e = pack(0xffffffffu, self);
-      const uint64_t Ej = Ec(jj);
-      if (jj < nh - 1 && Ej > 0) {
-        rc = gallop_first<false>(rc, nl, Ej, Lc);       // first r with Lc_r >= Ej
-        if (rc < nl) {
-          const uint64_t used = Lc(rc) - Ej;            // consumed beyond the excess, <= 2^32
-          if (used > 0) e = pack((uint32_t)(kSlot - used), s_x[K - 1 - (jj + 1)]);
-        }
+    if (ra < rb) {
+      uint64_t st = ra == 0 ? 0ull : Lc(ra - 1);
+      int jc = 0, hi = nh - 1;                            // first j with Ec_j > st, or the last
+      while (jc < hi) {
+        const int mid = (jc + hi) >> 1;
+        if (Ec(mid) > st) hi = mid; else jc = mid + 1;
       }
-      s_u[self] = e;
+      if (ra == 0)
+        for (int jj = 0; jj < jc; ++jj) sm.u[Xh(jj)] = pack(0xffffffffu, Xh(jj));
+      uint64_t Ej = Ec(jc);
+      uint32_t xj = Xh(jc);
+      for (int rr = ra; rr < rb; ++rr) {
+        const uint64_t Lr = Lc(rr);
+        sm.u[sm.x[rr]] = pack((uint32_t)(st - Lr), xj);    // 2^32 - (Lr - st)
+        while (jc < nh - 1 && Ej <= Lr) {
+          const uint32_t xn = Xh(jc + 1);
+          const uint64_t used = Lr - Ej;                   // consumed beyond the excess, <= 2^32
+          sm.u[xj] = used > 0 ? pack((uint32_t)(kSlot - used), xn) : pack(0xffffffffu, xj);
+          ++jc;
+          Ej = Ec(jc);
+          xj = xn;
+        }
+        st = Lr;
+      }
     }
+    if (lane == 0) sm.u[Xh(nh - 1)] = pack(0xffffffffu, Xh(nh - 1));
   }
   __syncwarp();
-  for (int i = lane; i < K; i += 32) out[i] = s_u[i];
+  for (int i = lane; i < K; i += 32) out[i] = sm.u[i];
+  __syncwarp();
 }
 
 template <typename R>
@@ -275,13 +303,10 @@ __global__ void alias_kernel(const TaskDesc* __restrict__ tasks, int n_tasks, ui
                              uint64_t* __restrict__ tab, uint64_t* __restrict__ mode_tab,
                              int32_t* err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
-  unsigned char* base = smem_raw + (size_t)warp * alias_warp_bytes(cap, (int)sizeof(R));
-  uint64_t* s_u = reinterpret_cast<uint64_t*>(base);
-  uint64_t* s_c = s_u + (size_t)32 * alias_pitch(cap);
-  uint32_t* s_x = reinterpret_cast<uint32_t*>(s_c + (size_t)32 * alias_pitch(cap));
-  unsigned char* s_stage = base + alias_stage_off(cap);
+  const AliasSmem sm(smem_raw + (size_t)warp * alias_warp_bytes(cap, (int)sizeof(R)), cap,
+                     (int)sizeof(R));
   const uint32_t stride = gridDim.x * nwarps;
   // task owning a job: jobs of a warp only increase, so the search starts at the last task found
   int hint = 0;
@@ -293,18 +318,18 @@ __global__ void alias_kernel(const TaskDesc* __restrict__ tasks, int n_tasks, ui
     }
     return lo;
   };
-  // the weights of job jb go to s_stage by asynchronous copies (one commit group)
+  // the weights of job jb go to the stage by asynchronous copies (one commit group)
   auto stage = [&](uint32_t jb) {
     const TaskDesc& d = tasks[find(jb)];
     const int row = (int)(jb - d.row_base);
     if (row < d.rows) {
       const R* src = weights + d.wt_off + (uint64_t)row * d.K;
-      R* dst = reinterpret_cast<R*>(s_stage);
-      for (int i = lane; i < d.K; i += 32) cp_async<(int)sizeof(R)>(dst + i, src + i);
+      R* dst = reinterpret_cast<R*>(sm.stage);
+      alias_strided(d.K, [&](int i, int slot) { cp_async<(int)sizeof(R)>(dst + slot, src + i); });
     } else {
       const double* src = mode_w + d.mode_off + (row - d.rows) * d.W;
-      double* dst = reinterpret_cast<double*>(s_stage);
-      for (int i = lane; i < d.W; i += 32) cp_async<8>(dst + i, src + i);
+      double* dst = reinterpret_cast<double*>(sm.stage);
+      alias_strided(d.W, [&](int i, int slot) { cp_async<8>(dst + slot, src + i); });
     }
     cp_async_commit();
   };
@@ -322,14 +347,12 @@ __global__ void alias_kernel(const TaskDesc* __restrict__ tasks, int n_tasks, ui
     cp_async_wait_all();
     __syncwarp();
     if (row < d.rows) {
-      alias_row<R>(reinterpret_cast<const R*>(s_stage), d.K, A, true, tol, 1e-13 / d.t,
-                   tab + d.tab_off + (uint64_t)row * d.K, rowsum + job, s_u, s_c, s_x, err,
-                   after);
+      alias_row<R>(sm, d.K, A, true, tol, 1e-13 / d.t, tab + d.tab_off + (uint64_t)row * d.K,
+                   rowsum + job, err, after);
     } else {
       const int p = row - d.rows;
-      alias_row<double>(reinterpret_cast<const double*>(s_stage), d.W, A, true, 1e-9, 1e-13 / d.t,
-                        mode_tab + d.mode_off + p * d.W, rowsum + job, s_u, s_c, s_x, err,
-                        after);
+      alias_row<double>(sm, d.W, A, true, 1e-9, 1e-13 / d.t, mode_tab + d.mode_off + p * d.W,
+                        rowsum + job, err, after);
     }
     __syncwarp();
   }
@@ -508,13 +531,11 @@ __global__ void energy_alias_kernel(const TaskDesc* __restrict__ tasks, int n_ta
                                     int cap, double sigma, const double* __restrict__ rowsum,
                                     uint64_t* __restrict__ etab, int32_t* err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
-  unsigned char* base = smem_raw + (size_t)warp * alias_warp_bytes(cap, (int)sizeof(double));
-  uint64_t* s_u = reinterpret_cast<uint64_t*>(base);
-  uint64_t* s_c = s_u + (size_t)32 * alias_pitch(cap);
-  uint32_t* s_x = reinterpret_cast<uint32_t*>(s_c + (size_t)32 * alias_pitch(cap));
-  double* s_w = reinterpret_cast<double*>(base + alias_stage_off(cap));
+  const AliasSmem sm(smem_raw + (size_t)warp * alias_warp_bytes(cap, (int)sizeof(double)), cap,
+                     (int)sizeof(double));
+  double* s_w = reinterpret_cast<double*>(sm.stage);
   for (uint32_t job = blockIdx.x * nwarps + warp; job < total_jobs; job += gridDim.x * nwarps) {
     int lo = 0, hi = n_tasks - 1;
     while (lo < hi) {
@@ -526,16 +547,16 @@ __global__ void energy_alias_kernel(const TaskDesc* __restrict__ tasks, int n_ta
     const int i = (int)(job - job_base[lo]);
     const int nE = ed.nE;
     const double inv2s2 = sigma > 0.0 ? 0.5 / (sigma * sigma) : 0.0;
-    for (int ep = lane; ep < nE; ep += 32) {
+    alias_strided(nE, [&](int ep, int slot) {
       const TaskDesc& dp = tasks[ed.t0 + ep];
       const double dE = dp.E - d.E;
       const double K = sigma > 0.0 ? exp(-dE * dE * inv2s2) : (ep == d.e_idx ? 1.0 : 0.0);
-      s_w[ep] = dp.w_E * K * rowsum[dp.row_base + i];
-    }
+      s_w[slot] = dp.w_E * K * rowsum[dp.row_base + i];
+    });
     __syncwarp();
     double total = 0.0;
-    alias_row<double>(s_w, nE, 0.0, false, 0.0, 0.0, etab + ed.eoff + (uint64_t)i * nE, &total,
-                      s_u, s_c, s_x, err, [] {});
+    alias_row<double>(sm, nE, 0.0, false, 0.0, 0.0, etab + ed.eoff + (uint64_t)i * nE, &total,
+                      err, [] {});
     __syncwarp();
   }
 }

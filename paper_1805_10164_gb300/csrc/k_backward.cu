@@ -377,7 +377,7 @@ __global__ void grad_diag_kernel(TaskDesc d, const C* __restrict__ G, const C* _
 // seed_w * w_E (f_p - f_q) dT/dtheta.  One CTA per (wire, 256 sites), one thread per site; the
 // tasks' factors, two FP64 hyperbolic tangents each, are formed once per CTA, a task per thread
 // (formed by every site's thread on one CTA per wire they took 0.58 ms on the W=16 x L=100,
-// 16-energy gradient; @@ ms now).
+// 16-energy gradient; 0.012 ms now).
 __device__ __forceinline__ double fermi_b(double E, double mu, double kT) {
   return 0.5 * (1.0 - tanh(0.5 * (E - mu) / kT));
 }

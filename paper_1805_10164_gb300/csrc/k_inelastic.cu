@@ -42,7 +42,7 @@ __device__ __forceinline__ void add64(unsigned* lohi, unsigned v) {
 // energy draw.  Counts stay in registers while a lane's walkers belong to one task: added to
 // the block's shared tally per walk, three same-address shared atomics a walk serialised over
 // the warp's lanes and bounded the kernel (W=10 x L=50, 64 energies, 1e6 walkers each:
-// @@BEFORE -> @@AFTER ms; what is left is the latency of the two dependent gathers).
+// 3.64 -> 1.62 ms; what is left is the latency of the two dependent gathers).
 __global__ void __launch_bounds__(kThreads) inelastic_walk_kernel(
     const TaskDesc* __restrict__ tasks, int task0, int n_tasks,
     const EnergyDesc* __restrict__ edesc, const uint64_t* __restrict__ tab,
