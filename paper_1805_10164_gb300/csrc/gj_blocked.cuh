@@ -6,21 +6,21 @@
 // inversion is what counts.  One pivot at a time (cta_gj) needs two barriers and ~150
 // instructions a warp per pivot; at W = 64 that took 67 us a slice.  Here four pivots make a
 // panel, and one barrier serves a panel:
-//   * warp 0 (the panel warp) holds the next panel's columns in registers, a lane two rows: it
-//     applies the current panel's four pivots to them, then eliminates within the panel, the
-//     pivot row broadcast by shuffles.  It publishes the four pivot columns f_k (at time k) and
-//     the reciprocals;
-//   * meanwhile the other warps apply the current panel to every other column: a thread owns
+//   * the panel warps (a lane a row) bring the next panel's four columns up to date with the
+//     current panel, pass its four pivot rows around, eliminate that 4 x 4 block - every lane
+//     for itself, which costs no exchange within the serial chain of reciprocals - and then
+//     their own rows, and publish the four pivot columns f_k (at time k) and the reciprocals;
+//   * meanwhile the column warps apply the current panel to every other column: a thread owns
 //     one column and up to eight rows, forms its column's four t_k = a_kj / a_kk from the four
-//     pivot rows, and updates its entries from registers.  The block is read from one of two
-//     buffers and written to the other, so no thread waits for another within a panel.
+//     pivot rows, and updates its entries four rows at a time.  The block is read from one of
+//     two buffers and written to the other, so no thread waits for another within a panel.
 // Each entry sees the same operations in the same order as in cta_gj
 //   a_kk <- 1/a_kk;  a_kj <- t = a_kj / a_kk;  a_ik <- -a_ik / a_kk;  a_ij <- a_ij - a_ik t
 // for k = 0, 1, ..., each rounding written out (bg_mul, bg_sub, bg_col), so the inverse does not
 // depend on how a compiler contracts the expressions and stays what cta_gj gives.
-//
-// The panel warp shares its scheduler (warps 0, 4, 8, ...) with fewer column warps than the
-// other three schedulers hold: its serial chain is as long as the other warps' work.
+// Measured at W = 64: 67 us a slice with one pivot at a time; 26 with one panel warp of two rows
+// a lane and the pivot row broadcast by shuffles; 24 as it is.  Updates as (re, im) pairs
+// (f32x2, two columns a thread, half the warps) measured 30: too few warps to hide the latencies.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -34,16 +34,24 @@ namespace {
 constexpr int kBgPitch = 65;                  // row pitch: rows and columns free of conflicts
 constexpr int kBgGroups = 8;                  // row groups of the column warps
 
-// NH halves of 32 columns: W <= 32 -> 1, W <= 64 -> 2.
-template <int NH> constexpr int kBgThreads = NH == 2 ? 19 * 32 : 11 * 32;
-// column unit (half, row group) of a warp, -1 for the panel warp and the warps that only keep
-// the schedulers balanced
+// NH halves of 32 columns: W <= 32 -> 1, W <= 64 -> 2.  Warps 0 .. NH - 1 are the panel warps; the
+// column units (half, row group) go to warps so that the schedulers (warp mod 4) with a panel
+// warp, whose chain issues as much as two units, hold fewer of them.
+template <int NH> constexpr int kBgThreads = NH == 2 ? 20 * 32 : 12 * 32;
 template <int NH>
 __device__ __forceinline__ int bg_unit(int warp) {
-  if (NH == 1) return (warp & 3) ? (warp >> 2) * 3 + (warp & 3) - 1 : -1;   // 1,2,3,5,6,7,9,10
-  if (warp >= 17) return warp - 3;                                        // 17, 18 -> 14, 15
-  if (warp & 3) return (warp >> 2) * 3 + (warp & 3) - 1;                  // 0 .. 11
-  return warp == 4 ? 12 : warp == 8 ? 13 : -1;
+  if (NH == 2) {
+    if (warp & 2) return (warp >> 2) * 2 + (warp & 1);            // 2, 3, 6, 7, .. 19 -> 0 .. 9
+    return warp >= 4 && warp < 16 ? 8 + (warp >> 2) * 2 + (warp & 1) : -1;   // -> 10 .. 15
+  }
+  // 1, 2, 3, 5, 6, 7, 9, 10 -> 0 .. 7
+  return (warp & 3) && warp < 11 ? (warp >> 2) * 3 + (warp & 3) - 1 : -1;
+}
+// the warps without columns that fetch the next slice's diagonal (its half h), -1 otherwise
+template <int NH>
+__device__ __forceinline__ int bg_side(int warp) {
+  if (NH == 2) return warp == 16 ? 0 : warp == 17 ? 1 : -1;
+  return warp == 8 ? 0 : -1;
 }
 
 // a b, a - b c, -(b c), 1 / a with every rounding explicit
@@ -66,8 +74,9 @@ __device__ __forceinline__ cf bg_inv(cf a) {
 struct BgShared {
   cf B[2][64 * kBgPitch];       // the block, ping-pong
   float4 F[2][64][2];           // pivot columns f_q of a panel, a row's four together
+  float4 t[2][4][2];            // per panel warp: the current panel's t_q of the next columns
+  float4 blk[4][2];             // the next panel's pivot rows
   cf inv[2][4];                 // reciprocals of the panel's pivots
-  cf t[4][4];                   // the current panel's t_q of the next panel's columns
   cf diag[2][64];               // diagonal of E - H - Sigma_s of a slice
   int undephased[2][2];         // nonzero: the slice (half of it) has a site without dephasing
   int perm[64];                 // pivoted fallback
@@ -75,55 +84,74 @@ struct BgShared {
   int bad;                      // a pivot without a finite reciprocal
 };
 
-// Eliminate the nb pivots k1 .. k1 + nb - 1 within the panel's columns v (lane's rows lane and
-// lane + 32), leaving the pivot columns in f and the reciprocals in inv; publishes them in
-// buffer buf and the panel's columns, now as after these pivots, in Bout.
+__device__ __forceinline__ void bg_put4(float4* dst, const cf (&v)[4]) {
+  dst[0] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+  dst[1] = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
+}
+__device__ __forceinline__ void bg_get4(const float4* src, cf (&v)[4]) {
+  const float4 a = src[0], b = src[1];
+  v[0] = cf{a.x, a.y};
+  v[1] = cf{a.z, a.w};
+  v[2] = cf{b.x, b.y};
+  v[3] = cf{b.z, b.w};
+}
+// The panel warps' own barrier
 template <int NH>
+__device__ __forceinline__ void bg_panel_sync() {
+  if (NH == 1) __syncwarp();
+  else asm volatile("bar.sync 1, 64;\n" ::: "memory");
+}
+
+// Panel warps: eliminate the nb pivots k1 .. k1 + nb - 1 within the panel's columns v of this
+// lane's row, leaving the pivot columns in f and the reciprocals in inv; publishes them in
+// buffer buf and the panel's columns, now as after these pivots, in Bout.
+// kFull: nb = 4 (every panel but perhaps the last), without branches between the pivots.
+template <int NH, bool kFull>
 __device__ __forceinline__ void bg_factor(BgShared& S, int k1, int nb, int buf, cf* Bout,
-                                          cf (&v)[NH][4], cf (&f)[NH][4], cf (&inv)[4]) {
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
+                                          cf (&v)[4], cf (&f)[4], cf (&inv)[4]) {
+  const int row = threadIdx.x;                      // panel warps are warps 0 .. NH - 1
+  const int own = row - k1;                         // 0 .. 3: this lane's row is pivot row `own`
+  if ((unsigned)own < 4u) bg_put4(S.blk[own], v);
+  bg_panel_sync<NH>();
+  // the 4 x 4 block: t_q and 1 / a_kk of each pivot, from the rows below it only
+  cf D[4][4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) bg_get4(S.blk[r], D[r]);
   bool bad = false;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    if (q < nb) {
-      const int k = k1 + q, src = k & 31;
-      cf r[4];
-#pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
-        const int c = (q + cc) & 3;                        // the pivot first
-        const cf own = NH == 2 && k >= 32 ? v[NH - 1][c] : v[0][c];
-        r[c].x = __shfl_sync(FULL, own.x, src);
-        r[c].y = __shfl_sync(FULL, own.y, src);
-      }
-      const cf iv = bg_inv(r[q]);
+    if (kFull || q < nb) {
+      const cf iv = bg_inv(D[q][q]);
       bad |= !finite_c(iv);
-      cf t[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) t[c] = c == q ? iv : bg_mul(r[c], iv);
-#pragma unroll
-      for (int m = 0; m < NH; ++m) {
-        const bool me = lane + 32 * m == k;
-        const cf fm = v[m][q];
-        f[m][q] = fm;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const cf n = c == q ? bg_col(fm, iv) : bg_sub(v[m][c], fm, t[c]);
-          v[m][c] = me ? t[c] : n;
-        }
-      }
       inv[q] = iv;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) D[q][c] = c == q ? iv : bg_mul(D[q][c], iv);    // t_q
+#pragma unroll
+      for (int r = q + 1; r < 4; ++r) {
+        const cf fr = D[r][q];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          D[r][c] = c == q ? bg_col(fr, iv) : bg_sub(D[r][c], fr, D[q][c]);
+      }
     }
   }
+  // this lane's row
 #pragma unroll
-  for (int m = 0; m < NH; ++m) {
-    const int row = lane + 32 * m;
-    S.F[buf][row][0] = make_float4(f[m][0].x, f[m][0].y, f[m][1].x, f[m][1].y);
-    S.F[buf][row][1] = make_float4(f[m][2].x, f[m][2].y, f[m][3].x, f[m][3].y);
+  for (int q = 0; q < 4; ++q) {
+    if (kFull || q < nb) {
+      const cf fq = v[q];
+      f[q] = fq;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) Bout[row * kBgPitch + k1 + c] = v[m][c];
+      for (int c = 0; c < 4; ++c) {
+        const cf n = c == q ? bg_col(fq, inv[q]) : bg_sub(v[c], fq, D[q][c]);
+        v[c] = own == q ? D[q][c] : n;
+      }
+    }
   }
-  if (lane == 0) {
+  bg_put4(S.F[buf][row], f);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) Bout[row * kBgPitch + k1 + c] = v[c];
+  if (row == 0) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) S.inv[buf][q] = inv[q];
     if (bad) S.bad = 1;
@@ -131,29 +159,29 @@ __device__ __forceinline__ void bg_factor(BgShared& S, int k1, int nb, int buf, 
 }
 
 // Invert the block.  On entry the columns >= 4 are in S.B[0], panel 0 has been eliminated by
-// bg_factor (buffer 0, columns in S.B[1]; the panel warp's f and inv from it), and the CTA has
+// bg_factor (buffer 0, columns in S.B[1]; the panel warps' f and inv from it), and the CTA has
 // synchronised.  On return (synchronised) the inverse is in S.B[NP & 1], NP = ceil(W / 4);
-// S.bad is set if some pivot had no finite reciprocal.  side(p) is called by the warps without
-// columns during panel 0.
+// S.bad is set if some pivot had no finite reciprocal.  side() is called by the warps without
+// rows during panel 0.
 template <int NH, typename Side>
-__device__ __forceinline__ void bg_invert(BgShared& S, int W, cf (&v)[NH][4], cf (&f)[NH][4],
-                                          cf (&inv)[4], Side side) {
+__device__ __forceinline__ void bg_invert(BgShared& S, int W, cf (&v)[4], cf (&f)[4], cf (&inv)[4],
+                                          Side side) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int unit = bg_unit<NH>(warp);
-  const int NP = (W + 3) >> 2;
   const int j = NH == 2 ? (unit & 1) * 32 + lane : lane;
   const int g = NH == 2 ? unit >> 1 : unit;
+  const int NP = (W + 3) >> 2;
   for (int p = 0; p < NP; ++p) {
     const int k0 = 4 * p, k1 = k0 + 4, b = p & 1;
     cf* X = S.B[b];
     cf* Y = S.B[b ^ 1];
-    if (warp == 0) {
+    if (warp < NH) {
       if (p + 1 < NP) {
-        // panel p (four pivots, since another follows) applied to the columns of panel p + 1
+        // panel p (four pivots, since another follows) applied to the columns of panel p + 1:
+        // t_q of column lane & 3, exchanged through shared memory, then this lane's row
+        const int row = threadIdx.x;
 #pragma unroll
-        for (int m = 0; m < NH; ++m)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) v[m][c] = X[(lane + 32 * m) * kBgPitch + k1 + c];
+        for (int c = 0; c < 4; ++c) v[c] = X[row * kBgPitch + k1 + c];
         const int c0 = lane & 3;
         cf R[4], t[4];
 #pragma unroll
@@ -167,87 +195,138 @@ __device__ __forceinline__ void bg_invert(BgShared& S, int W, cf (&v)[NH][4], cf
             R[r] = bg_sub(R[r], q & 1 ? cf{ff.z, ff.w} : cf{ff.x, ff.y}, t[q]);
           }
         }
+        cf* ts = reinterpret_cast<cf*>(S.t[warp]);
         if (lane < 4) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) S.t[q][lane] = t[q];
+          for (int q = 0; q < 4; ++q) ts[4 * q + lane] = t[q];
         }
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
+          cf tq[4];
+          bg_get4(S.t[warp][q], tq);
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            const cf tq = S.t[q][c];
-#pragma unroll
-            for (int m = 0; m < NH; ++m) {
-              const cf n = bg_sub(v[m][c], f[m][q], tq);
-              v[m][c] = lane + 32 * m == k0 + q ? tq : n;
-            }
+            const cf n = bg_sub(v[c], f[q], tq[c]);
+            v[c] = row == k0 + q ? tq[c] : n;
           }
         }
-        bg_factor<NH>(S, k1, min(4, W - k1), b ^ 1, X, v, f, inv);
+        if (W - k1 >= 4) bg_factor<NH, true>(S, k1, 4, b ^ 1, X, v, f, inv);
+        else bg_factor<NH, false>(S, k1, W - k1, b ^ 1, X, v, f, inv);
       }
     } else if (unit >= 0) {
-      const int pj = j >> 2;
-      if (j < W && pj != p && pj != p + 1) {
-        const int nb = min(4, W - k0);
-        cf R[4], t[4];
+      const int nb = min(4, W - k0);
+      const bool act = j < W && (j >> 2) != p && (j >> 2) != p + 1;
+      // the t_q of this column; with fewer than four pivots left the rest come from rows >= W
+      // and are not used
+      cf R[4], t[4];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) R[r] = X[(k0 + r) * kBgPitch + j];   // rows >= W: unused
+      for (int r = 0; r < 4; ++r) R[r] = X[(k0 + r) * kBgPitch + j];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          t[q] = cf{0.f, 0.f};
-          if (q < nb) {
-            t[q] = bg_mul(R[q], S.inv[b][q]);
+      for (int q = 0; q < 4; ++q) {
+        t[q] = bg_mul(R[q], S.inv[b][q]);
 #pragma unroll
-            for (int r = q + 1; r < 4; ++r) {
-              const float4 ff = S.F[b][k0 + r][q >> 1];
-              R[r] = bg_sub(R[r], q & 1 ? cf{ff.z, ff.w} : cf{ff.x, ff.y}, t[q]);
+        for (int r = q + 1; r < 4; ++r) {
+          const float4 ff = S.F[b][k0 + r][q >> 1];
+          R[r] = bg_sub(R[r], q & 1 ? cf{ff.z, ff.w} : cf{ff.x, ff.y}, t[q]);
+        }
+      }
+      if (nb == 4) {
+        // the rows that hold no pivot of this panel, four at a time (rows >= W are computed
+        // from whatever the buffer holds and not stored)
+#pragma unroll
+        for (int rc = 0; rc < 8; rc += 4) {
+          if (g + kBgGroups * rc < W) {
+            cf a[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              const int i = g + kBgGroups * (rc + r);
+              a[r] = X[i * kBgPitch + j];
+              cf fi[4];
+              bg_get4(S.F[b][i], fi);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) a[r] = bg_sub(a[r], fi[q], t[q]);
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              const int i = g + kBgGroups * (rc + r);
+              if (act && i < W && (unsigned)(i - k0) >= 4u) Y[i * kBgPitch + j] = a[r];
             }
           }
         }
-        if (nb == 4) {
-#pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            const int i = g + kBgGroups * r;
-            if (i < W) {
-              cf a = X[i * kBgPitch + j];
-              const float4 f01 = S.F[b][i][0], f23 = S.F[b][i][1];
-              a = bg_sub(a, cf{f01.x, f01.y}, t[0]);
-              a = bg_sub(a, cf{f01.z, f01.w}, t[1]);
-              a = bg_sub(a, cf{f23.x, f23.y}, t[2]);
-              a = bg_sub(a, cf{f23.z, f23.w}, t[3]);
-              if ((unsigned)(i - k0) >= 4u) Y[i * kBgPitch + j] = a;
-            }
-          }
-        } else {
-          for (int i = g; i < k0; i += kBgGroups) {        // the last, narrower panel
-            cf a = X[i * kBgPitch + j];
-            const float4 f01 = S.F[b][i][0], f23 = S.F[b][i][1];
-            a = bg_sub(a, cf{f01.x, f01.y}, t[0]);
-            if (nb > 1) a = bg_sub(a, cf{f01.z, f01.w}, t[1]);
-            if (nb > 2) a = bg_sub(a, cf{f23.x, f23.y}, t[2]);
-            Y[i * kBgPitch + j] = a;
-          }
-        }
-        // the pivot row of this group, if it has one: t at its own pivot, updated by the others
-        const int own = (g - k0) & (kBgGroups - 1);
-        if (own < nb) {
-          const int i = k0 + own;
+      } else {
+        for (int i = g; i < k0; i += kBgGroups) {
           cf a = X[i * kBgPitch + j];
-          const float4 f01 = S.F[b][i][0], f23 = S.F[b][i][1];
-          const cf fi[4] = {cf{f01.x, f01.y}, cf{f01.z, f01.w}, cf{f23.x, f23.y},
-                            cf{f23.z, f23.w}};
+          cf fi[4];
+          bg_get4(S.F[b][i], fi);
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (q < nb) a = q == own ? t[q] : bg_sub(a, fi[q], t[q]);
-          Y[i * kBgPitch + j] = a;
+          for (int q = 0; q < 3; ++q)
+            if (q < nb) a = bg_sub(a, fi[q], t[q]);
+          if (act) Y[i * kBgPitch + j] = a;
         }
+      }
+      // the pivot row of this group, if it has one: t at its own pivot, updated by the others
+      const int own = (g - k0) & (kBgGroups - 1);
+      if (own < nb) {
+        const int i = k0 + own;
+        cf a = X[i * kBgPitch + j];
+        cf fi[4];
+        bg_get4(S.F[b][i], fi);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q < nb) a = q == own ? t[q] : bg_sub(a, fi[q], t[q]);
+        if (act) Y[i * kBgPitch + j] = a;
       }
     } else if (p == 0) {
       side();
     }
     __syncthreads();
   }
+}
+
+// Form a slice's block, entry (i, c) = form(i, c), and invert it; the inverse is in S.B[NP & 1] on
+// return (synchronised), false (uniformly) on a pivot without a finite reciprocal.  form may
+// read entry (i, c) of the block before, which is in S.B[NP & 1].  pivot: partial pivoting (the
+// slice has a site without dephasing).  side() is called by the warps without columns.
+template <int NH, typename Form, typename Side>
+__device__ __forceinline__ bool bg_slice(BgShared& S, int W, bool pivot, Form form, Side side) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int NP = (W + 3) >> 2;
+  if (!pivot) {
+    const int unit = bg_unit<NH>(warp);
+    const int j = NH == 2 ? (unit & 1) * 32 + lane : lane;
+    const int g = NH == 2 ? unit >> 1 : unit;
+    cf v[4], f[4], inv[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = f[c] = inv[c] = cf{0.f, 0.f};
+    if (warp < NH) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (tid < W && c < W) v[c] = form(tid, c);
+      if (W >= 4) bg_factor<NH, true>(S, 0, 4, 0, S.B[1], v, f, inv);
+      else bg_factor<NH, false>(S, 0, W, 0, S.B[1], v, f, inv);
+    } else if (unit >= 0 && j >= 4 && j < W) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const int i = g + kBgGroups * r;
+        if (i < W) S.B[0][i * kBgPitch + j] = form(i, j);
+      }
+    }
+    __syncthreads();
+    bg_invert<NH>(S, W, v, f, inv, side);
+    return !S.bad;
+  }
+  cf* A = S.B[(NP & 1) ^ 1];
+  cf* Bg = S.B[NP & 1];
+  for (int idx = tid; idx < W * W; idx += blockDim.x) A[idx] = form(idx / W, idx % W);
+  side();
+  __syncthreads();
+  cf* rowk = reinterpret_cast<cf*>(S.F);
+  if (!cta_gj(A, rowk, rowk + 64, S.perm, S.flag, W, true)) return false;
+  __syncthreads();
+  for (int idx = tid; idx < W * W; idx += blockDim.x) Bg[(idx / W) * kBgPitch + idx % W] = A[idx];
+  __syncthreads();
+  return true;
 }
 
 }  // namespace

@@ -32,8 +32,8 @@ __device__ __forceinline__ cf wide_diag(const TaskDesc& d, const double* onsite,
 // one for forming its matrix, which happens while the previous slice's g is stored: the column
 // warps form columns >= 4 and the panel warp, from its own registers, the first panel, which
 // it then eliminates.  The next slice's diagonal is fetched by the two warps without columns.
-// Measured (GB300): W=64 x L=100, 8 energies 6.81 -> 2.58 ms, W=64 x L=1000, 4 energies
-// 66.7 -> 25.7 ms (26 us a slice), against one pivot at a time with 1024 threads.
+// Measured (GB300) against one pivot at a time with 1024 threads: W=64 x L=100, 8 energies 6.81 ->
+// 2.45 ms, W=64 x L=1000 66.7 -> 24.4 ms (24 us a slice); W=32 x L=100, 32 energies 1.83 -> 0.73 ms.
 template <int NH>
 __global__ void __launch_bounds__(kBgThreads<NH>) rgf_sweep_wide_kernel(
     const TaskDesc* __restrict__ tasks, int n_tasks, const double* __restrict__ wire, cf* gL,
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kBgThreads<NH>) rgf_sweep_wide_kernel(
       hs[a * 64 + b] = 0.f - (float)h[idx];
     }
   // the slices' diagonals, one slice ahead, by the warps without columns
-  const int dw = NH == 2 ? (warp == 12 ? 0 : warp == 16 ? 1 : -1) : (warp == 4 ? 0 : -1);
+  const int dw = bg_side<NH>(warp);
   auto fetch_diag = [&](int s) {
     if (dw < 0 || s >= L - 1) return;
     const int a = 32 * dw + lane, k = dir == 0 ? s : L - 1 - s;
@@ -88,23 +88,17 @@ __global__ void __launch_bounds__(kBgThreads<NH>) rgf_sweep_wide_kernel(
     bad |= !finite_c(v);
     return cf{__fmaf_rn(-tt, v.x, e.x), __fmaf_rn(-tt, v.y, e.y)};
   };
-  cf v[NH][4], f[NH][4], inv[4];
+  cf v[4], f[4], inv[4];
 #pragma unroll
-  for (int m = 0; m < NH; ++m)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) v[m][c] = f[m][c] = cf{0.f, 0.f};
+  for (int c = 0; c < 4; ++c) v[c] = f[c] = inv[c] = cf{0.f, 0.f};
   for (int s = 0; s < L - 1; ++s) {
     cf* gdst = s > 0 ? out + (uint64_t)(dir == 0 ? s - 1 : L - s) * WW : nullptr;
     if (!(S.undephased[s & 1][0] || (NH == 2 && S.undephased[s & 1][1]))) {
-      if (warp == 0) {
+      if (warp < NH) {
 #pragma unroll
-        for (int m = 0; m < NH; ++m) {
-          const int i = lane + 32 * m;
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-            if (i < W) v[m][c] = form(s, i, c, gdst);
-        }
-        bg_factor<NH>(S, 0, 4, 0, S.B[1], v, f, inv);
+        for (int c = 0; c < 4; ++c)
+          if (tid < W) v[c] = form(s, tid, c, gdst);
+        bg_factor<NH, true>(S, 0, 4, 0, S.B[1], v, f, inv);
       } else if (unit >= 0 && j >= 4 && j < W) {
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
@@ -162,7 +156,7 @@ __device__ __forceinline__ int wide_task(const TaskDesc* tasks, int n_tasks, uin
 
 // Diagonal blocks: one CTA per (task, y) as diag_cta_kernel (k_rgf.cu), same outputs.
 template <int NH>
-__global__ void __launch_bounds__(kBgThreads<NH>, NH == 1 ? 2 : 1) diag_wide_kernel(
+__global__ void __launch_bounds__(kBgThreads<NH>, 1) diag_wide_kernel(
     const TaskDesc* __restrict__ tasks, int n_tasks, uint32_t n_jobs,
     const double* __restrict__ wire, const double* __restrict__ phig,
     const double* __restrict__ gam, const cf* __restrict__ gL, const cf* __restrict__ gR,
@@ -178,7 +172,7 @@ __global__ void __launch_bounds__(kBgThreads<NH>, NH == 1 ? 2 : 1) diag_wide_ker
   BgShared& S = *reinterpret_cast<BgShared*>(smem_raw);
   const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5, lane = tid & 31;
   const int unit = bg_unit<NH>(warp);
-  const int jc = NH == 2 ? (unit & 1) * 32 + lane : lane;
+  const int j = NH == 2 ? (unit & 1) * 32 + lane : lane;
   const int g = NH == 2 ? unit >> 1 : unit;
   const int NP = (W + 3) >> 2;
   const int y = (int)(job - d.col_base);
@@ -209,23 +203,19 @@ __global__ void __launch_bounds__(kBgThreads<NH>, NH == 1 ? 2 : 1) diag_wide_ker
   cf* G = S.B[NP & 1];
   cf* T = S.B[(NP & 1) ^ 1];                              // free once the inverse is in G
   if (deph) {
-    cf v[NH][4], f[NH][4], inv[4];
+    cf v[4], f[4], inv[4];
 #pragma unroll
-    for (int m = 0; m < NH; ++m)
+    for (int c = 0; c < 4; ++c) v[c] = f[c] = inv[c] = cf{0.f, 0.f};
+    if (warp < NH) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) v[m][c] = f[m][c] = cf{0.f, 0.f};
-    if (warp == 0) {
-#pragma unroll
-      for (int m = 0; m < NH; ++m)
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if (lane + 32 * m < W) v[m][c] = form(lane + 32 * m, c);
-      bg_factor<NH>(S, 0, 4, 0, S.B[1], v, f, inv);
-    } else if (unit >= 0 && jc >= 4 && jc < W) {
+      for (int c = 0; c < 4; ++c)
+        if (tid < W) v[c] = form(tid, c);
+      bg_factor<NH, true>(S, 0, 4, 0, S.B[1], v, f, inv);
+    } else if (unit >= 0 && j >= 4 && j < W) {
 #pragma unroll
       for (int r = 0; r < 8; ++r) {
         const int i = g + kBgGroups * r;
-        if (i < W) S.B[0][i * kBgPitch + jc] = form(i, jc);
+        if (i < W) S.B[0][i * kBgPitch + j] = form(i, j);
       }
     }
     __syncthreads();
