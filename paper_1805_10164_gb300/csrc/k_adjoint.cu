@@ -36,6 +36,7 @@
 #include <math.h>
 
 #include "gj.cuh"
+#include "gj_blocked.cuh"
 #include "negf_internal.cuh"
 
 namespace negf {
@@ -170,6 +171,98 @@ __global__ void __launch_bounds__(kAdjThreads) adj_expand_kernel(
     if (!cta_gj(A, rowk, fcol, perm, flag, W, !deph)) {
       if (threadIdx.x == 0) atomicOr(err, ERR_SINGULAR);
       return;
+    }
+  }
+}
+
+// ---- complex64 sweeps: the same blocks by the panel inversion (gj_blocked.cuh) ---------------
+// One pivot at a time the sweep of the W=16 x L=100, 16-energy gradient took 0.90 ms (9 us a
+// slice), by panels 0.51.  The recompute keeps the smaller CTAs of adj_expand_kernel: its many
+// segments run side by side, and one panel CTA per SM measured 0.137 ms against 0.094.  The next
+// slice's diagonal is fetched one slice ahead by the warps without columns.
+template <int NH>
+struct AdjSlices {
+  BgShared& S;
+  const TaskDesc& d;
+  const double *onsite, *eta, *h, *phi;
+  const cd* sg;
+  const cf* Bg;                                     // the block before
+  __device__ AdjSlices(BgShared& s, const TaskDesc& t, const double* wire, const double* phig,
+                       const cd* sig)
+      : S(s), d(t), onsite(wire + t.onsite_off), eta(onsite + t.n), h(slice_block(t, onsite)),
+        phi(phig + t.phi_off), sg(sig + t.lead_off), Bg(s.B[((t.W + 3) >> 2) & 1]) {}
+  // diagonal and dephasing of slice k into buffer b
+  __device__ void fetch(int k, int b) const {
+    const int dw = bg_side<NH>(threadIdx.x >> 5);
+    if (dw < 0) return;
+    const int W = d.W, a = 32 * dw + (threadIdx.x & 31);
+    const bool und = a < W && !(eta[k * W + a] > 0.0);
+    if (a < W) {
+      const double e = d.E - onsite[k * W + a];
+      S.diag[b][a] = cf{(float)(h ? e - h[a * W + a] : e), (float)(0.5 * eta[k * W + a])};
+    }
+    const bool any = __any_sync(0xffffffffu, und);
+    if ((threadIdx.x & 31) == 0) S.undephased[b][dw] = any;
+  }
+  __device__ bool pivots(int b) const {
+    return S.undephased[b][0] || (NH == 2 && S.undephased[b][1]);
+  }
+  // entry of the slice matrix (form_slice): leads = how many leads end on the slice
+  __device__ cf entry(int i, int c, int b, int leads, bool with_prev) const {
+    const int W = d.W;
+    cf v;
+    if (i == c) v = S.diag[b][i];
+    else if (h) v = cf{0.f - (float)h[i * W + c], 0.f};
+    else v = cf{i - c == 1 || c - i == 1 ? (float)d.t : 0.f, 0.f};
+    if (leads) {
+      const cd s = lead_sigma(i, c, W, phi, sg);
+      v = cf{__fsub_rn(v.x, (float)(leads * s.x)), __fsub_rn(v.y, (float)(leads * s.y))};
+    }
+    if (with_prev) {
+      const float tt = (float)(d.t * d.t);
+      const cf p = Bg[i * kBgPitch + c];
+      v = cf{__fmaf_rn(-tt, p.x, v.x), __fmaf_rn(-tt, p.y, v.y)};
+    }
+    return v;
+  }
+};
+
+template <int NH>
+__global__ void __launch_bounds__(kBgThreads<NH>) adj_sweep32_kernel(
+    const TaskDesc* __restrict__ tasks, int n_tasks, const double* __restrict__ wire,
+    const double* __restrict__ phig, const cd* __restrict__ sig,
+    const uint64_t* __restrict__ ck_off, int s, cf* __restrict__ ck, int32_t* __restrict__ err) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  BgShared& S = *reinterpret_cast<BgShared*>(smem_raw);
+  const int job = blockIdx.x;
+  if (job >= 2 * n_tasks) return;
+  const int task = job >> 1, dir = job & 1;
+  const TaskDesc d = tasks[task];
+  const int W = d.W, L = d.L, WW = W * W;
+  if (NH == 1 ? W > 32 : W <= 32) return;           // the other instance's
+  const AdjSlices<NH> sl(S, d, wire, phig, sig);
+  const int nck = (L + s - 1) / s;
+  cf* out = ck + ck_off[task] + (uint64_t)dir * nck * WW;
+  const int steps = dir == 0 ? L : L - 1;
+  auto slice = [&](int i) { return dir == 0 ? i : L - 1 - i; };
+  if (steps > 0) sl.fetch(slice(0), 0);
+  if (threadIdx.x == 0) S.bad = 0;
+  __syncthreads();
+  for (int i = 0; i < steps; ++i) {
+    const int k = slice(i), b = i & 1;
+    const int leads = (dir == 0 && k == 0 ? 1 : 0) + (k == L - 1 ? 1 : 0);
+    const bool ok = bg_slice<NH>(
+        S, W, sl.pivots(b), [&](int r, int c) { return sl.entry(r, c, b, leads, i > 0); },
+        [&] { if (i + 1 < steps) sl.fetch(slice(i + 1), b ^ 1); });
+    if (!ok) {
+      if (threadIdx.x == 0) atomicOr(err, ERR_SINGULAR);
+      return;
+    }
+    if (i % s == 0) {
+      cf* dst = out + (uint64_t)(i / s) * WW;
+      for (int idx = threadIdx.x; idx < WW; idx += blockDim.x)
+        dst[idx] = sl.Bg[(idx / W) * kBgPitch + idx % W];
+      __syncthreads();
     }
   }
 }
@@ -714,6 +807,12 @@ __global__ void __launch_bounds__(kAdjThreads, RT >= 2 ? 1 : (sizeof(C) == 8 ? 3
   }
 }
 
+template <typename K>
+cudaError_t bg_smem(K kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)sizeof(BgShared));
+}
+
 template <typename C>
 size_t gj_smem(int W) {
   return sizeof(C) * (size_t)(W * W + 2 * W) + sizeof(int) * (size_t)(W + 2);
@@ -814,12 +913,19 @@ cudaError_t launch_adjoint_sweep(const TaskDesc* d_tasks, int n_tasks, int max_W
     adj_sweep_kernel<cd><<<2 * n_tasks, kAdjThreads, smem, s>>>(
         d_tasks, n_tasks, d_wire, d_phi, d_sig, d_ck_off, stride, static_cast<cd*>(d_ck), d_err);
   } else {
-    const size_t smem = gj_smem<cf>(max_W);
-    cudaError_t e = cudaFuncSetAttribute(adj_sweep_kernel<cf>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // widths up to 32 and above by kernels of their own; each skips the other's tasks
+    cudaError_t e = bg_smem(adj_sweep32_kernel<1>);
+    if (e == cudaSuccess) e = bg_smem(adj_sweep32_kernel<2>);
     if (e != cudaSuccess) return e;
-    adj_sweep_kernel<cf><<<2 * n_tasks, kAdjThreads, smem, s>>>(
+    adj_sweep32_kernel<1><<<2 * n_tasks, kBgThreads<1>, sizeof(BgShared), s>>>(
         d_tasks, n_tasks, d_wire, d_phi, d_sig, d_ck_off, stride, static_cast<cf*>(d_ck), d_err);
+    if (max_W > 32) {
+      e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+      adj_sweep32_kernel<2><<<2 * n_tasks, kBgThreads<2>, sizeof(BgShared), s>>>(
+          d_tasks, n_tasks, d_wire, d_phi, d_sig, d_ck_off, stride, static_cast<cf*>(d_ck),
+          d_err);
+    }
   }
   return cudaGetLastError();
 }
