@@ -627,10 +627,10 @@ __global__ void __launch_bounds__(kNThreads, 4) chain_cta_narrow_kernel(
 }  // namespace
 
 cudaError_t launch_chain_cta(const TaskDesc* d_tasks, const TcJob* d_jobs, uint32_t n_wide,
-                             uint32_t n_narrow, const float* d_eta32, const float* d_phi32,
-                             const double* d_gam, const void* d_gL, const void* d_gR,
-                             const void* d_start, void* d_weights, uint64_t* d_tab,
-                             int32_t* d_err, cudaStream_t s) {
+                             uint32_t n_narrow, uint32_t n_mid, const float* d_eta32,
+                             const float* d_phi32, const double* d_gam, const void* d_gL,
+                             const void* d_gR, const void* d_start, void* d_weights,
+                             uint64_t* d_tab, int32_t* d_err, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   if (n_wide) {
     e = cudaFuncSetAttribute(chain_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -652,8 +652,10 @@ cudaError_t launch_chain_cta(const TaskDesc* d_tasks, const TcJob* d_jobs, uint3
         static_cast<const cf*>(d_gR), static_cast<const cf*>(d_start),
         static_cast<float*>(d_weights));
     e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
   }
-  return e;
+  return launch_chain_mid(d_tasks, d_jobs + n_wide + n_narrow, n_mid, d_eta32, d_phi32, d_gam,
+                          d_gL, d_gR, d_start, d_weights, s);
 }
 
 }  // namespace negf

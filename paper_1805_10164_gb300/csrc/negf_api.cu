@@ -495,7 +495,7 @@ negf_status make_plan(negf_ctx ctx, const negf_wire* wires, int n_wires, bool de
       d.gamma_lead = wr.gamma_lead;
       d.layout = layout;
       d.fused = tc_wire ? 1 : 0;
-      d.cta_chain = (fp32 && (wr.W == 64 || (wr.W > 16 && wr.W <= 32)) && !tc_wire) ? 1 : 0;
+      d.cta_chain = (fp32 && wr.W > 16 && !tc_wire) ? 1 : 0;
       d.slice_h = wr.slice_h ? 1 : 0;
       // W = 64 two-level tables on the CTA chain, no weights kept: the chain writes level 2
       d.l2_fused = (fuse_l2 && d.cta_chain && wr.W == 64 && layout == NEGF_LAYOUT_TWO_LEVEL) ? 1 : 0;
@@ -578,18 +578,21 @@ struct Wave {
   std::vector<TaskDesc> adesc;       // alias_descs(desc)
   std::vector<TcJob> tcjobs;         // tensor-core chain jobs (task = index into desc), then
   size_t n_tc = 0;                   // the CTA-chain jobs: tcjobs[n_tc ..], those of W = 64
-  size_t n_cta_wide = 0;             // tasks first
+  size_t n_cta_wide = 0;             // tasks first, those of 32 < W < 64 last
+  size_t n_cta_mid = 0;
   int cols_max_W = 0;                // widest task of the warp-per-column chains
   int two_max_W = 0;                 // widest task with two-level tables
   bool any_two_split = false;        // two-level tasks whose level 2 comes from stored weights
-  uint32_t cta_narrow() const { return (uint32_t)(tcjobs.size() - n_tc - n_cta_wide); }
+  uint32_t cta_narrow() const {
+    return (uint32_t)(tcjobs.size() - n_tc - n_cta_wide - n_cta_mid);
+  }
 };
 
 using negf::add_tc_jobs;
 
 Wave make_wave(const Plan& P, int t0, int t1) {
   Wave w;
-  std::vector<TcJob> cta, cta_n;
+  std::vector<TcJob> cta, cta_n, cta_m;
   w.t0 = t0;
   w.t1 = t1;
   for (int k = t0; k < t1; ++k) {
@@ -609,7 +612,7 @@ Wave make_wave(const Plan& P, int t0, int t1) {
     }
     if (d.cta_chain) {
       if (d.W == 64) negf::add_sym_jobs(cta, k - t0, d.L);
-      else add_tc_jobs(cta_n, k - t0, d.L);
+      else add_tc_jobs(d.W > 32 ? cta_m : cta_n, k - t0, d.L);
     }
     if (!d.cta_chain && !d.fused) w.cols_max_W = std::max(w.cols_max_W, d.W);
     if (d.layout == NEGF_LAYOUT_TWO_LEVEL) {
@@ -640,10 +643,13 @@ Wave make_wave(const Plan& P, int t0, int t1) {
   negf::sort_jobs_longest_first(w.tcjobs, w.desc.data());
   negf::sort_jobs_longest_first(cta, w.desc.data());
   negf::sort_jobs_longest_first(cta_n, w.desc.data());
+  negf::sort_jobs_longest_first(cta_m, w.desc.data());
   w.n_tc = w.tcjobs.size();
   w.n_cta_wide = cta.size();
+  w.n_cta_mid = cta_m.size();
   w.tcjobs.insert(w.tcjobs.end(), cta.begin(), cta.end());
   w.tcjobs.insert(w.tcjobs.end(), cta_n.begin(), cta_n.end());
+  w.tcjobs.insert(w.tcjobs.end(), cta_m.begin(), cta_m.end());
   return w;
 }
 
@@ -837,7 +843,7 @@ negf_status build_wave(negf_ctx ctx, cudaStream_t s, const Plan& P, const Wave& 
   if (e == cudaSuccess && w.tcjobs.size() > w.n_tc) {
     ProfScope ps(ctx, "chain_cta_kernel", 1, s);
     e = negf::launch_chain_cta(d_wdesc, d_tcjobs + w.n_tc, (uint32_t)w.n_cta_wide,
-                               w.cta_narrow(), q.d_eta32, reinterpret_cast<const float*>(q.d_phi + P.phi_total),
+                               w.cta_narrow(), (uint32_t)w.n_cta_mid, q.d_eta32, reinterpret_cast<const float*>(q.d_phi + P.phi_total),
                                q.d_gam, d_gL, d_gR, d_start, d_weights, d_tab, q.d_err, s);
   }
   if (e == cudaSuccess && w.n_tc) {
@@ -2441,7 +2447,7 @@ negf_status plan_enqueue(negf_plan p, bool timed, cudaStream_t s) {
       SegScope sg(p, "chain_cta_kernel", 1, s, timed);
       CUDA_TRY(ctx, negf::launch_chain_cta(
                         dd, p->d_tcjobs + p->job_off[w] + wv.n_tc, (uint32_t)wv.n_cta_wide,
-                        wv.cta_narrow(), q.d_eta32,
+                        wv.cta_narrow(), (uint32_t)wv.n_cta_mid, q.d_eta32,
                         reinterpret_cast<const float*>(q.d_phi + P.phi_total), q.d_gam, p->d_gL,
                         p->d_gR, p->d_start[slot], p->d_weights[slot], p->d_tab[slot],
                         q.d_err, s));
@@ -2546,7 +2552,7 @@ negf_status plan_autotune(negf_plan p) {
     cudaError_t e = columns(cw);
     if (e == cudaSuccess && wv.tcjobs.size() > wv.n_tc)
       e = negf::launch_chain_cta(dd, p->d_tcjobs + wv.n_tc, (uint32_t)wv.n_cta_wide,
-                                 wv.cta_narrow(), q.d_eta32,
+                                 wv.cta_narrow(), (uint32_t)wv.n_cta_mid, q.d_eta32,
                                  reinterpret_cast<const float*>(q.d_phi + P.phi_total), q.d_gam,
                                  p->d_gL, p->d_gR, p->d_start[0], p->d_weights[0],
                                  p->d_tab[0], q.d_err, s);

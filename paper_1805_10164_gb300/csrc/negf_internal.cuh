@@ -41,7 +41,7 @@ struct TaskDesc {
   uint64_t l1_off;       // two-level: level-1 entries [rows][L + 2] (level 2 is at tab_off)
   uint64_t l1w_off;      // two-level: level-1 weights [rows][L + 2] in the weights array
   uint64_t edge_off;     // fused: slice-0 and slice-(L-1) blocks [L + 2][2][W][W] complex64
-  int32_t cta_chain;     // block columns by a CTA-wide FP32 kernel (W = 64 or 16 < W <= 32)
+  int32_t cta_chain;     // block columns by a CTA-wide FP32 kernel (W > 16)
   int32_t slice_h;       // multi-orbital slice block: h [W][W] at onsite + 2n, then the
                          // eigenvalues of h [W] (written on the device) at onsite + 2n + W^2
   int32_t l2_fused;      // two-level, W = 64 CTA chain: the chain writes the level-2 blocks and
@@ -160,6 +160,12 @@ cudaError_t launch_energy_tables(const TaskDesc* d_tasks, int n_tasks, const Ene
                                  const uint32_t* d_job_base, uint32_t total_jobs, int max_nE,
                                  double sigma, const double* d_rowsum, uint64_t* d_etab,
                                  int32_t* d_err, cudaStream_t s);
+// Consecutive walkers a warp of an inelastic or thermal walk takes at a time: up to 512 (lanes
+// are refilled within a chunk), down to one per lane when the grid has more warps than that.
+inline unsigned walk_chunk(uint64_t walkers, uint64_t warps) {
+  const uint64_t per = (walkers + warps - 1) / warps;
+  return per >= 512 ? 512u : (unsigned)((per + 31) / 32 * 32);
+}
 // Inelastic walks of every task (injection at the task's energy; Step 6' rows of the walker's
 // current energy, Step 7' energy rows after every site), tallied per injection task as the
 // elastic walk's tally.
@@ -190,10 +196,14 @@ cudaError_t launch_chain_tc(const TaskDesc* d_tasks, int n_tasks, uint32_t n_col
 // d_tab, d_err: the tables and error word, for the tasks with l2_fused (W = 64 two-level),
 // whose level-2 blocks and level-1 weights the wide kernel writes itself.
 cudaError_t launch_chain_cta(const TaskDesc* d_tasks, const TcJob* d_jobs, uint32_t n_wide,
-                             uint32_t n_narrow, const float* d_eta32, const float* d_phi32,
-                             const double* d_gam, const void* d_gL, const void* d_gR,
-                             const void* d_start, void* d_weights, uint64_t* d_tab,
-                             int32_t* d_err, cudaStream_t s);
+                             uint32_t n_narrow, uint32_t n_mid, const float* d_eta32,
+                             const float* d_phi32, const double* d_gam, const void* d_gL,
+                             const void* d_gR, const void* d_start, void* d_weights,
+                             uint64_t* d_tab, int32_t* d_err, cudaStream_t s);
+cudaError_t launch_chain_mid(const TaskDesc* d_tasks, const TcJob* d_jobs, uint32_t n_jobs,
+                             const float* d_eta32, const float* d_phi32, const double* d_gam,
+                             const void* d_gL, const void* d_gR, const void* d_start,
+                             void* d_weights, cudaStream_t s);
 // Warps per CTA the alias kernel can use for rows of max_K slots (shared memory bound).
 int alias_warps_max(int max_K);
 // Two-level tasks: from the weights [rows][K] of every table row, the level-1 weights (slice

@@ -71,8 +71,9 @@ extern "C" negf_status negf_build_tables_noalloc(const negf_wire* wire, int32_t 
     if (wr.lead_model == NEGF_LEAD_STRIP && !wr.slice_h && band_edge(wr.energy[k], wr.W, wr.t))
       return NEGF_E_INVALID;
   }
-  // block columns as negf_build_tables takes them: FP32 wires of W = 64 or 16 < W <= 32 on the
-  // CTA-wide chains (jobs listed here), every other wire on the warp-per-column chains
+  // FP32 wires of W = 64 or 16 < W <= 32 on the CTA-wide chains (jobs listed here), every other
+  // wire on the warp-per-column chains, which need no job list in the fixed scratch (and give the
+  // same bits as the CTA-wide chain of 32 < W < 64)
   const bool cta = prec == NEGF_FP32 && (wr.W == 64 || (wr.W > 16 && wr.W <= 32));
 
   // ---- carve the scratch array; reject problems that do not fit
@@ -191,7 +192,7 @@ extern "C" negf_status negf_build_tables_noalloc(const negf_wire* wire, int32_t 
                                    cta ? 0 : wr.W);
   if (e == cudaSuccess && cta)
     e = negf::launch_chain_cta(d_tasks, d_jobs, wr.W == 64 ? (uint32_t)jobs.size() : 0u,
-                               wr.W == 64 ? 0u : (uint32_t)jobs.size(), d_eta32, d_phi32, d_gam,
+                               wr.W == 64 ? 0u : (uint32_t)jobs.size(), 0u, d_eta32, d_phi32, d_gam,
                                d_gL, d_gR, d_st, d_w, d_alias, d_err, s);
   if (e == cudaSuccess)
     e = negf::launch_alias_build(d_tasks, nt, (uint32_t)(nt * (rows + 2)), (int)K, prec, d_w,
