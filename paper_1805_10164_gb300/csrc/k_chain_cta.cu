@@ -421,12 +421,14 @@ __global__ void __launch_bounds__(kThreads, 1) chain_cta_kernel(
 // ---- 16 < W <= 32: the same recursion with the pair's 2W columns side by side --------------
 // One CTA of 128 threads per job (four CTAs fit an SM): X_k [W][2W] = (-t g_k) [W][W] X_{k+1}
 // in shared memory, thread (ty, tx) = (t / 16, t mod 16) owning the outputs a = ty + 8 i,
-// b' = tx + 16 j.  g_{k-1} (or g_{k+1}) comes into registers while step k multiplies, so the
-// step's only wait on global memory is hidden behind its products.
+// b' = tx + 16 j.  X is overwritten in place between two barriers a step, and the step's weights
+// are read from it directly while the next product begins; odd row pitches keep rows and columns
+// free of bank conflicts.  g_{k-1} (or g_{k+1}) comes into registers while step k multiplies.
+// (With X in two buffers and the weights turned through a staging buffer, four barriers a step:
+// W=32 x L=100, 32 energies 2.42 ms, 2.08 now; W=24 1.25, 1.04.)
 constexpr int kNThreads = 128;
 constexpr int kNMax = 32;
-constexpr size_t kNSmem = sizeof(cf) * (kNMax * kNMax + 2 * kNMax * 2 * kNMax) +
-                          sizeof(float) * 2 * kNMax * (kNMax + 1);
+constexpr size_t kNSmem = sizeof(cf) * (kNMax * (2 * kNMax + 1) + kNMax * (kNMax + 1));
 
 template <int W>
 __device__ __forceinline__ void chain_cta_narrow_body(const TaskDesc& d, const TcJob& job,
@@ -439,14 +441,12 @@ __device__ __forceinline__ void chain_cta_narrow_body(const TaskDesc& d, const T
                                                       float* __restrict__ weights,
                                                       unsigned char* smem) {
   constexpr int N = 2 * W;                    // the pair's columns
+  constexpr int XP = N + 1, GP = W | 1;       // row pitches
   constexpr int RI = (W + 7) / 8;             // output rows a = ty + 8 i
   constexpr int CJ = (N + 15) / 16;           // output columns b' = tx + 16 j
-  constexpr int WP = W + 1;                   // padded row of the weight staging
   constexpr int kPre = (W * W + kNThreads - 1) / kNThreads;
-  cf* Gs = reinterpret_cast<cf*>(smem);                    // [a][c] (-t g_k); Phi at the edges
-  cf* Xa = Gs + kNMax * kNMax;                             // [c][b'] ping
-  cf* Xb = Xa + 2 * kNMax * kNMax;                         // [c][b'] pong
-  float* Wt = reinterpret_cast<float*>(Xb + 2 * kNMax * kNMax);   // [b'][a] weights staging
+  cf* X = reinterpret_cast<cf*>(smem);                     // [c][b']
+  cf* Gs = X + W * XP;                                     // [a][c] (-t g_k); Phi at the edges
 
   const int tid = threadIdx.x;
   const int L = d.L, n = d.n, K = d.K;
@@ -460,60 +460,58 @@ __device__ __forceinline__ void chain_cta_narrow_body(const TaskDesc& d, const T
   auto row_of = [&](int y, int b) -> uint64_t {
     return y < L ? (uint64_t)y * W + b : (uint64_t)n + (uint64_t)(y - L) * W + b;
   };
-  auto load_start = [&](cf* X, int col) {
+  auto load_start = [&](int col) {
     const cf* st = start + d.start_off + (uint64_t)ys[col] * W * W;
-    for (int i = tid; i < W * W; i += kNThreads) {
-      const int c = i / W, b = i - c * W;
-      X[c * N + col * W + b] = st[i];
+    for (int i = tid; i < W * W; i += kNThreads) X[(i / W) * XP + col * W + i % W] = st[i];
+  };
+  // weights of slice k for the columns in `mask`, from X
+  auto emit = [&](int k, unsigned mask) {
+#pragma unroll
+    for (int q = 0; q < (N * W + kNThreads - 1) / kNThreads; ++q) {
+      const int i = tid + kNThreads * q;
+      const int r = i / W, a = i - r * W;                  // a consecutive: coalesced rows
+      const int col = r >= W;
+      if (i < N * W && (mask & (1u << col))) {
+        const cf v = X[a * XP + r];
+        wt[row_of(ys[col], r - col * W) * K + (uint64_t)k * W + a] =
+            __fmul_rn(__ldg(eta + k * W + a), __fmaf_rn(v.x, v.x, __fmul_rn(v.y, v.y)));
+      }
     }
   };
-  auto emit = [&](const cf* X, int k, unsigned mask) {
-    for (int i = tid; i < N * W; i += kNThreads) {
-      const int a = i / N, r = i - a * N;                  // r consecutive across threads
-      const cf v = X[a * N + r];
-      Wt[r * WP + a] = eta[k * W + a] * (v.x * v.x + v.y * v.y);
+  // lead weights sum_nu Gamma_nu |(Phi^T X)_nu b'|^2 at a boundary slice: Phi (FP32) takes the g
+  // buffer, which no product needs any more (or yet); two threads per column, each half of the
+  // modes, then the sum of the halves.  Synchronised before and after.
+  auto lead_weights = [&](int k, unsigned mask) {
+    float* phis = reinterpret_cast<float*>(Gs);
+    float* gams = phis + W * W;
+    float* parts = gams + W;
+    for (int i = tid; i < W * W; i += kNThreads) phis[i] = phi32[d.phi_off + i];
+    for (int i = tid; i < W; i += kNThreads) gams[i] = (float)gam[d.lead_off + i];
+    __syncthreads();
+    const int r = tid % 64, h = tid / 64;
+    if (r < N) {
+      float part = 0.f;
+      for (int nu = h * (W / 2); nu < (h ? W : W / 2); ++nu) {
+        float zr = 0.f, zi = 0.f;
+#pragma unroll 8
+        for (int a = 0; a < W; ++a) {
+          const float p = phis[a * W + nu];
+          const cf v = X[a * XP + r];
+          zr = __fmaf_rn(p, v.x, zr);
+          zi = __fmaf_rn(p, v.y, zi);
+        }
+        part = __fmaf_rn(gams[nu], __fmaf_rn(zr, zr, __fmul_rn(zi, zi)), part);
+      }
+      parts[h * N + r] = part;
     }
     __syncthreads();
-    for (int i = tid; i < N * W; i += kNThreads) {
-      const int r = i / W, a = i - r * W;                  // a consecutive: coalesced rows
+    if (h == 0 && r < N) {
       const int col = r / W;
-      if (mask & (1u << col))
-        wt[row_of(ys[col], r - col * W) * K + (uint64_t)k * W + a] = Wt[r * WP + a];
-    }
-    if (k == 0 || k == L - 1) {
-      // lead weights sum_nu Gamma_nu |(Phi^T X)_nu b'|^2: Phi (FP32) staged in Gs, free outside
-      // the product; two threads per column, each half of the modes
-      float* phis = reinterpret_cast<float*>(Gs);
-      float* gams = phis + W * W;
-      __syncthreads();
-      for (int i = tid; i < W * W; i += kNThreads) phis[i] = phi32[d.phi_off + i];
-      for (int i = tid; i < W; i += kNThreads) gams[i] = (float)gam[d.lead_off + i];
-      __syncthreads();
-      const int r = tid % 64, h = tid / 64;
-      if (r < N) {
-        float part = 0.f;
-        for (int nu = h * (W / 2); nu < (h ? W : W / 2); ++nu) {
-          float zr = 0.f, zi = 0.f;
-#pragma unroll 8
-          for (int a = 0; a < W; ++a) {
-            const float p = phis[a * W + nu];
-            const cf v = X[a * N + r];
-            zr += p * v.x;
-            zi += p * v.y;
-          }
-          part += gams[nu] * (zr * zr + zi * zi);
-        }
-        Wt[r * WP + h] = part;                             // staging is free again
-      }
-      __syncthreads();
-      if (h == 0 && r < N) {
-        const int col = r / W;
-        if (mask & (1u << col)) {
-          const float lw = Wt[r * WP] + Wt[r * WP + 1];
-          const uint64_t base = row_of(ys[col], r - col * W) * K + n;
-          if (k == 0) wt[base] = lw;
-          if (k == L - 1) wt[base + 1] = lw;
-        }
+      if (mask & (1u << col)) {
+        const float lw = parts[r] + parts[N + r];
+        const uint64_t base = row_of(ys[col], r - col * W) * K + n;
+        if (k == 0) wt[base] = lw;
+        if (k == L - 1) wt[base + 1] = lw;
       }
     }
     __syncthreads();
@@ -525,15 +523,19 @@ __device__ __forceinline__ void chain_cta_narrow_body(const TaskDesc& d, const T
   if (dir == 0) {
     for (int col = 0; col < 2; ++col) {
       if (!(have & (1u << col))) continue;
-      load_start(Xa, col);
+      const int m0 = m0_of(ys[col]);
+      load_start(col);
       __syncthreads();
-      emit(Xa, m0_of(ys[col]), 1u << col);
+      emit(m0, 1u << col);
+      if (m0 == 0 || m0 == L - 1) lead_weights(m0, 1u << col);
     }
+    __syncthreads();
   }
   const int m0a = m0_of(job.y0), m0b = job.y1 >= 0 ? m0_of(job.y1) : m0a;
   const int k_first = dir == 0 ? max(m0a, m0b) - 1 : min(m0a, m0b) + 1;
   const int k_end = dir == 0 ? -1 : L;
   const int kstep = dir == 0 ? -1 : 1;
+  if (k_first == k_end) return;
   cf gp[kPre];
   auto fetch = [&](int k) {
     const cf* gk = gsrc + (uint64_t)k * W * W;
@@ -543,39 +545,49 @@ __device__ __forceinline__ void chain_cta_narrow_body(const TaskDesc& d, const T
       if (i < W * W) gp[r] = gk[i];
     }
   };
-  if (k_first != k_end) fetch(k_first);
-  cf* Xc = Xa;
-  cf* Xn = Xb;
+  auto put = [&]() {
+#pragma unroll
+    for (int r = 0; r < kPre; ++r) {
+      const int i = tid + kNThreads * r;
+      if (i < W * W) Gs[(i / W) * GP + i % W] = cf{mt * gp[r].x, mt * gp[r].y};
+    }
+  };
+  fetch(k_first);
+  put();
   const int ty = tid / 16, tx = tid % 16;
+  // operand rows and columns; those beyond the block read its last ones and are not stored
+  int ra[RI], cb[CJ];
+#pragma unroll
+  for (int i = 0; i < RI; ++i) ra[i] = (RI * 8 == W ? ty + 8 * i : min(ty + 8 * i, W - 1)) * GP;
+#pragma unroll
+  for (int j = 0; j < CJ; ++j) cb[j] = CJ * 16 == N ? tx + 16 * j : min(tx + 16 * j, N - 1);
   for (int k = k_first; k != k_end; k += kstep) {
-    unsigned active = 0;
+    unsigned active = 0, join = 0;
     for (int col = 0; col < 2; ++col) {
       if (!(have & (1u << col))) continue;
       const int m0 = m0_of(ys[col]);
       if (dir == 0 ? k < m0 : k > m0) active |= 1u << col;
-      if (dir == 0 ? k == m0 - 1 : k == m0 + 1) load_start(Xc, col);
+      if (dir == 0 ? k == m0 - 1 : k == m0 + 1) join |= 1u << col;
     }
-#pragma unroll
-    for (int r = 0; r < kPre; ++r) {
-      const int i = tid + kNThreads * r;
-      if (i < W * W) Gs[i] = cf{mt * gp[r].x, mt * gp[r].y};
+    if (join) {
+      if (join & 1u) load_start(0);
+      if (join & 2u) load_start(1);
+      __syncthreads();                                     // (also the first g block)
     }
-    __syncthreads();
-    if (k + kstep != k_end) fetch(k + kstep);
+    const bool more = k + kstep != k_end;
+    if (more) fetch(k + kstep);
     float accr[RI][CJ], acci[RI][CJ];
 #pragma unroll
     for (int i = 0; i < RI; ++i)
 #pragma unroll
       for (int j = 0; j < CJ; ++j) accr[i][j] = acci[i][j] = 0.f;
-    // rows a >= W and columns b' >= N read in-bounds shared memory (a < 32, c N + b' < 64 W)
-    // and are never stored
 #pragma unroll 4
     for (int c = 0; c < W; ++c) {
       cf g[RI], x[CJ];
 #pragma unroll
-      for (int i = 0; i < RI; ++i) g[i] = Gs[(ty + 8 * i) * W + c];
+      for (int i = 0; i < RI; ++i) g[i] = Gs[ra[i] + c];
 #pragma unroll
-      for (int j = 0; j < CJ; ++j) x[j] = Xc[c * N + tx + 16 * j];
+      for (int j = 0; j < CJ; ++j) x[j] = X[c * XP + cb[j]];
 #pragma unroll
       for (int i = 0; i < RI; ++i)
 #pragma unroll
@@ -586,19 +598,19 @@ __device__ __forceinline__ void chain_cta_narrow_body(const TaskDesc& d, const T
           acci[i][j] = fmaf(g[i].y, x[j].x, acci[i][j]);
         }
     }
+    __syncthreads();                                       // X and g have been read
 #pragma unroll
     for (int i = 0; i < RI; ++i)
 #pragma unroll
       for (int j = 0; j < CJ; ++j) {
         const int a = ty + 8 * i, b = tx + 16 * j;
         if ((RI * 8 == W || a < W) && (CJ * 16 == N || b < N))
-          Xn[a * N + b] = cf{accr[i][j], acci[i][j]};
+          X[a * XP + b] = cf{accr[i][j], acci[i][j]};
       }
+    if (more) put();
     __syncthreads();
-    if (active) emit(Xn, k, active);
-    cf* tmp = Xc;
-    Xc = Xn;
-    Xn = tmp;
+    emit(k, active);
+    if (k == 0 || k == L - 1) lead_weights(k, active);     // the last step of its direction
   }
 }
 
