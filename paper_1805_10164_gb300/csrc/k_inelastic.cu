@@ -26,7 +26,6 @@ constexpr int kThreads = 256;
 constexpr int kFields = NEGF_TALLY_FIELDS;   // done, absorbed L, absorbed R, truncated, steps
 constexpr int kWindow = 1024;                // injection tasks per launch (40 KB shared tally)
 
-constexpr unsigned kChunk = 512;             // consecutive walkers a warp takes at a time
 constexpr unsigned kFlushAt = 1u << 26;      // flush a lane's counters before they can overflow
 
 // 64-bit counters in shared memory as (lo, hi) words: each addition carries its own overflow
@@ -48,7 +47,8 @@ __global__ void __launch_bounds__(kThreads) inelastic_walk_kernel(
     const EnergyDesc* __restrict__ edesc, const uint64_t* __restrict__ tab,
     const uint64_t* __restrict__ mode_tab, const double* __restrict__ cvals,
     const uint64_t* __restrict__ etab, int start_lead, PhiloxKey key, uint64_t walkers_per_task,
-    uint64_t id_offset, uint32_t max_steps, unsigned long long* __restrict__ tally) {
+    uint64_t id_offset, uint32_t max_steps, unsigned long long* __restrict__ tally,
+    unsigned chunk_size) {
   extern __shared__ unsigned s_tally[];                        // [task][field][lo, hi]
   for (int i = threadIdx.x; i < n_tasks * kFields * 2; i += blockDim.x) s_tally[i] = 0u;
   __syncthreads();
@@ -57,9 +57,9 @@ __global__ void __launch_bounds__(kThreads) inelastic_walk_kernel(
   const unsigned lt_mask = (1u << lane) - 1u;
   const unsigned long long total = (unsigned long long)n_tasks * walkers_per_task;
   const unsigned long long stride =
-      (unsigned long long)gridDim.x * (kThreads / 32) * kChunk;
+      (unsigned long long)gridDim.x * (kThreads / 32) * chunk_size;
   unsigned long long chunk =
-      ((unsigned long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * kChunk;
+      ((unsigned long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * chunk_size;
   unsigned taken = 0;                        // walkers of the chunk handed out
   // the lane's task (counts a not yet in shared memory) and what its walks need of it
   int tl = -1;
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kThreads) inelastic_walk_kernel(
     if (idle) {
       if (chunk < total) {
         const unsigned size =
-            total - chunk < (unsigned long long)kChunk ? (unsigned)(total - chunk) : kChunk;
+            total - chunk < chunk_size ? (unsigned)(total - chunk) : chunk_size;
         const unsigned mine = taken + __popc(idle & lt_mask);
         taken += __popc(idle);
         if (!has && mine < size) {
@@ -192,13 +192,13 @@ cudaError_t launch_inelastic_walk(const TaskDesc* d_tasks, int n_tasks, const En
     if (per_sm < 1) per_sm = 1;
     const unsigned long long total = (unsigned long long)nt * walkers_per_task;
     unsigned long long blocks = (unsigned long long)sm_count * per_sm;
-    // few walkers: a warp takes 32 at a time at least
     const unsigned long long need = (total + kThreads - 1) / kThreads;
     if (blocks > need) blocks = need;
     inelastic_walk_kernel<<<(unsigned)blocks, kThreads, smem, s>>>(
         d_tasks, w0, nt, d_edesc, d_tab, d_mode_tab, d_c, d_etab, start_lead, key,
         walkers_per_task, id_offset, max_steps,
-        reinterpret_cast<unsigned long long*>(d_tally) + (size_t)w0 * kFields);
+        reinterpret_cast<unsigned long long*>(d_tally) + (size_t)w0 * kFields,
+        walk_chunk(total, blocks * (kThreads / 32)));
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
