@@ -8,7 +8,10 @@
 // Schur decomposition, t = sign(theta) / (|theta| + sqrt(theta^2 + 1)),
 // theta = (a_qq - a_pp) / (2 a_pq)), the W (W - 1) / 2 index pairs of a sweep visited in W - 1
 // rounds of disjoint pairs (round-robin order), so that one round's rotations commute and are
-// applied together: rows, then columns, then the accumulated eigenvectors.  Sweeps stop when
+// applied together: rows, then columns, then the accumulated eigenvectors.  The FP64 pipe bounds
+// a round (two lanes a cycle per SM), so pairs whose entry is already zero are left out of it: an
+// sp3-like block couples s with py only and leaves px and pz to themselves, which leaves about
+// a third of the pairs (W=40: 1.55 -> 0.95 ms).  Sweeps stop when
 // the off-diagonal sum of squares falls below 1e-30 of the matrix's; the eigenpairs are written
 // in ascending order of eigenvalue (phi [a][m] in FP64 and FP32, eps after h in the wire data).
 #include <cuda_runtime.h>
@@ -36,6 +39,7 @@ __global__ void __launch_bounds__(kJacobiThreads) slice_modes_kernel(
   double* red = cs + 2 * np;                          // 2 * blockDim partial sums
   int* pq = reinterpret_cast<int*>(red + 2 * blockDim.x);   // (p, q) per pair
   int* perm = pq + 2 * np;
+  __shared__ int n_rot;                               // rotations of the round
   const double* h = wire + d.onsite_off + 2 * (uint64_t)d.n;
   double* eps = wire + d.onsite_off + 2 * (uint64_t)d.n + WW;
   for (int i = tid; i < WW; i += blockDim.x) {
@@ -69,39 +73,37 @@ __global__ void __launch_bounds__(kJacobiThreads) slice_modes_kernel(
       break;
     }
     for (int r = 0; r < Wp - 1; ++r) {
-      if (tid < np) {
-        int p, q;
+      if (tid < 32) {                                 // np <= 32 pairs: one warp
+        int p = 0, q = W;
         if (tid == 0) {
           p = r;
           q = Wp - 1;
-        } else {
+        } else if (tid < np) {
           p = (r + tid) % (Wp - 1);
           q = (r - tid + Wp - 1) % (Wp - 1);
         }
         if (p > q) { const int x = p; p = q; q = x; }
-        double c = 1.0, s = 0.0;
-        if (q < W) {
-          const double apq = A[p * W + q];
-          if (apq != 0.0) {
-            const double theta = (A[q * W + q] - A[p * W + p]) / (2.0 * apq);
-            const double t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-            c = 1.0 / sqrt(t * t + 1.0);
-            s = t * c;
-          }
-        } else {
-          p = q = -1;                                 // the padding index of an odd W
+        // (q == W: the padding index of an odd W, or no pair)
+        const double apq = q < W ? A[p * W + q] : 0.0;
+        const unsigned rot = __ballot_sync(0xffffffffu, apq != 0.0);
+        if (apq != 0.0) {
+          const double theta = (A[q * W + q] - A[p * W + p]) / (2.0 * apq);
+          const double t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
+          const double c = 1.0 / sqrt(t * t + 1.0);
+          const int at = __popc(rot & ((1u << tid) - 1u));
+          pq[2 * at] = p;
+          pq[2 * at + 1] = q;
+          cs[2 * at] = c;
+          cs[2 * at + 1] = t * c;
         }
-        pq[2 * tid] = p;
-        pq[2 * tid + 1] = q;
-        cs[2 * tid] = c;
-        cs[2 * tid + 1] = s;
+        if (tid == 0) n_rot = __popc(rot);
       }
       __syncthreads();
       // rows p, q of every pair: A <- J^T A
-      for (int idx = tid; idx < np * W; idx += blockDim.x) {
+      const int work = n_rot * W;
+      for (int idx = tid; idx < work; idx += blockDim.x) {
         const int k = idx / W, j = idx - k * W;
         const int p = pq[2 * k], q = pq[2 * k + 1];
-        if (p < 0) continue;
         const double c = cs[2 * k], s = cs[2 * k + 1];
         const double ap = A[p * W + j], aq = A[q * W + j];
         A[p * W + j] = c * ap - s * aq;
@@ -109,10 +111,9 @@ __global__ void __launch_bounds__(kJacobiThreads) slice_modes_kernel(
       }
       __syncthreads();
       // columns p, q: A <- A J, V <- V J
-      for (int idx = tid; idx < np * W; idx += blockDim.x) {
+      for (int idx = tid; idx < work; idx += blockDim.x) {
         const int k = idx / W, i = idx - k * W;
         const int p = pq[2 * k], q = pq[2 * k + 1];
-        if (p < 0) continue;
         const double c = cs[2 * k], s = cs[2 * k + 1];
         const double ap = A[i * W + p], aq = A[i * W + q];
         A[i * W + p] = c * ap - s * aq;
