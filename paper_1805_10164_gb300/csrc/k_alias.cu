@@ -47,43 +47,77 @@ __device__ __forceinline__ uint64_t pack(uint32_t thr, uint32_t alias) {
 // (W=16 x L=100, 16 energies, weights kept) 1.38 -> 0.65, of 2002 (W=40 x L=50, 16 tasks)
 // 2.03 -> 1.35, FP64 rows of 502 0.61 -> 0.54.
 //
-// Each lane owns a block of npl = ceil(K/32) consecutive items.  Per-item values live in shared
-// memory at slot (i / npl) * pitch + i % npl, with an odd pitch (npl or npl + 1) so that the 32
-// lanes walking their blocks in step touch 32 different banks.
-__host__ __device__ inline int alias_npl(int K) { return (K + 31) >> 5; }
-__host__ __device__ inline int alias_pitch(int K) { return alias_npl(K) | 1; }
-// Per-warp shared memory: s_u, s_c : u64 [32 pitch] | the row's weights (32 pitch elements of
-// `elem` bytes, or 32 alias_pitch(64) FP64 mode weights) | s_x : u16 [cap]
+// A row of more than kAliasWarpRow slots is built by four warps, shorter ones by one: a row's
+// arrays (22 bytes a slot) leave room for few rows per SM, and one warp each then leaves it
+// idle between its dependent steps; four warps share a row's arrays for seven barriers a row.
+// One warp against four, ms: 702 slots (64 energies) 0.39, 0.78; 1002 (64,128 rows) 0.91, 1.01; 1602 0.65, 0.56;
+// 1702 (32 energies) 1.98, 1.25; 2002 (16 tasks) 1.34, 0.83.  A build launches one kernel per
+// class of row lengths among its tasks, the short rows (up to kAliasShortRow) with shared memory
+// for their own length: 1280 uneven tasks 42 -> 28 ms.
+//
+// Each of the group's threads (the lanes of its NW warps) owns a block of npl consecutive items,
+// npl = ceil(K / (32 NW)).  Per-item values live in shared memory at slot
+// (i / npl) * pitch + i % npl, with an odd pitch (npl or npl + 1) so that the lanes walking their
+// blocks in step touch 32 different banks.
+constexpr int kAliasShortRow = 512, kAliasWarpRow = 1200;
+template <int NW>
+__host__ __device__ inline int alias_npl(int K) { return (K + 32 * NW - 1) / (32 * NW); }
+template <int NW>
+__host__ __device__ inline int alias_pitch(int K) { return alias_npl<NW>(K) | 1; }
+// Per-group shared memory: s_u, s_c : u64 [32 NW pitch] | the row's weights (32 NW pitch elements
+// of `elem` bytes, or those of 64 FP64 mode weights) | s_x : u16 [cap] | exchange between warps
+template <int NW>
 __host__ __device__ inline size_t alias_stage_bytes(int cap, int elem) {
-  const size_t row = (size_t)32 * alias_pitch(cap) * elem;
-  const size_t modes = (size_t)32 * alias_pitch(64) * sizeof(double);
+  const size_t row = (size_t)32 * NW * alias_pitch<NW>(cap) * elem;
+  const size_t modes = (size_t)32 * NW * alias_pitch<NW>(64) * sizeof(double);
   return ((row > modes ? row : modes) + 15) & ~(size_t)15;
 }
-__host__ __device__ inline size_t alias_warp_bytes(int cap, int elem) {
-  const size_t slots = (size_t)32 * alias_pitch(cap);
-  return 2 * slots * sizeof(uint64_t) + alias_stage_bytes(cap, elem) +
-         (((size_t)cap * sizeof(uint16_t) + 15) & ~(size_t)15);
+struct AliasExchange {            // one slot per warp of the group
+  uint64_t a, b, c;
+  uint32_t m, k;
+};
+template <int NW>
+__host__ __device__ inline size_t alias_group_bytes(int cap, int elem) {
+  const size_t slots = (size_t)32 * NW * alias_pitch<NW>(cap);
+  return 2 * slots * sizeof(uint64_t) + alias_stage_bytes<NW>(cap, elem) +
+         (((size_t)cap * sizeof(uint16_t) + 15) & ~(size_t)15) +
+         (NW > 1 ? 2 * NW * sizeof(AliasExchange) : 0);
 }
-// A warp's arrays in its shared memory
-struct AliasSmem {
+// A group's arrays in its shared memory, and its threads
+template <int NW>
+struct AliasGroup {
   uint64_t *u, *c;
   unsigned char* stage;
   uint16_t* x;
-  __device__ AliasSmem(unsigned char* base, int cap, int elem) {
+  AliasExchange* ex;              // two sets in turn
+  int lane, t;                    // lane of the warp, thread of the group
+  int bar;                        // the group's barrier
+  __device__ AliasGroup(unsigned char* smem, int group, int cap, int elem) {
+    unsigned char* base = smem + (size_t)group * alias_group_bytes<NW>(cap, elem);
     u = reinterpret_cast<uint64_t*>(base);
-    c = u + (size_t)32 * alias_pitch(cap);
-    stage = reinterpret_cast<unsigned char*>(c + (size_t)32 * alias_pitch(cap));
-    x = reinterpret_cast<uint16_t*>(stage + alias_stage_bytes(cap, elem));
+    c = u + (size_t)32 * NW * alias_pitch<NW>(cap);
+    stage = reinterpret_cast<unsigned char*>(c + (size_t)32 * NW * alias_pitch<NW>(cap));
+    unsigned char* xb = stage + alias_stage_bytes<NW>(cap, elem);
+    x = reinterpret_cast<uint16_t*>(xb);
+    ex = reinterpret_cast<AliasExchange*>(xb + (((size_t)cap * sizeof(uint16_t) + 15) & ~(size_t)15));
+    lane = threadIdx.x & 31;
+    t = threadIdx.x % (32 * NW);
+    bar = 1 + group;
+  }
+  __device__ void sync() const {
+    if (NW == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;\n" ::"r"(bar), "n"(32 * NW) : "memory");
   }
 };
 
-// f(i, slot) for the lane's items i = lane, lane + 32, ... of a K-item row
-template <typename F>
-__device__ __forceinline__ void alias_strided(int K, F f) {
-  const int lane = threadIdx.x & 31, npl = alias_npl(K), pitch = alias_pitch(K);
-  const int q32 = 32 / npl, r32 = 32 - q32 * npl;
-  int q = lane / npl, r = lane - q * npl;
-  for (int i = lane; i < K; i += 32) {
+// f(i, slot) for the thread's items i = t, t + 32 NW, ... of a K-item row
+template <int NW, typename F>
+__device__ __forceinline__ void alias_strided(const AliasGroup<NW>& g, int K, F f) {
+  constexpr int NT = 32 * NW;
+  const int npl = alias_npl<NW>(K), pitch = alias_pitch<NW>(K);
+  const int q32 = NT / npl, r32 = NT - q32 * npl;
+  int q = g.t / npl, r = g.t - q * npl;
+  for (int i = g.t; i < K; i += NT) {
     f(i, q * pitch + r);
     q += q32;
     r += r32;
@@ -104,24 +138,26 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 __device__ __forceinline__ uint32_t fixp(float w, int sh) { return small_fixp(w, sh); }
 __device__ __forceinline__ uint32_t fixp(double w, int sh) { return __double2uint_rz(ldexp(w, sh)); }
 
-// Build one row.  sm.stage: the K weights, item i at its slot (alias_strided); A: the value the
+// Build one row by the group's threads.  sm.stage: the K weights, item i at its slot (alias_strided); A: the value the
 // row must sum to (checked when check_A, to tol A + atol: a row whose spectral weight is at the
 // rounding level of G, such as an orbital no open channel reaches, carries only rounding noise);
 // out: K entries; rowsum_out: receives the row sum.  after_stage() is called by every lane once
 // the weights have been read (the caller reuses the stage for the next row).
-template <typename R, typename After>
-__device__ void alias_row(const AliasSmem& sm, int K, double A, bool check_A, double tol,
+template <typename R, int NW, typename After>
+__device__ void alias_row(const AliasGroup<NW>& sm, int K, double A, bool check_A, double tol,
                           double atol, uint64_t* __restrict__ out, double* rowsum_out,
                           int32_t* err, After after_stage) {
-  const int lane = threadIdx.x & 31;
+  constexpr int NT = 32 * NW;
+  const int lane = sm.lane, warp = sm.t >> 5;
   const unsigned FULL = 0xffffffffu;
-  const int npl = alias_npl(K), pitch = alias_pitch(K);
-  const int i0 = lane * npl;                                    // this lane's items [i0, i1)
+  const int npl = alias_npl<NW>(K), pitch = alias_pitch<NW>(K);
+  const int i0 = min(K, sm.t * npl);                            // this thread's items [i0, i1)
   const int i1 = min(K, i0 + npl);
-  const int mine = max(0, i1 - i0);
-  uint64_t* my_u = sm.u + lane * pitch;
+  const int mine = i1 - i0;
+  uint64_t* my_u = sm.u + sm.t * pitch;
   const R* w = reinterpret_cast<const R*>(sm.stage);
-  const R* my_w = w + lane * pitch;
+  const R* my_w = w + sm.t * pitch;
+  AliasExchange* const ex = sm.ex;
   // pass 1: largest weight; FP64 rows also take their FP64 sum here (lane-strided order, tree to
   // lane 0)
   R wmax = 0;
@@ -133,21 +169,29 @@ __device__ void alias_row(const AliasSmem& sm, int K, double A, bool check_A, do
     if (ok && v > wmax) wmax = v;
   }
   double part = 0.0;
-  if (sizeof(R) == 8) alias_strided(K, [&](int, int slot) { part += (double)w[slot]; });
+  if (sizeof(R) == 8 && warp == 0)                // (by one warp, whatever NW is: one order)
+    for (int i = lane; i < K; i += 32) part += (double)w[i / npl * pitch + i % npl];
   for (int off = 16; off > 0; off >>= 1) wmax = max(wmax, __shfl_xor_sync(FULL, wmax, off));
   if (__any_sync(FULL, bad) && lane == 0) atomicOr(err, ERR_NONFINITE);
+  if (NW > 1) {
+    R* wm = reinterpret_cast<R*>(&ex[warp].a);
+    if (lane == 0) *wm = wmax;
+    sm.sync();
+#pragma unroll
+    for (int v = 0; v < NW; ++v) wmax = max(wmax, *reinterpret_cast<const R*>(&ex[v].a));
+  }
   if (!(wmax > 0)) {
-    __syncwarp();
+    sm.sync();
     after_stage();
-    if (lane == 0) *rowsum_out = 0.0;
-    if (lane == 0 && check_A && A > 1e-300 && A > atol) atomicOr(err, ERR_ROWSUM);
-    for (int i = lane; i < K; i += 32) out[i] = pack(0xffffffffu, (uint32_t)i);
+    if (sm.t == 0) *rowsum_out = 0.0;
+    if (sm.t == 0 && check_A && A > 1e-300 && A > atol) atomicOr(err, ERR_ROWSUM);
+    for (int i = sm.t; i < K; i += NT) out[i] = pack(0xffffffffu, (uint32_t)i);
     return;
   }
-  int ex = 0;
-  if (sizeof(R) == 4) frexpf((float)wmax, &ex);   // wmax = f 2^ex, f in [0.5, 1)
-  else frexp((double)wmax, &ex);
-  const int sh = 32 - ex;                          // wmax 2^sh in [2^31, 2^32)
+  int e2p = 0;
+  if (sizeof(R) == 4) frexpf((float)wmax, &e2p);  // wmax = f 2^e2p, f in [0.5, 1)
+  else frexp((double)wmax, &e2p);
+  const int sh = 32 - e2p;                          // wmax 2^sh in [2^31, 2^32)
   auto unit = [&](int k) {
     const R v = my_w[k];
     return v > 0 && v < (R)INFINITY ? fixp(v, sh) : 0u;
@@ -168,17 +212,36 @@ __device__ void alias_row(const AliasSmem& sm, int K, double A, bool check_A, do
     const int oi = __shfl_xor_sync(FULL, imax, off);
     if (om > mmax || (om == mmax && oi < imax)) { mmax = om; imax = oi; }
   }
+  if (NW > 1) {
+    AliasExchange* const e2 = ex + NW;
+    if (lane == 0) {
+      e2[warp].a = T;
+      e2[warp].m = mmax;
+      e2[warp].k = (uint32_t)imax;
+    }
+    sm.sync();
+    T = 0;
+#pragma unroll
+    for (int v = 0; v < NW; ++v) {
+      T += e2[v].a;
+      if (e2[v].m > mmax || (e2[v].m == mmax && (int)e2[v].k < imax)) {
+        mmax = e2[v].m;
+        imax = (int)e2[v].k;
+      }
+    }
+  }
   // row sum: FP64 weights are summed in FP64; FP32 weights use the exact fixed-point sum
   // (within K 2^-32 of the largest weight)
   if (sizeof(R) == 8)
     for (int off = 16; off > 0; off >>= 1) part += __shfl_down_sync(FULL, part, off);
-  // the FP64 steps run on lane 0 only (FP64 throughput is low); the reciprocal is broadcast
+  // the FP64 steps run on one lane of a warp only (FP64 throughput is low); the reciprocal is
+  // broadcast
   uint64_t rcp = 0;
   if (lane == 0) {
     const double total = sizeof(R) == 8 ? part : ldexp((double)T, -sh);
     rcp = (uint64_t)(ldexp(1.0, 94) / (double)T);   // < 2^63 since T >= 2^31
-    *rowsum_out = total;
-    if (check_A && A > 1e-300 && fabs(total - A) > tol * A + atol) atomicOr(err, ERR_ROWSUM);
+    if (sm.t == 0) *rowsum_out = total;
+    if (sm.t == 0 && check_A && A > 1e-300 && fabs(total - A) > tol * A + atol) atomicOr(err, ERR_ROWSUM);
   }
   rcp = __shfl_sync(FULL, rcp, 0);
   // pass 3: u_i = floor(m_i K 2^32 / T) = (m_i K) (2^94 / T) / 2^62, a 48 x 63-bit product in
@@ -202,12 +265,24 @@ __device__ void alias_row(const AliasSmem& sm, int K, double A, bool check_A, do
     cnt += heavy ? 1u << 16 : 1u;
     dl += heavy ? 0u : (uint32_t)u;               // lights' units
   }
-  __syncwarp();
+  // the other exchange set has been read by every warp (each has passed the barrier after it)
+  if (NW > 1) {
+    uint64_t s = usum;
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(FULL, s, off);
+    if (lane == 0) ex[warp].b = s;
+  }
+  sm.sync();
   after_stage();
   const int nl_mine = (int)(cnt & 0xffffu), nh_mine = (int)(cnt >> 16);
   uint64_t dh = usum - dl - ((uint64_t)nh_mine << 32);          // excesses
   dl = ((uint64_t)nl_mine << 32) - dl;                            // deficits
-  for (int off = 16; off > 0; off >>= 1) usum += __shfl_xor_sync(FULL, usum, off);
+  if (NW == 1) {
+    for (int off = 16; off > 0; off >>= 1) usum += __shfl_xor_sync(FULL, usum, off);
+  } else {
+    usum = 0;
+#pragma unroll
+    for (int v = 0; v < NW; ++v) usum += ex[v].b;
+  }
   if (i0 <= imax && imax < i1) {                  // the signed remainder goes to the largest item
     const uint64_t rem = ((uint64_t)K << 32) - usum;
     const uint64_t u0 = my_u[imax - i0], u1 = u0 + rem;
@@ -231,7 +306,26 @@ __device__ void alias_row(const AliasSmem& sm, int K, double A, bool check_A, do
     const uint64_t oh = __shfl_up_sync(FULL, hx, off);
     if (lane >= off) { cx += oc; lx += ol; hx += oh; }
   }
-  const uint32_t ctot = __shfl_sync(FULL, cx, 31);
+  uint32_t ctot = __shfl_sync(FULL, cx, 31);
+  if (NW > 1) {
+    AliasExchange* const e2 = ex + NW;
+    if (lane == 31) {
+      e2[warp].a = lx;
+      e2[warp].b = hx;
+      e2[warp].m = cx;
+    }
+    sm.sync();
+    ctot = 0;
+#pragma unroll
+    for (int v = 0; v < NW; ++v) {
+      ctot += e2[v].m;
+      if (v < warp) {
+        cx += e2[v].m;
+        lx += e2[v].a;
+        hx += e2[v].b;
+      }
+    }
+  }
   const int nl = (int)(ctot & 0xffffu), nh = (int)(ctot >> 16);
   int r = (int)((cx - cnt) & 0xffffu), j = (int)((cx - cnt) >> 16);   // first light / heavy
   uint64_t runl = lx - dl, runh = hx - dh;                             // of this lane
@@ -248,9 +342,9 @@ __device__ void alias_row(const AliasSmem& sm, int K, double A, bool check_A, do
     j += heavy;
     r += !heavy;
   }
-  __syncwarp();
+  sm.sync();
   if (nl == 0 || nh == 0) {   // every item holds one slot (nh == 0 cannot happen: the sum is K 2^32)
-    for (int i = lane; i < K; i += 32) out[i] = pack(0xffffffffu, (uint32_t)i);
+    for (int i = sm.t; i < K; i += NT) out[i] = pack(0xffffffffu, (uint32_t)i);
     return;
   }
   auto Ec = [&](int jj) { return sm.c[K - 1 - jj]; };
@@ -263,7 +357,7 @@ __device__ void alias_row(const AliasSmem& sm, int K, double A, bool check_A, do
   // by this light: heavy j keeps 2^32 - (Lc_r - Ec_j) and aliases heavy j + 1.  Heavies without
   // excess at the front of the list (Ec = 0) and the last heavy are full.
   {
-    const int ra = (lane * nl) >> 5, rb = ((lane + 1) * nl) >> 5;
+    const int ra = sm.t * nl / NT, rb = (sm.t + 1) * nl / NT;
     if (ra < rb) {
       uint64_t st = ra == 0 ? 0ull : Lc(ra - 1);
       int jc = 0, hi = nh - 1;                            // first j with Ec_j > st, or the last
@@ -289,72 +383,84 @@ __device__ void alias_row(const AliasSmem& sm, int K, double A, bool check_A, do
         st = Lr;
       }
     }
-    if (lane == 0) sm.u[Xh(nh - 1)] = pack(0xffffffffu, Xh(nh - 1));
+    if (sm.t == 0) sm.u[Xh(nh - 1)] = pack(0xffffffffu, Xh(nh - 1));
   }
-  __syncwarp();
-  for (int i = lane; i < K; i += 32) out[i] = sm.u[i];
-  __syncwarp();
+  sm.sync();
+  for (int i = sm.t; i < K; i += NT) out[i] = sm.u[i];
+  sm.sync();
 }
 
-template <typename R>
+// Rows of the tasks with min_K < K <= max_K, a row per group of NW warps.
+template <typename R, int NW>
 __global__ void alias_kernel(const TaskDesc* __restrict__ tasks, int n_tasks, uint32_t total_jobs,
-                             int cap, double tol, const R* __restrict__ weights,
-                             double* __restrict__ rowsum, const double* __restrict__ mode_w,
-                             uint64_t* __restrict__ tab, uint64_t* __restrict__ mode_tab,
-                             int32_t* err) {
+                             int min_K, int max_K, int cap, double tol,
+                             const R* __restrict__ weights, double* __restrict__ rowsum,
+                             const double* __restrict__ mode_w, uint64_t* __restrict__ tab,
+                             uint64_t* __restrict__ mode_tab, int32_t* err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5;
-  const int nwarps = blockDim.x >> 5;
-  const AliasSmem sm(smem_raw + (size_t)warp * alias_warp_bytes(cap, (int)sizeof(R)), cap,
-                     (int)sizeof(R));
-  const uint32_t stride = gridDim.x * nwarps;
-  // task owning a job: jobs of a warp only increase, so the search starts at the last task found
-  int hint = 0;
-  auto find = [&](uint32_t jb) {
-    int lo = hint, hi = n_tasks - 1;
-    while (lo < hi) {
+  const int group = threadIdx.x / (32 * NW), ngroups = blockDim.x / (32 * NW);
+  const AliasGroup<NW> sm(smem_raw, group, cap, (int)sizeof(R));
+  const uint32_t stride = gridDim.x * ngroups;
+  // The group's first job at or after jb whose task is of this class, and that task: jobs of a
+  // group only increase, so the search starts at the last task found and passes over the tasks
+  // of the other class.
+  auto next_job = [&](uint32_t jb, int& task) -> uint32_t {
+    int lo = task, hi = n_tasks - 1;
+    while (lo < hi && jb < total_jobs) {
       const int mid = (lo + hi + 1) >> 1;
       if (tasks[mid].row_base <= jb) lo = mid; else hi = mid - 1;
     }
-    return lo;
+    while (jb < total_jobs) {
+      const int K = tasks[lo].K;
+      if (K > min_K && K <= max_K) break;
+      if (lo + 1 >= n_tasks) return total_jobs;
+      const uint32_t base = tasks[++lo].row_base;
+      if (base > jb) jb += (base - jb + stride - 1) / stride * stride;
+      while (lo + 1 < n_tasks && tasks[lo + 1].row_base <= jb) ++lo;
+    }
+    task = lo;
+    return jb < total_jobs ? jb : total_jobs;
   };
   // the weights of job jb go to the stage by asynchronous copies (one commit group)
-  auto stage = [&](uint32_t jb) {
-    const TaskDesc& d = tasks[find(jb)];
+  auto stage = [&](uint32_t jb, int task) {
+    const TaskDesc& d = tasks[task];
     const int row = (int)(jb - d.row_base);
     if (row < d.rows) {
       const R* src = weights + d.wt_off + (uint64_t)row * d.K;
       R* dst = reinterpret_cast<R*>(sm.stage);
-      alias_strided(d.K, [&](int i, int slot) { cp_async<(int)sizeof(R)>(dst + slot, src + i); });
+      alias_strided<NW>(sm, d.K, [&](int i, int slot) { cp_async<(int)sizeof(R)>(dst + slot, src + i); });
     } else {
       const double* src = mode_w + d.mode_off + (row - d.rows) * d.W;
       double* dst = reinterpret_cast<double*>(sm.stage);
-      alias_strided(d.W, [&](int i, int slot) { cp_async<8>(dst + slot, src + i); });
+      alias_strided<NW>(sm, d.W, [&](int i, int slot) { cp_async<8>(dst + slot, src + i); });
     }
     cp_async_commit();
   };
-  uint32_t job = blockIdx.x * nwarps + warp;
-  if (job < total_jobs) stage(job);
-  for (; job < total_jobs; job += stride) {
-    hint = find(job);
-    const TaskDesc& d = tasks[hint];
+  int task = 0;
+  uint32_t job = next_job(blockIdx.x * ngroups + group, task);
+  if (job < total_jobs) stage(job, task);
+  while (job < total_jobs) {
+    const TaskDesc& d = tasks[task];
     const int row = (int)(job - d.row_base);
     const double A = rowsum[job];                 // <i|A|i> (rows) or c_p (mode rows)
-    const uint32_t next = job + stride;
+    int task2 = task;
+    const uint32_t next = total_jobs - job > stride ? next_job(job + stride, task2) : total_jobs;
     auto after = [&]() {
-      if (next < total_jobs) stage(next);
+      if (next < total_jobs) stage(next, task2);
     };
     cp_async_wait_all();
-    __syncwarp();
+    sm.sync();
     if (row < d.rows) {
-      alias_row<R>(sm, d.K, A, true, tol, 1e-13 / d.t, tab + d.tab_off + (uint64_t)row * d.K,
-                   rowsum + job, err, after);
+      alias_row<R, NW>(sm, d.K, A, true, tol, 1e-13 / d.t, tab + d.tab_off + (uint64_t)row * d.K,
+                       rowsum + job, err, after);
     } else {
       const int p = row - d.rows;
-      alias_row<double>(sm, d.W, A, true, 1e-9, 1e-13 / d.t, mode_tab + d.mode_off + p * d.W,
-                        rowsum + job, err, after);
+      alias_row<double, NW>(sm, d.W, A, true, 1e-9, 1e-13 / d.t, mode_tab + d.mode_off + p * d.W,
+                            rowsum + job, err, after);
     }
-    __syncwarp();
+    sm.sync();
+    job = next;
+    task = task2;
   }
   cp_async_wait_all();
 }
@@ -533,8 +639,7 @@ __global__ void energy_alias_kernel(const TaskDesc* __restrict__ tasks, int n_ta
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
-  const AliasSmem sm(smem_raw + (size_t)warp * alias_warp_bytes(cap, (int)sizeof(double)), cap,
-                     (int)sizeof(double));
+  const AliasGroup<1> sm(smem_raw, warp, cap, (int)sizeof(double));
   double* s_w = reinterpret_cast<double*>(sm.stage);
   for (uint32_t job = blockIdx.x * nwarps + warp; job < total_jobs; job += gridDim.x * nwarps) {
     int lo = 0, hi = n_tasks - 1;
@@ -547,7 +652,7 @@ __global__ void energy_alias_kernel(const TaskDesc* __restrict__ tasks, int n_ta
     const int i = (int)(job - job_base[lo]);
     const int nE = ed.nE;
     const double inv2s2 = sigma > 0.0 ? 0.5 / (sigma * sigma) : 0.0;
-    alias_strided(nE, [&](int ep, int slot) {
+    alias_strided<1>(sm, nE, [&](int ep, int slot) {
       const TaskDesc& dp = tasks[ed.t0 + ep];
       const double dE = dp.E - d.E;
       const double K = sigma > 0.0 ? exp(-dE * dE * inv2s2) : (ep == d.e_idx ? 1.0 : 0.0);
@@ -555,7 +660,7 @@ __global__ void energy_alias_kernel(const TaskDesc* __restrict__ tasks, int n_ta
     });
     __syncwarp();
     double total = 0.0;
-    alias_row<double>(sm, nE, 0.0, false, 0.0, 0.0, etab + ed.eoff + (uint64_t)i * nE, &total,
+    alias_row<double, 1>(sm, nE, 0.0, false, 0.0, 0.0, etab + ed.eoff + (uint64_t)i * nE, &total,
                       err, [] {});
     __syncwarp();
   }
@@ -600,7 +705,7 @@ cudaError_t launch_energy_tables(const TaskDesc* d_tasks, int n_tasks, const Ene
                                  int32_t* d_err, cudaStream_t s) {
   if (total_jobs == 0) return cudaSuccess;
   const int cap = max_nE < 64 ? 64 : max_nE;
-  const size_t per_warp = alias_warp_bytes(cap, (int)sizeof(double));
+  const size_t per_warp = alias_group_bytes<1>(cap, (int)sizeof(double));
   int warps = 4;
   while (warps > 1 && per_warp * warps > 200 * 1024) --warps;
   const size_t smem = per_warp * warps;
@@ -620,53 +725,79 @@ cudaError_t launch_energy_tables(const TaskDesc* d_tasks, int n_tasks, const Ene
 }
 
 int alias_warps_max(int max_K) {
-  const int cap = max_K < 64 ? 64 : max_K;
-  const size_t per_warp = alias_warp_bytes(cap, (int)sizeof(double));
+  const int cap = max_K < 64 ? 64 : max_K < kAliasWarpRow ? max_K : kAliasWarpRow;
+  const size_t per_warp = alias_group_bytes<1>(cap, (int)sizeof(double));
   int w = 16;
   while (w > 1 && per_warp * w > 200 * 1024) --w;
   return w;
 }
 
-cudaError_t launch_alias_build(const TaskDesc* d_tasks, int n_tasks, uint32_t total_jobs,
-                               int max_K, int precision, const void* d_weights,
-                               double* d_rowsum, const double* d_mode_w, uint64_t* d_tab,
-                               uint64_t* d_mode_tab, int32_t* d_err, cudaStream_t s,
-                               int warps_req) {
-  if (total_jobs == 0) return cudaSuccess;
+namespace {
+template <typename R, int NW>
+cudaError_t alias_class(const TaskDesc* d_tasks, int n_tasks, uint32_t total_jobs, int min_K,
+                        int max_K, const R* d_weights, double* d_rowsum, const double* d_mode_w,
+                        uint64_t* d_tab, uint64_t* d_mode_tab, int32_t* d_err, cudaStream_t s,
+                        int groups_req) {
   const int cap = max_K < 64 ? 64 : max_K;
-  const size_t per_warp =
-      alias_warp_bytes(cap, precision == NEGF_FP64 ? (int)sizeof(double) : (int)sizeof(float));
-  const int wmax = alias_warps_max(max_K);
-  int warps = 8;
-  while (warps > 1 && per_warp * warps > 96 * 1024) --warps;
-  if (warps_req > 0) warps = warps_req < wmax ? warps_req : wmax;
-  const size_t smem = per_warp * warps;
+  const size_t per_group = alias_group_bytes<NW>(cap, (int)sizeof(R));
+  int groups = NW == 1 ? 8 : 1;
+  while (groups > 1 && per_group * groups > 96 * 1024) --groups;
+  if (NW == 1 && groups_req > 0) {
+    int most = 16;
+    while (most > 1 && per_group * most > 200 * 1024) --most;
+    groups = groups_req < most ? groups_req : most;
+  }
+  const size_t smem = per_group * groups;
   if (smem > 220 * 1024) return cudaErrorInvalidValue;   // rows beyond the shared-memory path
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  uint32_t blocks = (total_jobs + warps - 1) / warps;
+  uint32_t blocks = (total_jobs + groups - 1) / groups;
   const uint32_t cap_blocks = (uint32_t)sms * 32;
   if (blocks > cap_blocks) blocks = cap_blocks;
   // sum-rule tolerance: FP64 weights agree with A to rounding; FP32 propagation to ~1e-5
-  const double tol = precision == NEGF_FP64 ? 1e-8 : 1e-3;
-  cudaError_t e;
-  if (precision == NEGF_FP64) {
-    e = cudaFuncSetAttribute(alias_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e != cudaSuccess) return e;
-    alias_kernel<double><<<blocks, warps * 32, smem, s>>>(
-        d_tasks, n_tasks, total_jobs, cap, tol, static_cast<const double*>(d_weights), d_rowsum,
-        d_mode_w, d_tab, d_mode_tab, d_err);
-  } else {
-    e = cudaFuncSetAttribute(alias_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e != cudaSuccess) return e;
-    alias_kernel<float><<<blocks, warps * 32, smem, s>>>(
-        d_tasks, n_tasks, total_jobs, cap, tol, static_cast<const float*>(d_weights), d_rowsum,
-        d_mode_w, d_tab, d_mode_tab, d_err);
-  }
+  const double tol = sizeof(R) == 8 ? 1e-8 : 1e-3;
+  const cudaError_t e = cudaFuncSetAttribute(
+      alias_kernel<R, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  alias_kernel<R, NW><<<blocks, groups * 32 * NW, smem, s>>>(
+      d_tasks, n_tasks, total_jobs, min_K, max_K, cap, tol, d_weights, d_rowsum, d_mode_w, d_tab,
+      d_mode_tab, d_err);
   return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t alias_classes(const TaskDesc* d_tasks, int n_tasks, uint32_t total_jobs, int min_K,
+                          int max_K, const R* d_weights, double* d_rowsum, const double* d_mode_w,
+                          uint64_t* d_tab, uint64_t* d_mode_tab, int32_t* d_err, cudaStream_t s,
+                          int warps_req) {
+  cudaError_t e = cudaSuccess;
+  const int ends[3] = {0, kAliasShortRow, kAliasWarpRow};
+  for (int c = 0; c < 2 && e == cudaSuccess; ++c)
+    if (max_K > ends[c] && min_K <= ends[c + 1])
+      e = alias_class<R, 1>(d_tasks, n_tasks, total_jobs, ends[c],
+                            max_K < ends[c + 1] ? max_K : ends[c + 1], d_weights, d_rowsum,
+                            d_mode_w, d_tab, d_mode_tab, d_err, s, warps_req);
+  if (e == cudaSuccess && max_K > kAliasWarpRow)
+    e = alias_class<R, 4>(d_tasks, n_tasks, total_jobs, kAliasWarpRow, max_K, d_weights, d_rowsum,
+                          d_mode_w, d_tab, d_mode_tab, d_err, s, 0);
+  return e;
+}
+}  // namespace
+
+cudaError_t launch_alias_build(const TaskDesc* d_tasks, int n_tasks, uint32_t total_jobs,
+                               int min_K, int max_K, int precision, const void* d_weights,
+                               double* d_rowsum, const double* d_mode_w, uint64_t* d_tab,
+                               uint64_t* d_mode_tab, int32_t* d_err, cudaStream_t s,
+                               int warps_req) {
+  if (total_jobs == 0) return cudaSuccess;
+  if (precision == NEGF_FP64)
+    return alias_classes<double>(d_tasks, n_tasks, total_jobs, min_K, max_K,
+                                 static_cast<const double*>(d_weights), d_rowsum, d_mode_w, d_tab,
+                                 d_mode_tab, d_err, s, warps_req);
+  return alias_classes<float>(d_tasks, n_tasks, total_jobs, min_K, max_K,
+                              static_cast<const float*>(d_weights), d_rowsum, d_mode_w, d_tab,
+                              d_mode_tab, d_err, s, warps_req);
 }
 
 }  // namespace negf

@@ -582,6 +582,7 @@ struct Wave {
   size_t n_cta_mid = 0;
   int cols_max_W = 0;                // widest task of the warp-per-column chains
   int two_max_W = 0;                 // widest task with two-level tables
+  int min_KA = 3, max_KA = 3;        // shortest and longest row the alias kernels build
   bool any_two_split = false;        // two-level tasks whose level 2 comes from stored weights
   uint32_t cta_narrow() const {
     return (uint32_t)(tcjobs.size() - n_tc - n_cta_wide - n_cta_mid);
@@ -640,6 +641,10 @@ Wave make_wave(const Plan& P, int t0, int t1) {
   for (TaskDesc& d : w.desc)
     if (d.layout == NEGF_LAYOUT_TWO_LEVEL) d.l1w_off += w.wt;
   w.adesc = alias_descs(w.desc);
+  for (size_t i = 0; i < w.adesc.size(); ++i) {
+    w.min_KA = i ? std::min(w.min_KA, w.adesc[i].K) : w.adesc[i].K;
+    w.max_KA = std::max(w.max_KA, w.adesc[i].K);
+  }
   negf::sort_jobs_longest_first(w.tcjobs, w.desc.data());
   negf::sort_jobs_longest_first(cta, w.desc.data());
   negf::sort_jobs_longest_first(cta_n, w.desc.data());
@@ -859,7 +864,7 @@ negf_status build_wave(negf_ctx ctx, cudaStream_t s, const Plan& P, const Wave& 
   }
   if (e == cudaSuccess) {
     ProfScope ps(ctx, "alias_kernel", 1, s);
-    e = negf::launch_alias_build(d_adesc, nt, w.rows, P.max_KA, prec, d_weights, d_rowsum,
+    e = negf::launch_alias_build(d_adesc, nt, w.rows, w.min_KA, w.max_KA, prec, d_weights, d_rowsum,
                                  q.d_mode_w, d_tab, q.d_mode_tab, q.d_err, s, alias_warps);
   }
   if (e != cudaSuccess) {
@@ -2467,7 +2472,7 @@ negf_status plan_enqueue(negf_plan p, bool timed, cudaStream_t s) {
     }
     {
       SegScope sg(p, "alias_kernel", 1, s, timed);
-      CUDA_TRY(ctx, negf::launch_alias_build(da, ntw, wv.rows, P.max_KA, prec, p->d_weights[slot],
+      CUDA_TRY(ctx, negf::launch_alias_build(da, ntw, wv.rows, wv.min_KA, wv.max_KA, prec, p->d_weights[slot],
                                              p->d_rs[slot], q.d_mode_w, p->d_tab[slot],
                                              q.d_mode_tab, q.d_err, s, p->tune.alias_warps));
     }
@@ -2567,7 +2572,7 @@ negf_status plan_autotune(negf_plan p) {
     return e;
   };
   auto alias = [&](int aw) {
-    return negf::launch_alias_build(da, nt0, wv.rows, P.max_KA, prec, p->d_weights[0],
+    return negf::launch_alias_build(da, nt0, wv.rows, wv.min_KA, wv.max_KA, prec, p->d_weights[0],
                                     p->d_rs[0], q.d_mode_w, p->d_tab[0], q.d_mode_tab, q.d_err,
                                     s, aw);
   };

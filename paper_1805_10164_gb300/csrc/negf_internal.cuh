@@ -177,8 +177,10 @@ cudaError_t launch_inelastic_walk(const TaskDesc* d_tasks, int n_tasks, const En
                                   cudaStream_t s);
 // Alias tables of every row (and mode row); replaces the A values in rowsum by the FP64 row
 // sums after checking them.
+// min_K, max_K: the shortest and longest row among the tasks.  warps: warps per CTA of the kernel
+// that builds a row per warp (0: default).
 cudaError_t launch_alias_build(const TaskDesc* d_tasks, int n_tasks, uint32_t total_jobs,
-                               int max_K, int precision, const void* d_weights,
+                               int min_K, int max_K, int precision, const void* d_weights,
                                double* d_rowsum, const double* d_mode_w, uint64_t* d_tab,
                                uint64_t* d_mode_tab, int32_t* d_err, cudaStream_t s,
                                int warps = 0);
