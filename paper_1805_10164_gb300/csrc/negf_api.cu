@@ -591,8 +591,12 @@ struct Wave {
 
 using negf::add_tc_jobs;
 
+// Tasks of 32 < W < 64 whose block columns the CTA chain forms.
+inline bool cta_mid(const TaskDesc& d) { return d.cta_chain && d.W > 32 && d.W < 64; }
+
 Wave make_wave(const Plan& P, int t0, int t1) {
   Wave w;
+  int mid_W = 0;
   std::vector<TcJob> cta, cta_n, cta_m;
   w.t0 = t0;
   w.t1 = t1;
@@ -616,6 +620,7 @@ Wave make_wave(const Plan& P, int t0, int t1) {
       else add_tc_jobs(d.W > 32 ? cta_m : cta_n, k - t0, d.L);
     }
     if (!d.cta_chain && !d.fused) w.cols_max_W = std::max(w.cols_max_W, d.W);
+    if (cta_mid(d)) mid_W = std::max(mid_W, d.W);
     if (d.layout == NEGF_LAYOUT_TWO_LEVEL) {
       d.l1_off = w.tab + l2_u64;
       d.l1w_off = w.l1w;                 // rebased past the wave's weights below
@@ -638,6 +643,10 @@ Wave make_wave(const Plan& P, int t0, int t1) {
     w.cols += (uint32_t)(d.L + 2);
     w.desc.push_back(d);
   }
+  // Beside tasks of 32 < W < 64 the columns of W <= 16 are chain_kernel's, as when those tasks
+  // took it too: its roundings differ from chain_cols_kernel's in the last bits, and a batch of
+  // mixed widths keeps its tables.
+  if (w.cols_max_W > 0) w.cols_max_W = std::max(w.cols_max_W, mid_W);
   for (TaskDesc& d : w.desc)
     if (d.layout == NEGF_LAYOUT_TWO_LEVEL) d.l1w_off += w.wt;
   w.adesc = alias_descs(w.desc);
@@ -675,13 +684,19 @@ uint64_t wave_bytes(const Wave& w, int prec) {
 // 29.7 -> 21.1; W=40 x L=50, 16 tasks 28.0 -> 12.8; W=32 x L=100, 32 energies 12.9 -> 8.4;
 // W=10 x L=50, 64 energies 2.50 -> 1.78 (FP64 13.9 -> 6.6).  Batches whose eighths fill the
 // device several times over keep them: 1280 uneven tasks 271 (eighths) against 276 (one wave).
+// Batches of W <= 16 beside 32 < W < 64 keep them too: which of the two shares a wave with the
+// other decides the narrow tasks' last bits (make_wave).
 int default_per_wave(const Plan& P, int sm_count) {
   const int nt = (int)P.tasks.size();
   double fill = 0.0;
+  bool mid = false, cols = false;
   for (const TaskDesc& d : P.tasks) {
+    mid |= cta_mid(d);
+    cols |= !d.cta_chain && !d.fused;
     const double at_once = (double)sm_count * (d.W > 32 ? 2 : d.W > 16 ? 8 : 96);
     fill += (d.L + 2) / at_once;
   }
+  if (mid && cols) return std::max(1, (nt + 7) / 8);
   const int waves = std::max(1, std::min(8, (int)(fill / 4.0)));
   return std::max(1, (nt + waves - 1) / waves);
 }
