@@ -128,21 +128,25 @@ __global__ void __launch_bounds__(kLeadBlockThreads) lead_block_kernel(
 // The sweeps (rgf_sweep_rows_kernel) keep the block in registers instead: thread t owns column
 // j = t mod W of rows g, g + RG, g + 2 RG, ...
 // (g = t / W, RG = ceil(W / RPT) row groups of at most RPT rows), and a pivot costs one
-// barrier: the owners of row k publish it, the owners of column k publish that column, and the
-// owner of a_kk publishes 1/a_kk, into one of two buffers (alternating with k, so that the next
-// pivot's writes cannot overtake this pivot's reads); then every thread updates its rows.  On
-// GB300's FP64 pipe the arithmetic of a pivot dominates, and this form computes the reciprocal
-// once per pivot instead of once per thread.  The next slice's matrix E - H - Sigma_s - t^2 g_k
-// is formed in the same registers while g_k is stored.
+// barrier: the owners of row k publish it and the owners of column k publish that column, into
+// one of two buffers (alternating with k, so that the next pivot's writes cannot overtake this
+// pivot's reads); then every warp forms 1/a_kk for itself, its even lanes dividing for the real
+// part and its odd lanes for the imaginary part, and every thread updates its rows.  What
+// bounds a pivot is the chain of FP64 instructions of its busiest warp, since a warp's FP64
+// instruction holds its scheduler's share of the pipe for 64 cycles, so RPT is the smallest for
+// which kSweepRowsThreads threads hold the block: a W = 10 block takes four warps with one row a
+// thread.  Measured, GB300, W=10 x L=50, 64 energies: 1.55 -> 0.54 ms against four rows a thread
+// (one warp) and the reciprocal formed by a_kk's owner; W=24 x L=40 4.48 -> 2.01; W=64 x L=30
+// 22.0 -> 15.5.  The next slice's matrix E - H - Sigma_s - t^2 g_k is formed in the same
+// registers while g_k is stored.
 constexpr int kSweepThreads = 256;       // diagonal blocks: many CTAs
 constexpr int kSweepRowsThreads = 256;   // complex128 sweeps
 constexpr int kSweepRegMaxW = 16;        // complex64 sweeps up to this width: one warp each
 
 template <typename C>
 __host__ __device__ inline size_t sweep_rows_bytes(int W) {
-  // A W x W | pivot rows 2 x 64 | pivot columns 2 x 64 | 1/pivot 2 (complex) | perm 64, flag
-  // (int)
-  return sizeof(C) * (size_t)(W * W + 4 * 64 + 2) + sizeof(int) * (size_t)(64 + 2);
+  // A W x W | pivot rows 2 x 64 | pivot columns 2 x 64 (complex) | perm 64, flag (int)
+  return sizeof(C) * (size_t)(W * W + 4 * 64) + sizeof(int) * (size_t)(64 + 2);
 }
 
 // In-place inverse of the register-held block (see above; no pivot search: the caller takes
@@ -150,7 +154,11 @@ __host__ __device__ inline size_t sweep_rows_bytes(int W) {
 // this thread's rows, valid while i_m < W; false (uniformly) on a zero or non-finite pivot.
 template <typename C, int RPT>
 __device__ bool gj_regcols(C (&a)[RPT], int W, int RG, int g, int j, bool own, C* rowk,
-                           C* fcol, C* sinv) {
+                           C* fcol) {
+  using R = typename Real<C>::T;
+  const bool odd = threadIdx.x & 1;
+  const bool warp_owns = (int)(threadIdx.x & ~31u) < RG * W;
+  bool bad = false;
   int kr = 0, km = 0;                       // pivot k = kr + RG km: its row group and slot
   for (int k = 0; k < W; ++k) {
     const int b = k & 1;
@@ -162,7 +170,6 @@ __device__ bool gj_regcols(C (&a)[RPT], int W, int RG, int g, int j, bool own, C
       for (int m = 1; m < RPT; ++m)
         if (m == km) v = a[m];
       rk[j] = v;
-      if (j == k) sinv[b] = cdiv(mkc(1.0, 0.0, C{}), v);
     }
     if (own && j == k) {
 #pragma unroll
@@ -170,26 +177,24 @@ __device__ bool gj_regcols(C (&a)[RPT], int W, int RG, int g, int j, bool own, C
         if (g + RG * m < W) fc[g + RG * m] = a[m];
     }
     __syncthreads();
-    const C inv = sinv[b];
-    if (!finite_c(inv)) return false;       // every thread reads the same value
-    if (own) {
-      if (j != k) {
-        const C t = rk[j] * inv;            // a_kj / a_kk
+    if (warp_owns) {
+      // 1/a_kk: the even lanes divide for its real part, the odd ones for its imaginary part
+      const C p = rk[k];
+      const R dd = p.x * p.x + p.y * p.y;
+      const R q = (odd ? (R)0 - p.y : p.x) / dd;
+      const R o = __shfl_xor_sync(0xffffffffu, q, 1);
+      const C inv = odd ? C{o, q} : C{q, o};
+      bad |= !finite_c(inv);
+      if (own) {
+        // a_ij - a_ik t with t = a_kj / a_kk; column k: 0 - a_ik / a_kk.  One code path for
+        // both: a branch would send the warp through the FP64 pipe twice
+        const C t = j == k ? inv : rk[j] * inv;
 #pragma unroll
         for (int m = 0; m < RPT; ++m) {
           const int i = g + RG * m;
           if (i < W) {
-            const C v = a[m] - fc[i] * t;
+            const C v = (j == k ? mkc(0.0, 0.0, C{}) : a[m]) - fc[i] * t;
             a[m] = i == k ? t : v;
-          }
-        }
-      } else {
-#pragma unroll
-        for (int m = 0; m < RPT; ++m) {
-          const int i = g + RG * m;
-          if (i < W) {
-            const C v = mkc(0.0, 0.0, C{}) - fc[i] * inv;
-            a[m] = i == k ? inv : v;
           }
         }
       }
@@ -199,7 +204,7 @@ __device__ bool gj_regcols(C (&a)[RPT], int W, int RG, int g, int j, bool own, C
       ++km;
     }
   }
-  return true;
+  return !__syncthreads_or(bad);
 }
 
 template <typename C, int RPT>
@@ -215,8 +220,7 @@ __device__ __forceinline__ void sweep_rows_body(const TaskDesc& d, int dir,
   C* A = reinterpret_cast<C*>(smem_raw);   // the block, for the pivoted inversion only
   C* rowk = A + WW;
   C* fcol = rowk + 2 * 64;
-  C* sinv = fcol + 2 * 64;
-  int* perm = reinterpret_cast<int*>(sinv + 2);
+  int* perm = reinterpret_cast<int*>(fcol + 2 * 64);
   int* flag = perm + 64;
   const double* onsite = wire + d.onsite_off;
   const double* eta = onsite + d.n;
@@ -239,7 +243,7 @@ __device__ __forceinline__ void sweep_rows_body(const TaskDesc& d, int dir,
     const bool deph = __syncthreads_and(tid >= W || eta[k * W + tid] > 0.0);
     bool ok;
     if (deph) {
-      ok = gj_regcols<C, RPT>(a, W, RG, g, j, own, rowk, fcol, sinv);
+      ok = gj_regcols<C, RPT>(a, W, RG, g, j, own, rowk, fcol);
     } else {
       // an undephased site: partial pivoting on the block in shared memory
 #pragma unroll
@@ -284,11 +288,14 @@ __global__ void __launch_bounds__(kSweepRowsThreads) rgf_sweep_rows_kernel(
   const TaskDesc d = tasks[job >> 1];
   const int dir = job & 1;
   if (d.L < 2 || d.W > 64) return;
-  // rows per thread: W <= 16 -> 4, W <= 32 -> 8, W <= 64 -> 16 (at most 4 row groups, so that
-  // kSweepRowsThreads = 256 threads cover every width)
+  // rows per thread: the fewest with which kSweepRowsThreads threads hold the block
   if (d.W <= 16)
-    sweep_rows_body<cd, 4>(d, dir, wire, gL, gR, err, smem_raw);
+    sweep_rows_body<cd, 1>(d, dir, wire, gL, gR, err, smem_raw);
+  else if (d.W <= 22)
+    sweep_rows_body<cd, 2>(d, dir, wire, gL, gR, err, smem_raw);
   else if (d.W <= 32)
+    sweep_rows_body<cd, 4>(d, dir, wire, gL, gR, err, smem_raw);
+  else if (d.W <= 42)
     sweep_rows_body<cd, 8>(d, dir, wire, gL, gR, err, smem_raw);
   else
     sweep_rows_body<cd, 16>(d, dir, wire, gL, gR, err, smem_raw);
