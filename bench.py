@@ -78,8 +78,8 @@ def tensor_peak(kind):
 # wire (8 tasks) by the units processed (the blocks written and the g blocks read both grow as
 # n^2 per task): x 100 per task, x 256 / 8 tasks.
 MEASURED_TRAFFIC = {
-    ("walk_kernel", "wire_W10_L50_eta0.05_64E", "83e0ebef3d6f1969"): 133926400,
-    ("chain_cta_kernel", "wire_W64_L1000_eta0.005_256E", "a3bffe9ce92a6da4"): 5145210496000,
+    ("walk_kernel", "wire_W10_L50_eta0.05_64E", "f2e0d58f8c278a46"): 133581824,
+    ("chain_cta_kernel", "wire_W64_L1000_eta0.005_256E", "ba6ca48a4cf00100"): 5110117606400,
 }
 TRAFFIC_SOURCES = {"walk_kernel": ["k_walk.cu", "philox.cuh"],
                    "chain_cta_kernel": ["k_chain_cta.cu", "level2.cuh"]}
@@ -273,7 +273,7 @@ def adjoint_flops(w):
 def cta_chain_flops(wl, precision):
     """FP32 flops of the CTA-wide block-column products per step: 8 W^3 per block-column step
     (one W x W complex block times a W x W block); W = 64 runs towards slice 0 only
-    (G = G^T) plus the lead-L injection column: L(L-1)/2 + 2(L-1) steps per task; 16 < W <= 32
+    (G = G^T) plus the lead-L injection column: L(L-1)/2 + 2(L-1) steps per task; 16 < W < 64
     runs both directions: (L + 2)(L - 1) steps."""
     if precision != "fp32":
         return 0
@@ -282,7 +282,7 @@ def cta_chain_flops(wl, precision):
         W, L = w.W, w.L
         if W == 64:
             st = L * (L - 1) // 2 + 2 * (L - 1)
-        elif 16 < W <= 32:
+        elif 16 < W < 64:
             st = (L + 2) * (L - 1)
         else:
             continue
