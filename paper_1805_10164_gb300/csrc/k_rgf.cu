@@ -941,6 +941,163 @@ __global__ void chain_kernel(const TaskDesc* __restrict__ tasks, int n_tasks, ui
   }
 }
 
+// Complex128 block columns without kept G: one warp per (task, y).  G = G^T, so the chains run
+// towards slice 0 only (y < L: from slice y; the injection columns of lead L from slice 0 to
+// slice L-1, those of lead R back), and a step emits its block G_{k,m} twice: as the weights of
+// slice m's rows and, transposed, as those of slice k's.  The injection columns pass every
+// (G Phi)_k, which holds the lead weights of slice k's rows.  Bound by the FP64 pipe (two lanes a cycle
+// per SM): four fused multiply-adds per complex product, and half the products of both
+// directions.  A pair of consecutive warps takes a long and a short chain (y and L - 1 - y), the
+// longer one first or second by the parity of the pair's bits, so that every CTA and, within an
+// SM, every scheduler's share of the pipe gets about the same work; loops stay rolled (the kernel
+// of a tiny call is bound by its instruction fetches).  Measured, GB300, diagonal blocks and
+// columns against one warp per direction: W=10 x L=50, 64 energies 3.25 -> 1.50 ms (the columns
+// alone 3.0 -> 1.24, the pipe 87 % active while an SM has work); W=16 x L=100, 16 energies
+// 9.56 -> 4.29; W=24 x L=40, 4 energies 4.11 -> 3.28; W=64 x L=30, 2 energies 54.0 -> 40.8.
+__global__ void __maxnreg__(80) chain_sym_kernel(const TaskDesc* __restrict__ tasks, int n_tasks,
+                                 uint32_t n_jobs, int max_W, const double* __restrict__ wire,
+                                 const double* __restrict__ phig, const double* __restrict__ gam,
+                                 const cd* __restrict__ gL, const cd* __restrict__ gR,
+                                 const cd* __restrict__ start, double* __restrict__ weights) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t job = blockIdx.x * (blockDim.x >> 5) + warp;
+  if (job >= n_jobs) return;
+  const int task = find_task(n_tasks, job, [&](int t) { return tasks[t].col_base; });
+  const TaskDesc d = tasks[task];
+  if (d.fused || d.cta_chain) return;
+  const int W = d.W, L = d.L, n = d.n, K = d.K, WW = W * W;
+  const int i = (int)(job - d.col_base);
+  const int q = i >> 1;
+  const int y = i >= L ? i : ((i ^ __popc(q)) & 1) ? L - 1 - q : q;
+  const bool inj = y >= L, up = y == L;
+  const int m0 = inj ? (up ? 0 : L - 1) : y;
+  cd* X0 = reinterpret_cast<cd*>(smem_raw + (size_t)warp * chain_warp_bytes<cd>(max_W));
+  cd* X1 = X0 + WW;
+  cd* Gb = X1 + WW;
+  double* phi = reinterpret_cast<double*>(Gb + WW);
+  double* lgam = phi + WW;
+  const double* eta = wire + d.onsite_off + n;
+  for (int idx = lane; idx < WW; idx += 32) {
+    phi[idx] = phig[d.phi_off + idx];
+    X0[idx] = start[d.start_off + (uint64_t)y * WW + idx];
+  }
+  for (int m = lane; m < W; m += 32) lgam[m] = gam[d.lead_off + m];
+  __syncwarp();
+  double* wt = weights + d.wt_off;
+  const int row0 = inj ? n + (y - L) * W : m0 * W;
+  // idx / W without an integer division (see chain_kernel)
+  const float rW = 1.0f / (float)W;
+  auto div_w = [&](int idx) { return (int)(((float)idx + 0.5f) * rW); };
+  cd* cur = X0;
+  cd* nxt = X1;
+  const double mt = -d.t;
+  const bool split = W >= 4;
+  const int k_end = up ? L : -1, step = up ? 1 : -1;
+  const cd* gsrc = (up ? gR : gL) + d.g_off;
+  // the next block g_k is loaded into registers one step ahead (lane's entries idx = lane + 32 i)
+  constexpr int kPre = 4;                        // covers W * W <= 128 entries
+  const bool pre = WW <= 32 * kPre;
+  cd gpre[kPre];
+#pragma unroll 1
+  for (int k = m0;; k += step) {
+    const int kn = k + step;
+    if (pre && kn != k_end) {
+      const cd* gk = gsrc + (uint64_t)kn * WW;
+#pragma unroll
+      for (int q = 0; q < kPre; ++q)
+        if (lane + 32 * q < WW) gpre[q] = gk[lane + 32 * q];
+    }
+    // weights of block k (cur[a][b] = G_{(k,a),(m0,b)} or (G Phi)_{(k,a),mu}), |cur|^2 kept in sq
+    double* sq = reinterpret_cast<double*>(nxt);
+#pragma unroll 1
+    for (int idx = lane; idx < WW; idx += 32) {
+      const int b = div_w(idx), a = idx - b * W;
+      const double q = norm2(cur[a * W + b]);
+      wt[(uint64_t)(row0 + b) * K + k * W + a] = eta[k * W + a] * q;
+      sq[idx] = q;
+    }
+    __syncwarp();
+    if (inj) {
+      // the rows of slice k: <psi_a|Gamma|psi_a> = sum_nu Gamma_nu |(G Phi)_{(k,a),nu}|^2
+      for (int a = lane; a < W; a += 32) {
+        double sum = 0.0;
+#pragma unroll 1
+        for (int nu = 0; nu < W; ++nu) sum = fma(lgam[nu], sq[nu * W + a], sum);
+        wt[(uint64_t)(k * W + a) * K + n + (y - L)] = sum;
+      }
+      // the injection rows themselves: sum_nu Gamma_nu |(Phi^T X)_{nu b}|^2
+#pragma unroll 1
+      for (int col = 0; col < 2; ++col) {
+        if (k != (col ? L - 1 : 0)) continue;
+        __syncwarp();
+#pragma unroll 1
+        for (int idx = lane; idx < WW; idx += 32) {
+          const int nu = div_w(idx), b = idx - nu * W;
+          double re = 0.0, im = 0.0;
+#pragma unroll 1
+          for (int a = 0; a < W; ++a) {
+            const double f = phi[a * W + nu];
+            re = fma(f, cur[a * W + b].x, re);
+            im = fma(f, cur[a * W + b].y, im);
+          }
+          sq[idx] = norm2(cd{re, im});
+        }
+        __syncwarp();
+        for (int b = lane; b < W; b += 32) {
+          double sum = 0.0;
+#pragma unroll 1
+          for (int nu = 0; nu < W; ++nu) sum = fma(lgam[nu], sq[nu * W + b], sum);
+          wt[(uint64_t)(row0 + b) * K + n + col] = sum;
+        }
+      }
+    } else if (k != m0) {
+#pragma unroll 1
+      for (int idx = lane; idx < WW; idx += 32) {
+        const int a = div_w(idx), b = idx - a * W;
+        wt[(uint64_t)(k * W + a) * K + m0 * W + b] = eta[m0 * W + b] * sq[b * W + a];
+      }
+    }
+    if (kn == k_end) break;
+    if (pre) {
+#pragma unroll
+      for (int q = 0; q < kPre; ++q)
+        if (lane + 32 * q < WW) Gb[lane + 32 * q] = gpre[q];
+    } else {
+      const cd* gk = gsrc + (uint64_t)kn * WW;
+      for (int idx = lane; idx < WW; idx += 32) Gb[idx] = gk[idx];
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int idx = lane; idx < WW; idx += 32) {
+      const int a = div_w(idx), b = idx - a * W;
+      // partial sums of the four real products, from W = 4 of even and odd c apart: a fused
+      // multiply-add each, and no more rounding than one sum over c of rounded complex products
+      double p[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+      auto mac = [&](int c, double* o) {
+        const cd u = Gb[a * W + c], v = cur[c * W + b];
+        o[0] = fma(u.x, v.x, o[0]);
+        o[1] = fma(u.y, v.y, o[1]);
+        o[2] = fma(u.x, v.y, o[2]);
+        o[3] = fma(u.y, v.x, o[3]);
+      };
+      int c = 0;
+#pragma unroll 1
+      for (; split && c + 1 < W; c += 2) {
+        mac(c, p);
+        mac(c + 1, p + 4);
+      }
+#pragma unroll 1
+      for (; c < W; ++c) mac(c, p);
+      if (split)
+        for (int m = 0; m < 4; ++m) p[m] += p[m + 4];
+      nxt[idx] = cd{mt * (p[0] - p[1]), mt * (p[2] + p[3])};
+    }
+    __syncwarp();
+    cd* tmp = cur; cur = nxt; nxt = tmp;
+  }
+}
+
 int warps_for(size_t per_warp, int max_warps) {
   int w = max_warps;
   while (w > 1 && per_warp * w > 96 * 1024) --w;
@@ -1035,6 +1192,21 @@ cudaError_t columns_impl(const TaskDesc* d_tasks, int n_tasks, uint32_t n_cols, 
   int warps = warps_for(per, 8);
   if (chain_warps > 0) warps = chain_warps < chain_max<C>(max_W) ? chain_warps : chain_max<C>(max_W);
   const size_t smem = per * warps;
+  if (sizeof(C) == sizeof(cd) && d_green == nullptr) {
+    // two warps a CTA where the caller leaves it open, a long and a short chain, so that the
+    // SMs' shares of the CTAs are the same work (eight warps a CTA 1.77 ms, two 1.67)
+    if (chain_warps <= 0) warps = warps < 2 ? warps : 2;
+    const size_t smem_sym = per * warps;
+    cudaError_t e = cudaFuncSetAttribute(chain_sym_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem_sym);
+    if (e != cudaSuccess) return e;
+    chain_sym_kernel<<<(n_cols + warps - 1) / warps, 32 * warps, smem_sym, s>>>(
+        d_tasks, n_tasks, n_cols, max_W, d_wire, d_phi, d_gam, reinterpret_cast<const cd*>(d_gL),
+        reinterpret_cast<const cd*>(d_gR), reinterpret_cast<const cd*>(d_start),
+        reinterpret_cast<double*>(d_w));
+    return cudaGetLastError();
+  }
   cudaError_t e = cudaFuncSetAttribute(chain_kernel<C>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
