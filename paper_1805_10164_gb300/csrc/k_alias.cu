@@ -50,10 +50,10 @@ __device__ __forceinline__ uint64_t pack(uint32_t thr, uint32_t alias) {
 // A row of more than kAliasWarpRow slots is built by four warps, shorter ones by one: a row's
 // arrays (22 bytes a slot) leave room for few rows per SM, and one warp each then leaves it
 // idle between its dependent steps; four warps share a row's arrays for seven barriers a row.
-// One warp against four, ms: 702 slots (64 energies) 0.39, 0.78; 1002 (64,128 rows) 0.91, 1.01; 1602 0.65, 0.56;
-// 1702 (32 energies) 1.98, 1.25; 2002 (16 tasks) 1.34, 0.83.  A build launches one kernel per
-// class of row lengths among its tasks, the short rows (up to kAliasShortRow) with shared memory
-// for their own length: 1280 uneven tasks 42 -> 30 ms.
+// One warp against four, ms: 702 slots (64 energies) 0.39, 0.78; 1002 (64,128 rows) 0.91, 1.01;
+// 1602 0.65, 0.56; 1702 (32 energies) 1.98, 1.25; 2002 (16 tasks) 1.34, 0.83.  A build launches
+// one kernel per class of row lengths among its tasks, the short rows (up to kAliasShortRow) with
+// shared memory for their own length: 1280 uneven tasks 42 -> 30 ms.
 //
 // Each of the group's threads (the lanes of its NW warps) owns a block of npl consecutive items,
 // npl = ceil(K / (32 NW)).  Per-item values live in shared memory at slot

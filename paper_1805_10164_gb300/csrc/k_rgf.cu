@@ -213,7 +213,7 @@ __device__ __forceinline__ void sweep_rows_body(const TaskDesc& d, int dir,
                                                int32_t* err, unsigned char* smem_raw) {
   using R = typename Real<C>::T;
   const int W = d.W, L = d.L, WW = W * W;
-  const int tid = threadIdx.x, nth = blockDim.x;
+  const int tid = threadIdx.x;
   const int RG = (W + RPT - 1) / RPT;
   const int j = tid % W, g = tid / W;
   const bool own = g < RG;
