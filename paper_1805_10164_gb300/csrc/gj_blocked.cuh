@@ -81,7 +81,8 @@ struct BgShared {
   int undephased[2][2];         // nonzero: the slice (half of it) has a site without dephasing
   int perm[64];                 // pivoted fallback
   int flag[2];
-  int bad;                      // a pivot without a finite reciprocal
+  int bad[2];                   // a pivot without a finite reciprocal, inversions in turn: a warp
+                                // may still read one's flag while the next one's panel is made
 };
 
 __device__ __forceinline__ void bg_put4(float4* dst, const cf (&v)[4]) {
@@ -104,11 +105,12 @@ __device__ __forceinline__ void bg_panel_sync() {
 
 // Panel warps: eliminate the nb pivots k1 .. k1 + nb - 1 within the panel's columns v of this
 // lane's row, leaving the pivot columns in f and the reciprocals in inv; publishes them in
-// buffer buf and the panel's columns, now as after these pivots, in Bout.
+// buffer buf and the panel's columns, now as after these pivots, in Bout.  turn: 0, 1, 0, ... over
+// the inversions, the flag S.bad[turn] is this one's.
 // kFull: nb = 4 (every panel but perhaps the last), without branches between the pivots.
 template <int NH, bool kFull>
-__device__ __forceinline__ void bg_factor(BgShared& S, int k1, int nb, int buf, cf* Bout,
-                                          cf (&v)[4], cf (&f)[4], cf (&inv)[4]) {
+__device__ __forceinline__ void bg_factor(BgShared& S, int turn, int k1, int nb, int buf,
+                                          cf* Bout, cf (&v)[4], cf (&f)[4], cf (&inv)[4]) {
   const int row = threadIdx.x;                      // panel warps are warps 0 .. NH - 1
   const int own = row - k1;                         // 0 .. 3: this lane's row is pivot row `own`
   if ((unsigned)own < 4u) bg_put4(S.blk[own], v);
@@ -154,18 +156,18 @@ __device__ __forceinline__ void bg_factor(BgShared& S, int k1, int nb, int buf, 
   if (row == 0) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) S.inv[buf][q] = inv[q];
-    if (bad) S.bad = 1;
+    if (bad) S.bad[turn] = 1;
   }
 }
 
 // Invert the block.  On entry the columns >= 4 are in S.B[0], panel 0 has been eliminated by
 // bg_factor (buffer 0, columns in S.B[1]; the panel warps' f and inv from it), and the CTA has
 // synchronised.  On return (synchronised) the inverse is in S.B[NP & 1], NP = ceil(W / 4);
-// S.bad is set if some pivot had no finite reciprocal.  side() is called by the warps without
-// rows during panel 0.
+// S.bad[turn] is set if some pivot had no finite reciprocal, and not written again before the
+// inversion after the next.  side() is called by the warps without rows during panel 0.
 template <int NH, typename Side>
-__device__ __forceinline__ void bg_invert(BgShared& S, int W, cf (&v)[4], cf (&f)[4], cf (&inv)[4],
-                                          Side side) {
+__device__ __forceinline__ void bg_invert(BgShared& S, int turn, int W, cf (&v)[4], cf (&f)[4],
+                                          cf (&inv)[4], Side side) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int unit = bg_unit<NH>(warp);
   const int j = NH == 2 ? (unit & 1) * 32 + lane : lane;
@@ -211,8 +213,8 @@ __device__ __forceinline__ void bg_invert(BgShared& S, int W, cf (&v)[4], cf (&f
             v[c] = row == k0 + q ? tq[c] : n;
           }
         }
-        if (W - k1 >= 4) bg_factor<NH, true>(S, k1, 4, b ^ 1, X, v, f, inv);
-        else bg_factor<NH, false>(S, k1, W - k1, b ^ 1, X, v, f, inv);
+        if (W - k1 >= 4) bg_factor<NH, true>(S, turn, k1, 4, b ^ 1, X, v, f, inv);
+        else bg_factor<NH, false>(S, turn, k1, W - k1, b ^ 1, X, v, f, inv);
       }
     } else if (unit >= 0) {
       const int nb = min(4, W - k0);
@@ -287,9 +289,11 @@ __device__ __forceinline__ void bg_invert(BgShared& S, int W, cf (&v)[4], cf (&f
 // Form a slice's block, entry (i, c) = form(i, c), and invert it; the inverse is in S.B[NP & 1] on
 // return (synchronised), false (uniformly) on a pivot without a finite reciprocal.  form may
 // read entry (i, c) of the block before, which is in S.B[NP & 1].  pivot: partial pivoting (the
-// slice has a site without dephasing).  side() is called by the warps without columns.
+// slice has a site without dephasing).  side() is called by the warps without columns.  turn:
+// alternates over a CTA's inversions (bg_factor).
 template <int NH, typename Form, typename Side>
-__device__ __forceinline__ bool bg_slice(BgShared& S, int W, bool pivot, Form form, Side side) {
+__device__ __forceinline__ bool bg_slice(BgShared& S, int turn, int W, bool pivot, Form form,
+                                         Side side) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NP = (W + 3) >> 2;
   if (!pivot) {
@@ -303,8 +307,8 @@ __device__ __forceinline__ bool bg_slice(BgShared& S, int W, bool pivot, Form fo
 #pragma unroll
       for (int c = 0; c < 4; ++c)
         if (tid < W && c < W) v[c] = form(tid, c);
-      if (W >= 4) bg_factor<NH, true>(S, 0, 4, 0, S.B[1], v, f, inv);
-      else bg_factor<NH, false>(S, 0, W, 0, S.B[1], v, f, inv);
+      if (W >= 4) bg_factor<NH, true>(S, turn, 0, 4, 0, S.B[1], v, f, inv);
+      else bg_factor<NH, false>(S, turn, 0, W, 0, S.B[1], v, f, inv);
     } else if (unit >= 0 && j >= 4 && j < W) {
 #pragma unroll
       for (int r = 0; r < 8; ++r) {
@@ -313,8 +317,8 @@ __device__ __forceinline__ bool bg_slice(BgShared& S, int W, bool pivot, Form fo
       }
     }
     __syncthreads();
-    bg_invert<NH>(S, W, v, f, inv, side);
-    return !S.bad;
+    bg_invert<NH>(S, turn, W, v, f, inv, side);
+    return !S.bad[turn];
   }
   cf* A = S.B[(NP & 1) ^ 1];
   cf* Bg = S.B[NP & 1];

@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(kBgThreads<NH>) rgf_sweep_wide_kernel(
     if (lane == 0) S.undephased[s & 1][dw] = any;
   };
   fetch_diag(0);
-  if (tid == 0) S.bad = 0;
+  if (tid < 2) S.bad[tid] = 0;
   __syncthreads();
   const cf* lb = gL + d.g_off + (uint64_t)(L - 1) * WW;   // the lead block (launch_lead_blocks)
   cf* out = (dir == 0 ? gL : gR) + d.g_off;
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kBgThreads<NH>) rgf_sweep_wide_kernel(
 #pragma unroll
         for (int c = 0; c < 4; ++c)
           if (tid < W) v[c] = form(s, tid, c, gdst);
-        bg_factor<NH, true>(S, 0, 4, 0, S.B[1], v, f, inv);
+        bg_factor<NH, true>(S, s & 1, 0, 4, 0, S.B[1], v, f, inv);
       } else if (unit >= 0 && j >= 4 && j < W) {
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
@@ -107,8 +107,8 @@ __global__ void __launch_bounds__(kBgThreads<NH>) rgf_sweep_wide_kernel(
         }
       }
       __syncthreads();
-      bg_invert<NH>(S, W, v, f, inv, [&] { fetch_diag(s + 1); });
-      if (S.bad) {
+      bg_invert<NH>(S, s & 1, W, v, f, inv, [&] { fetch_diag(s + 1); });
+      if (S.bad[s & 1]) {
         if (tid == 0) atomicOr(err, ERR_SINGULAR);
         return;
       }
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kBgThreads<NH>, 1) diag_wide_kernel(
     return cf{__fsub_rn(__fsub_rn(e.x, l.x), r.x), __fsub_rn(__fsub_rn(e.y, l.y), r.y)};
   };
   if (tid < W) S.diag[0][tid] = wide_diag(d, onsite, eta, h, m0, tid);
-  if (tid == 0) S.bad = 0;
+  if (tid == 0) S.bad[0] = 0;
   const bool deph = __syncthreads_and(tid >= W || eta[m0 * W + tid] > 0.0);
   cf* G = S.B[NP & 1];
   cf* T = S.B[(NP & 1) ^ 1];                              // free once the inverse is in G
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kBgThreads<NH>, 1) diag_wide_kernel(
 #pragma unroll
       for (int c = 0; c < 4; ++c)
         if (tid < W) v[c] = form(tid, c);
-      bg_factor<NH, true>(S, 0, 4, 0, S.B[1], v, f, inv);
+      bg_factor<NH, true>(S, 0, 0, 4, 0, S.B[1], v, f, inv);
     } else if (unit >= 0 && j >= 4 && j < W) {
 #pragma unroll
       for (int r = 0; r < 8; ++r) {
@@ -219,8 +219,8 @@ __global__ void __launch_bounds__(kBgThreads<NH>, 1) diag_wide_kernel(
       }
     }
     __syncthreads();
-    bg_invert<NH>(S, W, v, f, inv, [] {});
-    if (S.bad) {
+    bg_invert<NH>(S, 0, W, v, f, inv, [] {});
+    if (S.bad[0]) {
       if (tid == 0) atomicOr(err, ERR_SINGULAR);
       return;
     }
