@@ -23,7 +23,12 @@
 // its longest walk.  What depends on the grid interval alone (its energies relative to mu,
 // thresholds, open ends, table offsets) is staged in shared memory once per block.  The block's
 // tally sits in shared memory too and is added to global memory once.  W=10 x L=50, 132 energies,
-// 1.6e7 walkers: 1.21 -> 0.76 ms.
+// 1.6e7 walkers: 1.21 -> 0.76 ms against a walker per thread and stride of the grid.
+//
+// Staging takes 88 bytes of shared memory an interval (the tally alone 24) and time per block, and
+// the votes of a warp lengthen every step of a lone walk.  Launches of few walkers and grids that
+// would leave fewer than four blocks an SM take thermal_few_kernel instead (which, and both
+// sides' times: launch_thermal_walk).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -46,6 +51,58 @@ struct ThermalInterval {
   bool open_lo, open_hi;
 };
 
+// Interval e of the grid of tasks task0 ..; thr and open channels of lead p
+__device__ __forceinline__ ThermalInterval thermal_interval(const TaskDesc* __restrict__ tasks,
+                                                            int task0, int e, bool two,
+                                                            const double* __restrict__ cvals, int p,
+                                                            double mu, unsigned long long thr) {
+  const TaskDesc &da = tasks[task0 + e], &db = tasks[task0 + e + 1];
+  ThermalInterval iv;
+  iv.thr = thr;
+  iv.tab_lo = two ? da.l1_off : da.tab_off;
+  iv.tab_hi = two ? db.l1_off : db.tab_off;
+  iv.l2_lo = da.tab_off;
+  iv.l2_hi = db.tab_off;
+  iv.e0 = (float)(da.E - mu);
+  iv.de = (float)(db.E - da.E);
+  iv.mode_lo = da.mode_off;
+  iv.mode_hi = db.mode_off;
+  iv.open_lo = cvals[2 * (task0 + e) + p] > 0.0;
+  iv.open_hi = cvals[2 * (task0 + e + 1) + p] > 0.0;
+  return iv;
+}
+
+// The word a = floor(alpha 2^32) of the energy of CDF value pE in interval `in`:
+// E - E_i = kT ln(F / (1 - F)) - (E_i - mu), the logarithms in FP32 of F and 1 - F (the latter
+// formed in FP64, so that both keep their relative precision); alpha to ~2^-20
+__device__ __forceinline__ uint32_t thermal_alpha(double pE, double kT, const ThermalInterval& in) {
+  const float lnr = logf((float)pE) - logf((float)(1.0 - pE));
+  const float dE = (float)kT * lnr - in.e0;
+  float alpha = dE / in.de;
+  alpha = alpha < 0.f ? 0.f : (alpha > 1.f ? 1.f : alpha);
+  const float af = floorf(alpha * 4294967296.f);
+  return af >= 4294967295.f ? 0xffffffffu : (uint32_t)af;
+}
+
+// The site drawn within slice k of a row's level-2 blocks (v = 31 random bits): the index of the
+// next row
+__device__ __forceinline__ uint32_t thermal_site(const uint64_t* __restrict__ blocks, uint32_t row,
+                                                 uint32_t k, uint32_t L, uint32_t W, uint32_t B2,
+                                                 uint32_t v) {
+  const uint4* blk =
+      reinterpret_cast<const uint4*>(blocks) + (((uint64_t)row * L + k) * B2 >> 2);
+  uint32_t oct = 0;
+  if (W > 8) {
+    const uint4 q0 = __ldg(blk), q1 = __ldg(blk + 1);
+    oct = (q0.x <= v) + (q0.y <= v) + (q0.z <= v) + (q0.w <= v) + (q1.x <= v) + (q1.y <= v) +
+          (q1.z <= v) + (q1.w <= v);
+    blk += 2 + 2 * oct;
+  }
+  const uint4 o0 = __ldg(blk), o1 = __ldg(blk + 1);
+  return k * W + 8 * oct + (o0.x <= v) + (o0.y <= v) + (o0.z <= v) + (o0.w <= v) + (o1.x <= v) +
+         (o1.y <= v) + (o1.z <= v) + (o1.w <= v);
+}
+
 __device__ __forceinline__ void smem_add64(unsigned* lohi, unsigned v) {
   const unsigned old = atomicAdd(lohi, v);
   if (old + v < old) atomicAdd(lohi + 1, 1u);
@@ -55,6 +112,21 @@ __device__ __forceinline__ void add64(unsigned* lohi, uint64_t v) {
   if (v == 0) return;
   smem_add64(lohi, (unsigned)v);
   if (v >> 32) atomicAdd(lohi + 1, (unsigned)(v >> 32));
+}
+
+// Per-interval sums of the walks just absorbed at q, lanes `done` (the calling lane among them):
+// lanes with the same interval pool theirs and one of them adds them
+__device__ __forceinline__ void thermal_add(unsigned* s_t, unsigned done, int iv, uint32_t a) {
+  const unsigned grp = __match_any_sync(done, iv);
+  const uint32_t a16 = a >> 16, sq = a16 * a16;
+  const uint32_t cnt = __popc(grp);
+  const uint32_t a_hi = __reduce_add_sync(grp, a >> 16), a_lo = __reduce_add_sync(grp, a & 0xffffu);
+  const uint32_t s_hi = __reduce_add_sync(grp, sq >> 16), s_lo = __reduce_add_sync(grp, sq & 0xffffu);
+  if ((int)(threadIdx.x & 31) == __ffs(grp) - 1) {
+    smem_add64(&s_t[2 * (3 * iv + 0)], cnt);
+    add64(&s_t[2 * (3 * iv + 1)], ((uint64_t)a_hi << 16) + a_lo);
+    add64(&s_t[2 * (3 * iv + 2)], ((uint64_t)s_hi << 16) + s_lo);
+  }
 }
 
 // kTwo: the grid's tables are two-level (level 1 an alias row over the slices and leads, level 2
@@ -78,22 +150,8 @@ __global__ void __launch_bounds__(kThermalThreads) thermal_walk_kernel(
   unsigned* s_t = reinterpret_cast<unsigned*>(s_iv + (M - 1));
   const int n_fields = 3 * (M - 1) + 5;
   for (int i = threadIdx.x; i < 2 * n_fields; i += blockDim.x) s_t[i] = 0u;
-  for (int e = threadIdx.x; e < M - 1; e += blockDim.x) {
-    const TaskDesc &da = tasks[task0 + e], &db = tasks[task0 + e + 1];
-    ThermalInterval iv;
-    iv.thr = thr[e];
-    iv.tab_lo = kTwo ? da.l1_off : da.tab_off;
-    iv.tab_hi = kTwo ? db.l1_off : db.tab_off;
-    iv.l2_lo = da.tab_off;
-    iv.l2_hi = db.tab_off;
-    iv.e0 = (float)(da.E - mu);
-    iv.de = (float)(db.E - da.E);
-    iv.mode_lo = da.mode_off;
-    iv.mode_hi = db.mode_off;
-    iv.open_lo = cvals[2 * (task0 + e) + p] > 0.0;
-    iv.open_hi = cvals[2 * (task0 + e + 1) + p] > 0.0;
-    s_iv[e] = iv;
-  }
+  for (int e = threadIdx.x; e < M - 1; e += blockDim.x)
+    s_iv[e] = thermal_interval(tasks, task0, e, kTwo, cvals, p, mu, thr[e]);
   __syncthreads();
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -153,14 +211,7 @@ __global__ void __launch_bounds__(kThermalThreads) thermal_walk_kernel(
         }
         iv = lo_i < M - 2 ? lo_i : M - 2;
         const ThermalInterval& in = s_iv[iv];
-        // E - E_i = kT ln(F / (1 - F)) - (E_i - mu): the logarithms in FP32 of F and 1 - F (the
-        // latter formed in FP64, so that both keep their relative precision); alpha to ~2^-20
-        const float lnr = logf((float)pE) - logf((float)(1.0 - pE));
-        const float dE = (float)kT * lnr - in.e0;
-        float alpha = dE / in.de;
-        alpha = alpha < 0.f ? 0.f : (alpha > 1.f ? 1.f : alpha);
-        const float af = floorf(alpha * 4294967296.f);
-        a = af >= 4294967295.f ? 0xffffffffu : (uint32_t)af;
+        a = thermal_alpha(pE, kT, in);
         // an interval open at both ends mixes the two tables; one open at a single end walks
         // with that end's table alone (a chain without an open lead never absorbs)
         open_hi = in.open_hi;
@@ -200,19 +251,7 @@ __global__ void __launch_bounds__(kThermalThreads) thermal_walk_kernel(
         if (k >= L) {
           j = n + (k - L);
         } else {
-          const uint32_t v = r.w >> 1;
-          const uint4* blk = reinterpret_cast<const uint4*>(tab + (up ? in.l2_hi : in.l2_lo)) +
-                             (((uint64_t)row * L + k) * B2 >> 2);
-          uint32_t oct = 0;
-          if (W > 8) {
-            const uint4 q0 = __ldg(blk), q1 = __ldg(blk + 1);
-            oct = (q0.x <= v) + (q0.y <= v) + (q0.z <= v) + (q0.w <= v) + (q1.x <= v) +
-                  (q1.y <= v) + (q1.z <= v) + (q1.w <= v);
-            blk += 2 + 2 * oct;
-          }
-          const uint4 o0 = __ldg(blk), o1 = __ldg(blk + 1);
-          j = k * W + 8 * oct + (o0.x <= v) + (o0.y <= v) + (o0.z <= v) + (o0.w <= v) +
-              (o1.x <= v) + (o1.y <= v) + (o1.z <= v) + (o1.w <= v);
+          j = thermal_site(tab + (up ? in.l2_hi : in.l2_lo), row, k, L, W, B2, r.w >> 1);
         }
       }
       ++steps;
@@ -225,21 +264,163 @@ __global__ void __launch_bounds__(kThermalThreads) thermal_walk_kernel(
         row = j;
       }
     }
-    // per-interval sums: lanes with the same interval pool theirs and one of them adds them
     const unsigned done = __ballot_sync(FULL, absorbed);
-    if (absorbed) {
-      const unsigned grp = __match_any_sync(done, iv);
-      const uint32_t a16 = a >> 16, sq = a16 * a16;
-      const uint32_t cnt = __popc(grp);
-      const uint32_t a_hi = __reduce_add_sync(grp, a >> 16), a_lo = __reduce_add_sync(grp, a & 0xffffu);
-      const uint32_t s_hi = __reduce_add_sync(grp, sq >> 16), s_lo = __reduce_add_sync(grp, sq & 0xffffu);
-      if (lane == __ffs(grp) - 1) {
-        smem_add64(&s_t[2 * (3 * iv + 0)], cnt);
-        add64(&s_t[2 * (3 * iv + 1)], ((uint64_t)a_hi << 16) + a_lo);
-        add64(&s_t[2 * (3 * iv + 2)], ((uint64_t)s_hi << 16) + s_lo);
+    if (absorbed) thermal_add(s_t, done, iv, a);
+  }
+  add64(&s_t[2 * (G0 + 0)], my_abs0);
+  add64(&s_t[2 * (G0 + 1)], my_abs1);
+  add64(&s_t[2 * (G0 + 2)], my_closed);
+  add64(&s_t[2 * (G0 + 3)], my_trunc);
+  add64(&s_t[2 * (G0 + 4)], my_steps);
+  __syncthreads();
+  for (int f = threadIdx.x; f < n_fields; f += blockDim.x) {
+    const unsigned long long v = ((unsigned long long)s_t[2 * f + 1] << 32) | s_t[2 * f];
+    if (v) atomicAdd(tally + f, v);
+  }
+}
+
+// The same walks where walkers are few or the grid is large: the intervals' data is read where a
+// walker is set up (only the tally takes shared memory), and once nothing is left to hand out
+// every lane goes on alone, without the warp's votes, the next Philox block drawn while a
+// table entry is fetched.  Four blocks an SM: with five, 48 registers, a lone walk's step
+// takes 30 % longer.
+template <bool kTwo>
+__global__ void __launch_bounds__(kThermalThreads, 4) thermal_few_kernel(
+    const TaskDesc* __restrict__ tasks, int task0, int M, uint32_t wire,
+    const uint64_t* __restrict__ tab, const uint64_t* __restrict__ mode_tab,
+    const double* __restrict__ cvals, int p, PhiloxKey key, uint64_t walkers, uint64_t id_offset,
+    uint32_t max_steps, double mu, double kT, double F0, double window,
+    const unsigned long long* __restrict__ thr, unsigned long long* __restrict__ tally,
+    int32_t* __restrict__ t_lead,
+    uint32_t* __restrict__ t_steps, int32_t* __restrict__ t_interval, uint32_t* __restrict__ t_a,
+    unsigned chunk_size) {
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  unsigned* s_t = reinterpret_cast<unsigned*>(s_raw);                      // the tally, as above
+  const int n_fields = 3 * (M - 1) + 5;
+  for (int i = threadIdx.x; i < 2 * n_fields; i += blockDim.x) s_t[i] = 0u;
+  __syncthreads();
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const unsigned lt_mask = (1u << lane) - 1u;
+  const int q = 1 - p;
+  const int G0 = 3 * (M - 1);
+  const uint32_t ctr3 = 0x80000000u | wire;
+  const TaskDesc& d0 = tasks[task0];
+  const uint32_t n = (uint32_t)d0.n, W = (uint32_t)d0.W, K = (uint32_t)d0.K;
+  const uint32_t L = (uint32_t)d0.L, K1 = kTwo ? L + 2 : K, B2 = (uint32_t)level2_words(d0.W);
+  uint64_t my_abs0 = 0, my_abs1 = 0, my_closed = 0, my_trunc = 0, my_steps = 0;
+  const uint64_t stride = (uint64_t)gridDim.x * (kThermalThreads / 32) * chunk_size;
+  uint64_t chunk = ((uint64_t)blockIdx.x * (kThermalThreads / 32) + (threadIdx.x >> 5)) * chunk_size;
+  unsigned taken = 0;                                 // walkers of the chunk handed out
+  // the walk in flight, its tables and (ended at q, not in the tally yet) whether it was absorbed
+  bool has = false, mix = false, open_hi = false, absorbed = false;
+  uint64_t g = 0;
+  uint32_t lo = 0, hi = 0, a = 0, b = 0, row = 0, steps = 0;
+  const uint64_t *t_lo = tab, *t_hi = tab, *l2_lo = tab, *l2_hi = tab;
+  int iv = 0;
+  auto upper = [&](uint32_t word) { return mix ? word < a : open_hi; };
+  auto draw = [&](uint32_t at) { return philox4x32_10(make_uint4(at, lo, hi, ctr3), key); };
+  auto finish = [&](int outcome) {
+    if (outcome == 0) ++my_abs0;
+    else if (outcome == 1) ++my_abs1;
+    else if (outcome == -1) ++my_closed;
+    else ++my_trunc;
+    my_steps += steps;
+    if (t_lead) t_lead[g] = outcome;
+    if (t_steps) t_steps[g] = steps;
+    if (t_interval) t_interval[g] = iv;
+    if (t_a) t_a[g] = a;
+    has = false;
+    absorbed = outcome == q;
+  };
+  // one transition from Philox block r; meanwhile() runs while the table entry is fetched
+  auto step = [&](const uint4 r, auto meanwhile) {
+    const bool up = upper(r.z);
+    const uint32_t cc = __umulhi(r.x, K1);
+    const uint64_t ee = __ldg((up ? t_hi : t_lo) + (uint64_t)row * K1 + cc);
+    meanwhile();
+    uint32_t j = r.y < (uint32_t)ee ? cc : (uint32_t)(ee >> 32);
+    if (kTwo) {
+      const uint32_t k = j;
+      j = k >= L ? n + (k - L)
+                 : thermal_site(up ? l2_hi : l2_lo, row, k, L, W, B2, r.w >> 1);
+    }
+    ++steps;
+    if (j >= n) finish((int)(j - n));
+    else if (steps >= max_steps) finish(-2);
+    else row = j;
+  };
+  while (chunk < walkers) {
+    // ---- set up new walkers once 20 lanes are idle
+    const unsigned idle = __ballot_sync(FULL, !has);
+    if (__popc(idle) >= 20) {
+      const unsigned size =
+          walkers - chunk < chunk_size ? (unsigned)(walkers - chunk) : chunk_size;
+      const unsigned mine = taken + __popc(idle & lt_mask);
+      taken += __popc(idle);
+      if (!has && mine < size) {
+        g = chunk + mine;
+        const uint64_t wid = id_offset + g;
+        lo = (uint32_t)wid;
+        hi = (uint32_t)(wid >> 32);
+        const uint4 r0 = draw(0u);
+        const uint64_t v = (((uint64_t)r0.x << 32) | r0.y) >> 11;
+        const double u = ((double)v + 0.5) * 0x1p-53;
+        const double pE = F0 + u * window;                // F(E) of the drawn energy
+        int lo_i = 0, hi_i = M - 1;                       // the interval, as above
+        while (lo_i < hi_i) {
+          const int mid = (lo_i + hi_i) >> 1;
+          if (thr[mid] <= v) lo_i = mid + 1; else hi_i = mid;
+        }
+        iv = lo_i < M - 2 ? lo_i : M - 2;
+        const ThermalInterval in = thermal_interval(tasks, task0, iv, kTwo, cvals, p, mu, 0ull);
+        a = thermal_alpha(pE, kT, in);
+        open_hi = in.open_hi;
+        mix = in.open_lo && in.open_hi;
+        t_lo = tab + in.tab_lo;
+        t_hi = tab + in.tab_hi;
+        l2_lo = tab + in.l2_lo;
+        l2_hi = tab + in.l2_hi;
+        steps = 0;
+        if (in.open_lo || in.open_hi) {
+          const uint4 r1 = draw(1u);
+          const uint64_t* mrow = mode_tab + (upper(r0.z) ? in.mode_hi : in.mode_lo) + p * W;
+          const uint32_t c = __umulhi(r1.x, W);
+          const uint64_t e = __ldg(mrow + c);
+          row = n + p * W + (r1.y < (uint32_t)e ? c : (uint32_t)(e >> 32));
+          b = 2;
+          has = true;
+        } else {
+          finish(-1);
+        }
       }
+      if (taken >= size) {
+        chunk += stride;
+        taken = 0;
+      }
+      if (chunk >= walkers) break;
+    }
+    // ---- one transition of every walk in flight
+    if (has) {
+      const uint4 r = draw(b++);
+      step(r, [] {});
+    }
+    const unsigned done = __ballot_sync(FULL, absorbed);
+    if (absorbed) thermal_add(s_t, done, iv, a);
+    absorbed = false;
+  }
+  // ---- nothing left to hand out: every walk to its end
+  if (has) {
+    uint4 r = draw(b);
+    while (has) {
+      uint4 next;
+      step(r, [&] { next = draw(++b); });
+      r = next;
     }
   }
+  __syncwarp();
+  const unsigned done = __ballot_sync(FULL, absorbed);
+  if (absorbed) thermal_add(s_t, done, iv, a);
   add64(&s_t[2 * (G0 + 0)], my_abs0);
   add64(&s_t[2 * (G0 + 1)], my_abs1);
   add64(&s_t[2 * (G0 + 2)], my_closed);
@@ -341,19 +522,49 @@ cudaError_t launch_thermal_walk(const TaskDesc* d_tasks, int task0, int M, int w
                                 uint32_t* d_a, int sm_count, cudaStream_t s, bool two_level) {
   if (walkers == 0 || M < 2) return cudaSuccess;
   const PhiloxKey key{(uint32_t)seed, (uint32_t)(seed >> 32)};
-  const size_t smem = sizeof(ThermalInterval) * (size_t)(M - 1) +
-                      sizeof(unsigned) * 2 * (size_t)(3 * (M - 1) + 5);
-  const uint64_t need = (walkers + kThermalThreads - 1) / kThermalThreads;
-  uint64_t blocks = (uint64_t)sm_count * 8;
-  if (blocks > need) blocks = need;
-  auto kern = two_level ? thermal_walk_kernel<true> : thermal_walk_kernel<false>;
-  const cudaError_t e =
+  // Which kernel (GB300, us of the kernel; "before" a walker per thread and stride of the grid):
+  // * grids of more than 651 intervals: staged, fewer than four blocks fit an SM.  W=4 x L=10,
+  //   1.6e7 walkers: 1000 energies 914 staged, 683 few (before 657), 2046 energies 1728, 856 (780);
+  //   W=10 x L=50, 1000 energies 1306, 949 (1452);
+  // * up to three walkers a lane (four blocks an SM; 466,944 walkers on 152 SMs): a lone walk's
+  //   latency counts.  W=3 x L=150, 9 energies, 1e5 walkers 195, 109 (before 134), 5e5 267, 170
+  //   (226); W=4 x L=10 1e5 17, 16 (17), 5e5 33, 38 (31).
+  // The staging kernel takes the blocks that fit while a lane has fewer than eight walkers (those
+  // of a second round would wait for the first: W=10 x L=50, 9 energies, 7e5 walkers 73 -> 65), and
+  // more beyond, which evens out the ends of the blocks (4e6 walkers 201 -> 188).  The few kernel
+  // takes the blocks that fit, or up to half as many more if each lane then has one walker.
+  const size_t tally = sizeof(unsigned) * 2 * (size_t)(3 * (M - 1) + 5);
+  const size_t staged = tally + sizeof(ThermalInterval) * (size_t)(M - 1);
+  constexpr size_t kStagedMost = 56 * 1024;
+  const uint64_t lanes = (uint64_t)sm_count * 4 * kThermalThreads;
+  const bool few = staged > kStagedMost || walkers <= 3 * lanes;
+  const size_t smem = few ? tally : staged;
+  auto kern = two_level ? (few ? thermal_few_kernel<true> : thermal_walk_kernel<true>)
+                        : (few ? thermal_few_kernel<false> : thermal_walk_kernel<false>);
+  cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  int per_sm = 8;
+  if (few || walkers < 8 * lanes) {
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThermalThreads, smem);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) per_sm = 1;
+  }
+  const uint64_t need = (walkers + kThermalThreads - 1) / kThermalThreads;
+  uint64_t blocks = (uint64_t)sm_count * per_sm;
+  if (blocks > need || (few && 2 * need <= 3 * blocks)) blocks = need;
+  const uint64_t warps = blocks * (kThermalThreads / 32);
+  unsigned chunk = walk_chunk(walkers, warps);
+  if (few && chunk == 512) {
+    // equal chunks: with as many blocks as fit, a share of 513 walkers in chunks of 512 would give
+    // some warps twice the walks of the others (4e6 walkers, 1000 energies: 207 -> 193)
+    const uint64_t per = (walkers + warps - 1) / warps, n = (per + 511) / 512;
+    chunk = (unsigned)(((per + n - 1) / n + 31) / 32 * 32);
+  }
   kern<<<(unsigned)blocks, kThermalThreads, smem, s>>>(
       d_tasks, task0, M, (uint32_t)wire, d_tab, d_mode_tab, d_c, start_lead, key, walkers,
       id_offset, max_steps, mu, kT, F0, window, d_thr, d_tally, d_lead, d_steps, d_interval,
-      d_a, walk_chunk(walkers, blocks * (kThermalThreads / 32)));
+      d_a, chunk);
   return cudaGetLastError();
 }
 
