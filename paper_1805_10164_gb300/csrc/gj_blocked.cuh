@@ -79,8 +79,7 @@ struct BgShared {
   cf inv[2][4];                 // reciprocals of the panel's pivots
   cf diag[2][64];               // diagonal of E - H - Sigma_s of a slice
   int undephased[2][2];         // nonzero: the slice (half of it) has a site without dephasing
-  int perm[64];                 // pivoted fallback
-  int flag[2];
+  int perm[64];                 // pivoted inversions
   int bad[2];                   // a pivot without a finite reciprocal, inversions in turn: a warp
                                 // may still read one's flag while the next one's panel is made
 };
@@ -286,6 +285,70 @@ __device__ __forceinline__ void bg_invert(BgShared& S, int turn, int W, cf (&v)[
   }
 }
 
+// The buffer of S.B in which bg_pivoted takes its block (one exchange of buffers per pivot, and
+// one as the result is put in order)
+__device__ __forceinline__ cf* bg_pivoted_in(BgShared& S, int W) {
+  return S.B[((((W + 3) >> 2) & 1) ^ 1) ^ (W & 1)];
+}
+
+// Invert the W x W block in bg_pivoted_in (pitch kBgPitch) with partial pivoting into S.B[NP & 1]:
+// what cta_gj does, in the same order and rounding, so the same inverse.  Slices with a site
+// without dephasing take it.  A pivot's latency bounds it, so every warp finds the pivot for
+// itself, every thread forms the reciprocal and the exchanged rows as it reads them, and the
+// block is read from one buffer and written to the other: one barrier a pivot, where cta_gj has
+// five.  The columns are put in order on the way out.  Synchronised before and after; false
+// (uniformly) on a zero or non-finite pivot.  GB300, every third site undephased: with cta_gj
+// the W = 64 sweep's 640 threads took 7.5 ms at L = 60 (6.1 with 1024 threads before the panels).
+__device__ __forceinline__ bool bg_pivoted(BgShared& S, int W) {
+  const unsigned FULL = 0xffffffffu;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int j = tid % W, g = tid / W, G = blockDim.x / W;   // this thread's column and row group
+  cf* X = bg_pivoted_in(S, W);
+  cf* Y = X == S.B[0] ? S.B[1] : S.B[0];
+  for (int k = 0; k < W; ++k) {
+    // the row p >= k with the largest |a_pk|, the first of equals; non-negative floats order like
+    // their bits, and a NaN is never the largest
+    const int i0 = k + lane, i1 = i0 + 32;
+    const float v0 = i0 < W ? norm2(X[i0 * kBgPitch + k]) : 0.f;
+    const float v1 = i1 < W ? norm2(X[i1 * kBgPitch + k]) : 0.f;
+    const unsigned b0 = v0 > 0.f ? __float_as_uint(v0) : 0u, b1 = v1 > 0.f ? __float_as_uint(v1) : 0u;
+    const unsigned best = __reduce_max_sync(FULL, b0 > b1 ? b0 : b1);
+    const unsigned at0 = __ballot_sync(FULL, b0 == best), at1 = __ballot_sync(FULL, b1 == best);
+    if (best == 0u || best >= 0x7f800000u) return false;    // zero, infinite or no number at all
+    const int p = at0 ? k + __ffs(at0) - 1 : k + 32 + __ffs(at1) - 1;
+    if (tid == 0) S.perm[k] = p;
+    const cf inv = cdiv(cf{1.f, 0.f}, X[p * kBgPitch + k]);
+    if (!finite_c(inv)) return false;
+    if (g < G) {
+      const cf t = j == k ? inv : bg_mul(X[p * kBgPitch + j], inv);        // a_kj / a_kk
+      for (int i = g; i < W; i += G) {
+        const int from = i == p ? k : i;                    // rows k and p exchanged
+        const cf f = X[from * kBgPitch + k];
+        cf v;
+        if (i == k) v = t;
+        else if (j == k) v = bg_col(f, inv);
+        else v = bg_sub(X[from * kBgPitch + j], f, t);
+        Y[i * kBgPitch + j] = v;
+      }
+    }
+    __syncthreads();
+    cf* const Z = X;
+    X = Y;
+    Y = Z;
+  }
+  // the exchanges of rows undone as exchanges of columns, in reverse order: column j goes to `at`
+  if (g < G) {
+    int at = j;
+    for (int k = W - 1; k >= 0; --k) {
+      const int p = S.perm[k];
+      at = at == k ? p : at == p ? k : at;
+    }
+    for (int i = g; i < W; i += G) Y[i * kBgPitch + at] = X[i * kBgPitch + j];
+  }
+  __syncthreads();
+  return true;
+}
+
 // Form a slice's block, entry (i, c) = form(i, c), and invert it; the inverse is in S.B[NP & 1] on
 // return (synchronised), false (uniformly) on a pivot without a finite reciprocal.  form may
 // read entry (i, c) of the block before, which is in S.B[NP & 1].  pivot: partial pivoting (the
@@ -320,17 +383,12 @@ __device__ __forceinline__ bool bg_slice(BgShared& S, int turn, int W, bool pivo
     bg_invert<NH>(S, turn, W, v, f, inv, side);
     return !S.bad[turn];
   }
-  cf* A = S.B[(NP & 1) ^ 1];
-  cf* Bg = S.B[NP & 1];
-  for (int idx = tid; idx < W * W; idx += blockDim.x) A[idx] = form(idx / W, idx % W);
+  cf* A = bg_pivoted_in(S, W);
+  for (int idx = tid; idx < W * W; idx += blockDim.x)
+    A[idx / W * kBgPitch + idx % W] = form(idx / W, idx % W);
   side();
   __syncthreads();
-  cf* rowk = reinterpret_cast<cf*>(S.F);
-  if (!cta_gj(A, rowk, rowk + 64, S.perm, S.flag, W, true)) return false;
-  __syncthreads();
-  for (int idx = tid; idx < W * W; idx += blockDim.x) Bg[(idx / W) * kBgPitch + idx % W] = A[idx];
-  __syncthreads();
-  return true;
+  return bg_pivoted(S, W);
 }
 
 }  // namespace

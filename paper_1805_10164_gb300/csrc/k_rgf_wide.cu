@@ -1,6 +1,6 @@
 // RGF sweeps and diagonal blocks of complex64 wires wider than 16 sites (Sec. III.B), one CTA
-// per sweep or diagonal block, the W x W inversions by gj_blocked.cuh on slices where every
-// site dephases and by the pivoted cta_gj on the others.
+// per sweep or diagonal block, the W x W inversions by gj_blocked.cuh: panels on slices where
+// every site dephases, partial pivoting on the others.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -114,24 +114,17 @@ __global__ void __launch_bounds__(kBgThreads<NH>) rgf_sweep_wide_kernel(
       }
     } else {
       // a site without dephasing: partial pivoting on the block in shared memory
-      cf* A = S.B[(NP & 1) ^ 1];
+      cf* A = bg_pivoted_in(S, W);
       for (int idx = tid; idx < WW; idx += nth) {
         const int i = idx / W, c = idx - i * W;
-        A[idx] = form(s, i, c, gdst);
+        A[i * kBgPitch + c] = form(s, i, c, gdst);
       }
       fetch_diag(s + 1);
       __syncthreads();
-      cf* rowk = reinterpret_cast<cf*>(S.F);
-      if (!cta_gj(A, rowk, rowk + 64, S.perm, S.flag, W, true)) {
+      if (!bg_pivoted(S, W)) {
         if (tid == 0) atomicOr(err, ERR_SINGULAR);
         return;
       }
-      __syncthreads();
-      for (int idx = tid; idx < WW; idx += nth) {
-        const int i = idx / W, c = idx - i * W;
-        Bg[i * kBgPitch + c] = A[idx];
-      }
-      __syncthreads();
     }
   }
   cf* gdst = out + (uint64_t)(dir == 0 ? L - 2 : 1) * WW;
@@ -225,22 +218,16 @@ __global__ void __launch_bounds__(kBgThreads<NH>, 1) diag_wide_kernel(
       return;
     }
   } else {
+    cf* A = bg_pivoted_in(S, W);
     for (int idx = tid; idx < WW; idx += nth) {
       const int i = idx / W, c = idx - i * W;
-      T[idx] = form(i, c);
+      A[i * kBgPitch + c] = form(i, c);
     }
     __syncthreads();
-    cf* rowk = reinterpret_cast<cf*>(S.F);
-    if (!cta_gj(T, rowk, rowk + 64, S.perm, S.flag, W, true)) {
+    if (!bg_pivoted(S, W)) {
       if (tid == 0) atomicOr(err, ERR_SINGULAR);
       return;
     }
-    __syncthreads();
-    for (int idx = tid; idx < WW; idx += nth) {
-      const int i = idx / W, c = idx - i * W;
-      G[i * kBgPitch + c] = T[idx];
-    }
-    __syncthreads();
   }
   // start block: G_mm, or G_mm Phi for the injection columns
   cf* dst = start + d.start_off + (uint64_t)y * WW;
