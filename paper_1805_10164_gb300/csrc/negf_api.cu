@@ -237,11 +237,28 @@ bool band_edge(double E, int W, double t) {
   return false;
 }
 
-// Walkers per lane of a walk launch when no tuning picked them: two when the launch has
-// two-level tables (tables far larger than L2, two dependent gathers per transition: more
-// walks in flight hide more of the latency), one otherwise (L2-resident one-level tables and
-// short walks, where the start and refill work of a second walker costs more than it hides).
-int walk_slots(bool any_two) { return any_two ? 2 : 1; }
+// Walkers per lane of the launch that walks tasks d[0 .. n) when no tuning picked them.  One-level
+// tables (in L2, short walks): one, since the start and refill work of a second costs more than
+// it hides.  Two-level tables: two (three dependent gathers per transition in flight twice, at
+// three CTAs an SM) while lanes are few or the tables far larger than L2, one (at four CTAs)
+// where every lane of four CTAs has 45 walkers (it takes runs of 32) and the tables are at most
+// 2 GB, or the slices so narrow (W <= 4) that a transition is two gathers.  GB300, kernel ms, two
+// against one: W=64 x L=64, 8 energies, 1.6e6 walkers 0.30, 0.36, 3.2e7 1.52, 1.46; W=64 x L=40 at
+// eta = 0.005 (1.1 steps a walk), 3.2e7 0.77, 0.72 (two, slot after slot at four CTAs, 0.69);
+// W=16 x L=150, 16 energies, 1.6e7 1.75, 1.61; W=24 x L=150, 32 energies (2.2 GB), 3.2e7 3.07, 3.37; W=4 x L=600,
+// 8 energies, 1.6e6 9.0, 7.4; W=2 x L=1100, 4 energies, 4e6 63, 44.
+int walk_slots(const TaskDesc* d, int n, uint64_t walkers_per_task, int sm_count) {
+  int W = 0;
+  double bytes = 0.0;
+  for (int k = 0; k < n; ++k)
+    if (d[k].layout == NEGF_LAYOUT_TWO_LEVEL) {
+      W = std::max(W, d[k].W);
+      bytes += (double)d[k].rows * (4.0 * d[k].L * negf::level2_words(d[k].W) + 8.0 * (d[k].L + 2));
+    }
+  if (W <= 4) return 1;
+  const double full = 45.0 * 4 * 256 * sm_count;
+  return (double)n * (double)walkers_per_task >= full && bytes <= 2.0 * (1u << 30) ? 1 : 2;
+}
 
 }  // namespace
 
@@ -1205,7 +1222,9 @@ negf_status negf_run(negf_ctx ctx, const negf_wire* wires, int32_t n_wires,
                             r.walkers_per_task, r.walker_id_offset, r.max_steps, ctx->d_counter,
                             tl->d_counts + (size_t)wv.t0 * NEGF_TALLY_FIELDS, nullptr, nullptr,
                             nullptr, 0, nullptr, 0, ctx->sm_count, r.walk_blocks_per_sm, sw,
-                            nullptr, walk_slots(wv.any_two), wv.any_two);
+                            nullptr,
+                            walk_slots(wv.desc.data(), wv.t1 - wv.t0, r.walkers_per_task, ctx->sm_count),
+                            wv.any_two);
     }
     cudaFreeAsync(d_tab, sw);
     cudaEventRecord(walked[w], sw);
@@ -1445,7 +1464,8 @@ negf_status negf_walk(negf_ctx ctx, negf_tables t, int32_t start_lead, uint64_t 
     e = negf::launch_walk(t->d_tasks, 0, t->n_tasks, 0, t->d_tab, t->d_mode_tab, t->d_c,
                           start_lead, seed, walkers_per_task, walker_id_offset, max_steps,
                           ctx->d_counter, tl->d_counts, nullptr, nullptr, nullptr, 0, nullptr,
-                          0, ctx->sm_count, 0, ctx->stream, nullptr, walk_slots(t->any_two),
+                          0, ctx->sm_count, 0, ctx->stream, nullptr,
+                          walk_slots(t->h_tasks.data(), t->n_tasks, walkers_per_task, ctx->sm_count),
                           t->any_two);
   }
   if (e != cudaSuccess) {
@@ -1611,7 +1631,8 @@ negf_status negf_walk_trace(negf_ctx ctx, negf_tables t, int32_t task, int32_t s
     e = negf::launch_walk(t->d_tasks, task, 1, 0, t->d_tab, t->d_mode_tab, t->d_c, start_lead,
                           seed, n_walkers, walker_id_offset, max_steps, ctx->d_counter, tmp,
                           d_lead, d_steps, nullptr, 0, nullptr, 0, ctx->sm_count, 0,
-                          ctx->stream, nullptr, walk_slots(t->any_two), t->any_two);
+                          ctx->stream, nullptr,
+                          walk_slots(t->h_tasks.data() + task, 1, n_walkers, ctx->sm_count), t->any_two);
   cudaFreeAsync(tmp, ctx->stream);
   if (e != cudaSuccess) return fail(ctx, NEGF_E_CUDA, "negf_walk_trace: %s", cudaGetErrorString(e));
   return NEGF_OK;
@@ -2506,8 +2527,10 @@ negf_status plan_enqueue(negf_plan p, bool timed, cudaStream_t s) {
                                       p->d_counts + (size_t)wv.t0 * NEGF_TALLY_FIELDS, nullptr,
                                       nullptr, nullptr, 0, nullptr, 0, ctx->sm_count,
                                       p->tune.walk_blocks_per_sm, ws, p->d_run,
-                                      p->tune.walk_slots > 0 ? p->tune.walk_slots
-                                                             : walk_slots(wv.any_two),
+                                      p->tune.walk_slots > 0
+                                          ? p->tune.walk_slots
+                                          : walk_slots(wv.desc.data(), ntw, p->run.walkers_per_task,
+                                                       ctx->sm_count),
                                       wv.any_two));
     }
     if (split) CUDA_TRY(ctx, cudaEventRecord(walked, sw));
@@ -2623,11 +2646,13 @@ negf_status plan_autotune(negf_plan p) {
   const uint64_t h_run[2] = {0x5eedull, 0ull};
   CUDA_TRY(ctx, cudaMemcpyAsync(p->d_run, h_run, sizeof h_run, cudaMemcpyHostToDevice, s));
   CUDA_TRY(ctx, cudaStreamSynchronize(s));
-  // (walkers per lane, CTAs per SM): two walkers per lane fit four CTAs per SM
+  // (walkers per lane, CTAs per SM); with two-level tables four CTAs fit at one walker per lane
+  // and three at two, otherwise five and four
   int best_ws = 1;
   const int cand[][2] = {{1, 2}, {1, 3}, {1, 4}, {1, 5}, {2, 2}, {2, 3}, {2, 4}};
   for (const auto& c : cand) {
     const int ws = c[0], wb = c[1];
+    if (wv.any_two && ws + wb > 5) continue;         // more CTAs than fit
     const float ms = time_on(s, 2, [&]() {
       return negf::launch_walk(dd, 0, nt0, (uint32_t)wv.t0, p->d_tab[0], q.d_mode_tab, q.d_c,
                                p->run.start_lead, 0, p->run.walkers_per_task, 0,
