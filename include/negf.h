@@ -240,7 +240,9 @@ void negf_tally_free(negf_tally tally);
 typedef struct {
   int32_t start_lead;          /* 0 = L, 1 = R (as in negf_walk) */
   int32_t tasks_per_wave;      /* tasks built per wave; 0 = up to eight waves, each with block
-                                  columns enough to fill the device a few times */
+                                  columns enough to fill the device a few times: a small batch
+                                  is one wave, all of its tables and scratch held at once
+                                  (memory_budget still bounds them) */
   uint64_t seed;
   uint64_t walkers_per_task;
   uint64_t walker_id_offset;

@@ -19,8 +19,8 @@
 // (5 L for the column s_p), against the n^3 of the dense adjoint product; its memory is two
 // block columns per CTA in flight.
 //
-// Checkpoints (ckpt_stride s): adj_sweep_kernel runs both RGF sweeps of every task once and keeps
-// only every s-th block (left: g^L_k at k = 0, s, 2s, ...; right: g^R_k at k = L-1, L-1-s, ...).
+// Checkpoints (ckpt_stride s): adj_sweep_kernel (complex128) or adj_sweep32_kernel (complex64, panel
+// inversions) runs both RGF sweeps of every task once and keeps only every s-th block (left: g^L_k at k = 0, s, 2s, ...; right: g^R_k at k = L-1, L-1-s, ...).
 // Before a group of tasks runs its columns, adj_expand_kernel recomputes the blocks between
 // checkpoints, one CTA per segment of s slices (s serial inversions each, the segments in
 // parallel), into buffers that live only while that group's columns run.  The kept blocks take
@@ -80,24 +80,23 @@ __device__ __forceinline__ bool slice_dephased(const double* eta, int k, int W) 
   return __syncthreads_and(threadIdx.x >= W || eta[k * W + threadIdx.x] > 0.0);
 }
 
-// ---- checkpointed sweeps: one CTA per (task, direction) --------------------------------------
+// ---- checkpointed sweeps, complex128: one CTA per (task, direction) --------------------------
 // Left (dir 0): k = 0 .. L-1, the last block the full G_{L-1,L-1} (right lead included).
 // Right (dir 1): k = L-1 .. 1.  Kept: every s-th block of each direction, at ck + task's
 // offset + (index along the sweep / s) W^2.
-template <typename C>
 __global__ void __launch_bounds__(kAdjThreads) adj_sweep_kernel(
     const TaskDesc* __restrict__ tasks, int n_tasks, const double* __restrict__ wire,
     const double* __restrict__ phig, const cd* __restrict__ sig,
-    const uint64_t* __restrict__ ck_off, int s, C* __restrict__ ck, int32_t* __restrict__ err) {
+    const uint64_t* __restrict__ ck_off, int s, cd* __restrict__ ck, int32_t* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int job = blockIdx.x;
   if (job >= 2 * n_tasks) return;
   const int task = job >> 1, dir = job & 1;
   const TaskDesc d = tasks[task];
   const int W = d.W, L = d.L, WW = W * W;
-  C* A = reinterpret_cast<C*>(smem_raw);
-  C* rowk = A + WW;
-  C* fcol = rowk + W;
+  cd* A = reinterpret_cast<cd*>(smem_raw);
+  cd* rowk = A + WW;
+  cd* fcol = rowk + W;
   int* perm = reinterpret_cast<int*>(fcol + W);
   int* flag = perm + W;
   const double* onsite = wire + d.onsite_off;
@@ -105,7 +104,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_sweep_kernel(
   const double* phi = phig + d.phi_off;
   const cd* sg = sig + d.lead_off;
   const int nck = (L + s - 1) / s;
-  C* out = ck + ck_off[task] + (uint64_t)dir * nck * WW;
+  cd* out = ck + ck_off[task] + (uint64_t)dir * nck * WW;
   const int steps = dir == 0 ? L : L - 1;
   for (int i = 0; i < steps; ++i) {
     const int k = dir == 0 ? i : L - 1 - i;
@@ -117,7 +116,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_sweep_kernel(
       return;
     }
     if (i % s == 0) {
-      C* dst = out + (uint64_t)(i / s) * WW;
+      cd* dst = out + (uint64_t)(i / s) * WW;
       for (int idx = threadIdx.x; idx < WW; idx += blockDim.x) dst[idx] = A[idx];
     }
     __syncthreads();
@@ -907,10 +906,10 @@ cudaError_t launch_adjoint_sweep(const TaskDesc* d_tasks, int n_tasks, int max_W
   if (n_tasks == 0) return cudaSuccess;
   if (precision == NEGF_FP64) {
     const size_t smem = gj_smem<cd>(max_W);
-    cudaError_t e = cudaFuncSetAttribute(adj_sweep_kernel<cd>,
+    cudaError_t e = cudaFuncSetAttribute(adj_sweep_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    adj_sweep_kernel<cd><<<2 * n_tasks, kAdjThreads, smem, s>>>(
+    adj_sweep_kernel<<<2 * n_tasks, kAdjThreads, smem, s>>>(
         d_tasks, n_tasks, d_wire, d_phi, d_sig, d_ck_off, stride, static_cast<cd*>(d_ck), d_err);
   } else {
     // widths up to 32 and above by kernels of their own; each skips the other's tasks

@@ -11,9 +11,9 @@
 // (w_e' K(E_e' - E_e) A_jj(E_e'), the model's lambda~ of Eq. condition4_buttiker).  A draw with
 // words (x, y) over a K-entry row takes c = (x K) >> 32 and keeps c if y < thr[c], else
 // alias[c].  Drawing a lead ends the walk; its count goes to the injection task, so that
-// T_qp(E_0) = c_p(E_0) P(q | p, E_0) as for elastic walks.  One walker per thread over a
-// persistent grid; counts per task in shared memory (tasks of the launch window), added to the
-// global tally once per block.
+// T_qp(E_0) = c_p(E_0) P(q | p, E_0) as for elastic walks.  Warps take chunks of consecutive
+// walkers and refill their lanes from them (below); counts per task in a lane's registers, then
+// in shared memory (tasks of the launch window), added to the global tally once per block.
 #include <cuda_runtime.h>
 
 #include "negf_internal.cuh"

@@ -1147,7 +1147,7 @@ cudaError_t sweep_fp32(const TaskDesc* d_tasks, int n_tasks, int max_W, const do
 template <typename C>
 cudaError_t columns_impl(const TaskDesc* d_tasks, int n_tasks, uint32_t n_cols, int max_W,
                          const double* d_wire, const typename Real<C>::T* d_eta,
-                         const double* d_phi, const typename Real<C>::T* d_phiR, const cd* d_sig,
+                         const double* d_phi, const typename Real<C>::T* d_phiR,
                          const double* d_gam, const C* d_gL, const C* d_gR, C* d_start,
                          typename Real<C>::T* d_w, double* d_rowsum, double* d_mode_w,
                          double* d_c, int32_t* d_err, C* d_green, C* d_gphi, cudaStream_t s,
@@ -1248,7 +1248,7 @@ cudaError_t launch_rgf_sweep(const TaskDesc* d_tasks, int n_tasks, int max_W, in
 cudaError_t launch_block_columns(const TaskDesc* d_tasks, int n_tasks, uint32_t n_cols,
                                  int max_W, int precision, const double* d_wire,
                                  const float* d_eta32, const double* d_phi, const float* d_phi32,
-                                 const cd* d_sig, const double* d_gam, const void* d_gL,
+                                 const double* d_gam, const void* d_gL,
                                  const void* d_gR, void* d_start, void* d_weights,
                                  double* d_rowsum, double* d_mode_w, double* d_c, int32_t* d_err,
                                  void* d_green, void* d_gphi, cudaStream_t s, int chain_warps,
@@ -1256,14 +1256,14 @@ cudaError_t launch_block_columns(const TaskDesc* d_tasks, int n_tasks, uint32_t 
   if (n_tasks == 0 || n_cols == 0) return cudaSuccess;
   if (cols_max_W < 0) cols_max_W = max_W;
   if (precision == NEGF_FP64)
-    return columns_impl<cd>(d_tasks, n_tasks, n_cols, max_W, d_wire, d_wire, d_phi, d_phi,
-                            d_sig, d_gam, static_cast<const cd*>(d_gL),
+    return columns_impl<cd>(d_tasks, n_tasks, n_cols, max_W, d_wire, d_wire, d_phi, d_phi, d_gam,
+                            static_cast<const cd*>(d_gL),
                             static_cast<const cd*>(d_gR), static_cast<cd*>(d_start),
                             static_cast<double*>(d_weights), d_rowsum, d_mode_w, d_c, d_err,
                             static_cast<cd*>(d_green), static_cast<cd*>(d_gphi), s,
                             chain_warps, cols_max_W);
-  return columns_impl<cf>(d_tasks, n_tasks, n_cols, max_W, d_wire, d_eta32, d_phi, d_phi32,
-                          d_sig, d_gam, static_cast<const cf*>(d_gL),
+  return columns_impl<cf>(d_tasks, n_tasks, n_cols, max_W, d_wire, d_eta32, d_phi, d_phi32, d_gam,
+                          static_cast<const cf*>(d_gL),
                           static_cast<const cf*>(d_gR), static_cast<cf*>(d_start),
                           static_cast<float*>(d_weights), d_rowsum, d_mode_w, d_c, d_err,
                           static_cast<cf*>(d_green), static_cast<cf*>(d_gphi), s,

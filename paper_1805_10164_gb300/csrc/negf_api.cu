@@ -691,18 +691,22 @@ uint64_t wave_bytes(const Wave& w, int prec) {
   return w.tab * 8 + (w.wt + w.l1w) * wsz + w.start * cb + 8ull * w.rows + 8ull * w.edge;
 }
 
-// Tasks per wave of negf_run when the caller leaves it open: up to eight waves (so that walks
-// overlap the next wave's build), but none so small that its block columns leave SMs idle.  A
-// task's block columns are counted against what the device holds at once (per SM two columns
-// of W > 32: one CTA of a column pair; eight of 16 < W <= 32: four CTAs; about 96 of W <= 16:
-// one-warp CTAs of up to three columns), and a wave gets at least four such fillings, so that
-// its last, partly empty round is a small share.  Measured (GB300, ms per call, an eighth of the
-// tasks per wave against one wave): W=64 x L=100, 8 energies 28.5 -> 11.1, 32 energies
-// 29.7 -> 21.1; W=40 x L=50, 16 tasks 28.0 -> 12.8; W=32 x L=100, 32 energies 12.9 -> 8.4;
-// W=10 x L=50, 64 energies 2.50 -> 1.78 (FP64 13.9 -> 6.6).  Batches whose eighths fill the
-// device several times over keep them: 1280 uneven tasks 271 (eighths) against 276 (one wave).
-// Batches of W <= 16 beside 32 < W < 64 keep them too: which of the two shares a wave with the
-// other decides the narrow tasks' last bits (make_wave).
+// Tasks per wave of negf_run when the caller leaves it open: up to eight waves, but none so small
+// that its block columns leave SMs idle.  A task's block columns are counted against what an SM
+// holds at once - two of W > 32 (one W = 64 CTA of a column pair), eight of 16 < W <= 32 (four
+// CTAs), about 96 of W <= 16 (one-warp CTAs of up to three columns) - and a wave gets at least four
+// such fillings, so that its last, partly empty round is a small share.  FP64 columns are counted
+// alike although fewer fit (a warp each: about 24 at W = 10, one at W = 64), and 32 < W < 64 holds
+// four: both get larger waves than the count would give them, which costs no time, since a wave's
+// walk takes every SM and its neighbours' builds run before or after it rather than beside it.
+// Measured (GB300, ms per call, eighths / this rule / one wave): W=64 x L=100, 8 energies 17.6 / 6.5
+// / 6.5, 32 energies 21.6 / 16.4 / 16.0; W=40 x L=50, 16 energies 6.2 / 3.1 / 3.1, 256 energies 36.6 /
+// 36.6 / 36.7; W=32 x L=100, 32 energies 10.0 / 6.9 / 6.9; W=24 x L=60, 128 energies 8.8 / 8.5 / 8.5;
+// W=10 x L=50, 64 energies 2.33 / 1.60 / 1.60, 512 energies 6.15 / 5.41 / 5.42; FP64 W=10 x L=50,
+// 512 energies 21.7 / 18.9 / 18.9, W=16 x L=60, 256 energies 40.2 / 33.4 / 33.3, W=32 x L=20, 128
+// energies 38.1 / 22.1 / 22.1.  W=4 x L=50, 1024 energies 3.44 / 3.57 / 3.57.
+// Batches of W <= 16 beside 32 < W < 64 take eighths: which of the two shares a wave with the other
+// decides the narrow tasks' last bits (make_wave).
 int default_per_wave(const Plan& P, int sm_count) {
   const int nt = (int)P.tasks.size();
   double fill = 0.0;
@@ -873,7 +877,7 @@ negf_status build_wave(negf_ctx ctx, cudaStream_t s, const Plan& P, const Wave& 
     ProfScope ps(ctx, "diag_chain_kernels", 2, s);
     e = negf::launch_block_columns(d_wdesc, nt, w.cols, P.max_W, prec, q.d_wire, q.d_eta32,
                                    q.d_phi, reinterpret_cast<float*>(q.d_phi + P.phi_total),
-                                   q.d_sig, q.d_gam, d_gL, d_gR, d_start, d_weights, d_rowsum,
+                                   q.d_gam, d_gL, d_gR, d_start, d_weights, d_rowsum,
                                    q.d_mode_w, q.d_c + 2 * (size_t)w.t0, q.d_err, d_green,
                                    d_gphi, s, chain_warps, w.cols_max_W);
   }
@@ -2479,7 +2483,7 @@ negf_status plan_enqueue(negf_plan p, bool timed, cudaStream_t s) {
       SegScope sg(p, "diag_chain_kernels", 2, s, timed);
       CUDA_TRY(ctx, negf::launch_block_columns(
                         dd, ntw, wv.cols, P.max_W, prec, q.d_wire, q.d_eta32, q.d_phi,
-                        reinterpret_cast<float*>(q.d_phi + P.phi_total), q.d_sig, q.d_gam,
+                        reinterpret_cast<float*>(q.d_phi + P.phi_total), q.d_gam,
                         p->d_gL, p->d_gR, p->d_start[slot], p->d_weights[slot], p->d_rs[slot],
                         q.d_mode_w, q.d_c + 2 * (size_t)wv.t0, q.d_err, nullptr, nullptr, s,
                         p->tune.chain_warps, wv.cols_max_W));
@@ -2587,7 +2591,7 @@ negf_status plan_autotune(negf_plan p) {
   auto columns = [&](int cw) {
     return negf::launch_block_columns(dd, nt0, wv.cols, P.max_W, prec, q.d_wire, q.d_eta32,
                                       q.d_phi, reinterpret_cast<float*>(q.d_phi + P.phi_total),
-                                      q.d_sig, q.d_gam, p->d_gL, p->d_gR, p->d_start[0],
+                                      q.d_gam, p->d_gL, p->d_gR, p->d_start[0],
                                       p->d_weights[0], p->d_rs[0], q.d_mode_w, q.d_c, q.d_err,
                                       nullptr, nullptr, s, cw, wv.cols_max_W);
   };

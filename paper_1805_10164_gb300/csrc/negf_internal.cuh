@@ -141,7 +141,7 @@ cudaError_t launch_chain_cols(const TaskDesc* d_tasks, int n_tasks, uint32_t n_j
 cudaError_t launch_block_columns(const TaskDesc* d_tasks, int n_tasks, uint32_t n_cols,
                                  int max_W, int precision, const double* d_wire,
                                  const float* d_eta32, const double* d_phi, const float* d_phi32,
-                                 const cd* d_sig, const double* d_gam, const void* d_gL,
+                                 const double* d_gam, const void* d_gL,
                                  const void* d_gR, void* d_start, void* d_weights,
                                  double* d_rowsum, double* d_mode_w, double* d_c, int32_t* d_err,
                                  void* d_green, void* d_gphi, cudaStream_t s,

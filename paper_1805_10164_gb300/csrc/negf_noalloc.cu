@@ -187,7 +187,7 @@ extern "C" negf_status negf_build_tables_noalloc(const negf_wire* wire, int32_t 
                                s);
   if (e == cudaSuccess)
     e = negf::launch_block_columns(d_tasks, nt, (uint32_t)(nt * (wr.L + 2)), wr.W, prec, d_wire,
-                                   d_eta32, d_phi, d_phi32, d_sig, d_gam, d_gL, d_gR, d_st, d_w,
+                                   d_eta32, d_phi, d_phi32, d_gam, d_gL, d_gR, d_st, d_w,
                                    d_rs, d_mw, d_c, d_err, nullptr, nullptr, s, 0,
                                    cta ? 0 : wr.W);
   if (e == cudaSuccess && cta)
