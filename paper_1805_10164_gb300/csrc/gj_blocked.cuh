@@ -80,8 +80,9 @@ struct BgShared {
   cf diag[2][64];               // diagonal of E - H - Sigma_s of a slice
   int undephased[2][2];         // nonzero: the slice (half of it) has a site without dephasing
   int perm[64];                 // pivoted inversions
-  int bad[2];                   // a pivot without a finite reciprocal, inversions in turn: a warp
-                                // may still read one's flag while the next one's panel is made
+  int bad;                      // some inversion met a pivot without a finite reciprocal: read it
+                                // after the last one only (warp 0 may set it in the next one's
+                                // first panel while other warps leave this one)
 };
 
 __device__ __forceinline__ void bg_put4(float4* dst, const cf (&v)[4]) {
@@ -104,12 +105,11 @@ __device__ __forceinline__ void bg_panel_sync() {
 
 // Panel warps: eliminate the nb pivots k1 .. k1 + nb - 1 within the panel's columns v of this
 // lane's row, leaving the pivot columns in f and the reciprocals in inv; publishes them in
-// buffer buf and the panel's columns, now as after these pivots, in Bout.  turn: 0, 1, 0, ... over
-// the inversions, the flag S.bad[turn] is this one's.
+// buffer buf and the panel's columns, now as after these pivots, in Bout.
 // kFull: nb = 4 (every panel but perhaps the last), without branches between the pivots.
 template <int NH, bool kFull>
-__device__ __forceinline__ void bg_factor(BgShared& S, int turn, int k1, int nb, int buf,
-                                          cf* Bout, cf (&v)[4], cf (&f)[4], cf (&inv)[4]) {
+__device__ __forceinline__ void bg_factor(BgShared& S, int k1, int nb, int buf, cf* Bout,
+                                          cf (&v)[4], cf (&f)[4], cf (&inv)[4]) {
   const int row = threadIdx.x;                      // panel warps are warps 0 .. NH - 1
   const int own = row - k1;                         // 0 .. 3: this lane's row is pivot row `own`
   if ((unsigned)own < 4u) bg_put4(S.blk[own], v);
@@ -155,18 +155,18 @@ __device__ __forceinline__ void bg_factor(BgShared& S, int turn, int k1, int nb,
   if (row == 0) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) S.inv[buf][q] = inv[q];
-    if (bad) S.bad[turn] = 1;
+    if (bad) S.bad = 1;
   }
 }
 
 // Invert the block.  On entry the columns >= 4 are in S.B[0], panel 0 has been eliminated by
 // bg_factor (buffer 0, columns in S.B[1]; the panel warps' f and inv from it), and the CTA has
 // synchronised.  On return (synchronised) the inverse is in S.B[NP & 1], NP = ceil(W / 4);
-// S.bad[turn] is set if some pivot had no finite reciprocal, and not written again before the
-// inversion after the next.  side() is called by the warps without rows during panel 0.
+// S.bad is set (and stays so) if some pivot had no finite reciprocal; the inverse then holds no
+// numbers.  side() is called by the warps without rows during panel 0.
 template <int NH, typename Side>
-__device__ __forceinline__ void bg_invert(BgShared& S, int turn, int W, cf (&v)[4], cf (&f)[4],
-                                          cf (&inv)[4], Side side) {
+__device__ __forceinline__ void bg_invert(BgShared& S, int W, cf (&v)[4], cf (&f)[4], cf (&inv)[4],
+                                          Side side) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int unit = bg_unit<NH>(warp);
   const int j = NH == 2 ? (unit & 1) * 32 + lane : lane;
@@ -212,8 +212,8 @@ __device__ __forceinline__ void bg_invert(BgShared& S, int turn, int W, cf (&v)[
             v[c] = row == k0 + q ? tq[c] : n;
           }
         }
-        if (W - k1 >= 4) bg_factor<NH, true>(S, turn, k1, 4, b ^ 1, X, v, f, inv);
-        else bg_factor<NH, false>(S, turn, k1, W - k1, b ^ 1, X, v, f, inv);
+        if (W - k1 >= 4) bg_factor<NH, true>(S, k1, 4, b ^ 1, X, v, f, inv);
+        else bg_factor<NH, false>(S, k1, W - k1, b ^ 1, X, v, f, inv);
       }
     } else if (unit >= 0) {
       const int nb = min(4, W - k0);
@@ -297,8 +297,10 @@ __device__ __forceinline__ cf* bg_pivoted_in(BgShared& S, int W) {
 // itself, every thread forms the reciprocal and the exchanged rows as it reads them, and the
 // block is read from one buffer and written to the other: one barrier a pivot, where cta_gj has
 // five.  The columns are put in order on the way out.  Synchronised before and after; false
-// (uniformly) on a zero or non-finite pivot.  GB300, every third site undephased: with cta_gj
-// the W = 64 sweep's 640 threads took 7.5 ms at L = 60 (6.1 with 1024 threads before the panels).
+// (uniformly) on a zero or non-finite pivot.  GB300, every third site undephased, sweeps: W=64 x
+// L=100, 8 energies 12.7 -> 7.4 ms, W=40 x L=50, 16 energies 2.67 -> 1.46, W=32 x L=100, 32 energies
+// 3.99 -> 1.94 (cta_gj by the panels' 640 or 384 threads was slower than by the 1024 threads that
+// sweeps had before the panels: W=64 x L=60 6.1 ms against 7.5).
 __device__ __forceinline__ bool bg_pivoted(BgShared& S, int W) {
   const unsigned FULL = 0xffffffffu;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -350,16 +352,15 @@ __device__ __forceinline__ bool bg_pivoted(BgShared& S, int W) {
 }
 
 // Form a slice's block, entry (i, c) = form(i, c), and invert it; the inverse is in S.B[NP & 1] on
-// return (synchronised), false (uniformly) on a pivot without a finite reciprocal.  form may
-// read entry (i, c) of the block before, which is in S.B[NP & 1].  pivot: partial pivoting (the
-// slice has a site without dephasing).  side() is called by the warps without columns.  turn:
-// alternates over a CTA's inversions (bg_factor).
+// return (synchronised).  form may read entry (i, c) of the block before, which is in S.B[NP & 1].
+// pivot: partial pivoting (the slice has a site without dephasing); false (uniformly) if a pivot
+// then has no finite reciprocal, without pivoting see S.bad.  side() is called by the warps without
+// columns.
 template <int NH, typename Form, typename Side>
-__device__ __forceinline__ bool bg_slice(BgShared& S, int turn, int W, bool pivot, Form form,
-                                         Side side) {
+__device__ __forceinline__ bool bg_slice(BgShared& S, int W, bool pivot, Form form, Side side) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NP = (W + 3) >> 2;
-  if (!pivot) {
+  if (__builtin_expect(!pivot, 1)) {
     const int unit = bg_unit<NH>(warp);
     const int j = NH == 2 ? (unit & 1) * 32 + lane : lane;
     const int g = NH == 2 ? unit >> 1 : unit;
@@ -370,8 +371,8 @@ __device__ __forceinline__ bool bg_slice(BgShared& S, int turn, int W, bool pivo
 #pragma unroll
       for (int c = 0; c < 4; ++c)
         if (tid < W && c < W) v[c] = form(tid, c);
-      if (W >= 4) bg_factor<NH, true>(S, turn, 0, 4, 0, S.B[1], v, f, inv);
-      else bg_factor<NH, false>(S, turn, 0, W, 0, S.B[1], v, f, inv);
+      if (W >= 4) bg_factor<NH, true>(S, 0, 4, 0, S.B[1], v, f, inv);
+      else bg_factor<NH, false>(S, 0, W, 0, S.B[1], v, f, inv);
     } else if (unit >= 0 && j >= 4 && j < W) {
 #pragma unroll
       for (int r = 0; r < 8; ++r) {
@@ -380,8 +381,8 @@ __device__ __forceinline__ bool bg_slice(BgShared& S, int turn, int W, bool pivo
       }
     }
     __syncthreads();
-    bg_invert<NH>(S, turn, W, v, f, inv, side);
-    return !S.bad[turn];
+    bg_invert<NH>(S, W, v, f, inv, side);
+    return true;
   }
   cf* A = bg_pivoted_in(S, W);
   for (int idx = tid; idx < W * W; idx += blockDim.x)

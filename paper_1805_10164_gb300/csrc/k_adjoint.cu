@@ -245,13 +245,13 @@ __global__ void __launch_bounds__(kBgThreads<NH>) adj_sweep32_kernel(
   const int steps = dir == 0 ? L : L - 1;
   auto slice = [&](int i) { return dir == 0 ? i : L - 1 - i; };
   if (steps > 0) sl.fetch(slice(0), 0);
-  if (threadIdx.x < 2) S.bad[threadIdx.x] = 0;
+  if (threadIdx.x == 0) S.bad = 0;
   __syncthreads();
   for (int i = 0; i < steps; ++i) {
     const int k = slice(i), b = i & 1;
     const int leads = (dir == 0 && k == 0 ? 1 : 0) + (k == L - 1 ? 1 : 0);
     const bool ok = bg_slice<NH>(
-        S, b, W, sl.pivots(b), [&](int r, int c) { return sl.entry(r, c, b, leads, i > 0); },
+        S, W, sl.pivots(b), [&](int r, int c) { return sl.entry(r, c, b, leads, i > 0); },
         [&] { if (i + 1 < steps) sl.fetch(slice(i + 1), b ^ 1); });
     if (!ok) {
       if (threadIdx.x == 0) atomicOr(err, ERR_SINGULAR);
@@ -264,6 +264,7 @@ __global__ void __launch_bounds__(kBgThreads<NH>) adj_sweep32_kernel(
       __syncthreads();
     }
   }
+  if (threadIdx.x == 0 && S.bad) atomicOr(err, ERR_SINGULAR);
 }
 
 // ---- block products ------------------------------------------------------------------------

@@ -33,7 +33,7 @@ __device__ __forceinline__ cf wide_diag(const TaskDesc& d, const double* onsite,
 // warps form columns >= 4 and the panel warp, from its own registers, the first panel, which
 // it then eliminates.  The next slice's diagonal is fetched by the two warps without columns.
 // Measured (GB300) against one pivot at a time with 1024 threads: W=64 x L=100, 8 energies 6.81 ->
-// 2.45 ms, W=64 x L=1000 66.7 -> 24.4 ms (24 us a slice); W=32 x L=100, 32 energies 1.83 -> 0.73 ms.
+// 2.41 ms, W=64 x L=1000 66.7 -> 24.0 ms (24 us a slice); W=32 x L=100, 32 energies 1.83 -> 0.73 ms.
 template <int NH>
 __global__ void __launch_bounds__(kBgThreads<NH>) rgf_sweep_wide_kernel(
     const TaskDesc* __restrict__ tasks, int n_tasks, const double* __restrict__ wire, cf* gL,
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(kBgThreads<NH>) rgf_sweep_wide_kernel(
     if (lane == 0) S.undephased[s & 1][dw] = any;
   };
   fetch_diag(0);
-  if (tid < 2) S.bad[tid] = 0;
+  if (tid == 0) S.bad = 0;
   __syncthreads();
   const cf* lb = gL + d.g_off + (uint64_t)(L - 1) * WW;   // the lead block (launch_lead_blocks)
   cf* out = (dir == 0 ? gL : gR) + d.g_off;
@@ -93,12 +93,14 @@ __global__ void __launch_bounds__(kBgThreads<NH>) rgf_sweep_wide_kernel(
   for (int c = 0; c < 4; ++c) v[c] = f[c] = inv[c] = cf{0.f, 0.f};
   for (int s = 0; s < L - 1; ++s) {
     cf* gdst = s > 0 ? out + (uint64_t)(dir == 0 ? s - 1 : L - s) * WW : nullptr;
-    if (!(S.undephased[s & 1][0] || (NH == 2 && S.undephased[s & 1][1]))) {
+    // (expected, so that the pivoted code is laid out behind the panels': 2.46 -> 2.41 ms at W=64 x
+    // L=100, 8 energies)
+    if (__builtin_expect(!(S.undephased[s & 1][0] || (NH == 2 && S.undephased[s & 1][1])), 1)) {
       if (warp < NH) {
 #pragma unroll
         for (int c = 0; c < 4; ++c)
           if (tid < W) v[c] = form(s, tid, c, gdst);
-        bg_factor<NH, true>(S, s & 1, 0, 4, 0, S.B[1], v, f, inv);
+        bg_factor<NH, true>(S, 0, 4, 0, S.B[1], v, f, inv);
       } else if (unit >= 0 && j >= 4 && j < W) {
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
@@ -107,11 +109,7 @@ __global__ void __launch_bounds__(kBgThreads<NH>) rgf_sweep_wide_kernel(
         }
       }
       __syncthreads();
-      bg_invert<NH>(S, s & 1, W, v, f, inv, [&] { fetch_diag(s + 1); });
-      if (S.bad[s & 1]) {
-        if (tid == 0) atomicOr(err, ERR_SINGULAR);
-        return;
-      }
+      bg_invert<NH>(S, W, v, f, inv, [&] { fetch_diag(s + 1); });
     } else {
       // a site without dephasing: partial pivoting on the block in shared memory
       cf* A = bg_pivoted_in(S, W);
@@ -135,6 +133,7 @@ __global__ void __launch_bounds__(kBgThreads<NH>) rgf_sweep_wide_kernel(
     bad |= !finite_c(x);
   }
   if (__syncthreads_or(bad) && tid == 0) atomicOr(err, ERR_NONFINITE);
+  if (tid == 0 && S.bad) atomicOr(err, ERR_SINGULAR);
 }
 
 // last task whose first job index is <= job
@@ -191,7 +190,7 @@ __global__ void __launch_bounds__(kBgThreads<NH>, 1) diag_wide_kernel(
     return cf{__fsub_rn(__fsub_rn(e.x, l.x), r.x), __fsub_rn(__fsub_rn(e.y, l.y), r.y)};
   };
   if (tid < W) S.diag[0][tid] = wide_diag(d, onsite, eta, h, m0, tid);
-  if (tid == 0) S.bad[0] = 0;
+  if (tid == 0) S.bad = 0;
   const bool deph = __syncthreads_and(tid >= W || eta[m0 * W + tid] > 0.0);
   cf* G = S.B[NP & 1];
   cf* T = S.B[(NP & 1) ^ 1];                              // free once the inverse is in G
@@ -203,7 +202,7 @@ __global__ void __launch_bounds__(kBgThreads<NH>, 1) diag_wide_kernel(
 #pragma unroll
       for (int c = 0; c < 4; ++c)
         if (tid < W) v[c] = form(tid, c);
-      bg_factor<NH, true>(S, 0, 0, 4, 0, S.B[1], v, f, inv);
+      bg_factor<NH, true>(S, 0, 4, 0, S.B[1], v, f, inv);
     } else if (unit >= 0 && j >= 4 && j < W) {
 #pragma unroll
       for (int r = 0; r < 8; ++r) {
@@ -212,8 +211,8 @@ __global__ void __launch_bounds__(kBgThreads<NH>, 1) diag_wide_kernel(
       }
     }
     __syncthreads();
-    bg_invert<NH>(S, 0, W, v, f, inv, [] {});
-    if (S.bad[0]) {
+    bg_invert<NH>(S, W, v, f, inv, [] {});
+    if (S.bad) {
       if (tid == 0) atomicOr(err, ERR_SINGULAR);
       return;
     }
