@@ -807,12 +807,6 @@ __global__ void __launch_bounds__(kAdjThreads, RT >= 2 ? 1 : (sizeof(C) == 8 ? 3
   }
 }
 
-template <typename K>
-cudaError_t bg_smem(K kernel) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(BgShared));
-}
-
 template <typename C>
 size_t gj_smem(int W) {
   return sizeof(C) * (size_t)(W * W + 2 * W) + sizeof(int) * (size_t)(W + 2);
@@ -832,8 +826,7 @@ template <typename C, int RT, int RTN>
 cudaError_t columns_rt(const AdjArgs& a, int W, const C* gl, const C* gr, C* psi, C* tl, C* xs,
                        C* ys, int slots, cudaStream_t s) {
   const size_t smem = column_smem<C>(W);
-  cudaError_t e = cudaFuncSetAttribute(adj_column_kernel<C, RT, RTN>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(adj_column_kernel<C, RT, RTN>);
   if (e != cudaSuccess) return e;
   adj_column_kernel<C, RT, RTN><<<slots, kAdjThreads, smem, s>>>(a, gl, gr, psi, tl, xs, ys);
   return cudaGetLastError();
@@ -843,9 +836,7 @@ cudaError_t columns_rt(const AdjArgs& a, int W, const C* gl, const C* gr, C* psi
 template <typename C, int RT, int RTN>
 int occupancy_rt(int W) {
   const size_t smem = column_smem<C>(W);
-  if (cudaFuncSetAttribute(adj_column_kernel<C, RT, RTN>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return 1;
+  if (allow_smem(adj_column_kernel<C, RT, RTN>) != cudaSuccess) return 1;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, adj_column_kernel<C, RT, RTN>,
                                                     kAdjThreads, smem) != cudaSuccess)
@@ -907,15 +898,14 @@ cudaError_t launch_adjoint_sweep(const TaskDesc* d_tasks, int n_tasks, int max_W
   if (n_tasks == 0) return cudaSuccess;
   if (precision == NEGF_FP64) {
     const size_t smem = gj_smem<cd>(max_W);
-    cudaError_t e = cudaFuncSetAttribute(adj_sweep_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(adj_sweep_kernel);
     if (e != cudaSuccess) return e;
     adj_sweep_kernel<<<2 * n_tasks, kAdjThreads, smem, s>>>(
         d_tasks, n_tasks, d_wire, d_phi, d_sig, d_ck_off, stride, static_cast<cd*>(d_ck), d_err);
   } else {
     // widths up to 32 and above by kernels of their own; each skips the other's tasks
-    cudaError_t e = bg_smem(adj_sweep32_kernel<1>);
-    if (e == cudaSuccess) e = bg_smem(adj_sweep32_kernel<2>);
+    cudaError_t e = allow_smem(adj_sweep32_kernel<1>);
+    if (e == cudaSuccess) e = allow_smem(adj_sweep32_kernel<2>);
     if (e != cudaSuccess) return e;
     adj_sweep32_kernel<1><<<2 * n_tasks, kBgThreads<1>, sizeof(BgShared), s>>>(
         d_tasks, n_tasks, d_wire, d_phi, d_sig, d_ck_off, stride, static_cast<cf*>(d_ck), d_err);
@@ -938,13 +928,8 @@ cudaError_t launch_adjoint_expand(const TaskDesc* d_tasks, int task0, int n_grou
   if (n_group == 0) return cudaSuccess;
   const int nck = (L + stride - 1) / stride;
   const unsigned blocks = (unsigned)(n_group * 2 * nck);
-  cudaError_t e = precision == NEGF_FP64
-                      ? cudaFuncSetAttribute(adj_expand_kernel<cd>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)gj_smem<cd>(W))
-                      : cudaFuncSetAttribute(adj_expand_kernel<cf>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)gj_smem<cf>(W));
+  const cudaError_t e = precision == NEGF_FP64 ? allow_smem(adj_expand_kernel<cd>)
+                                               : allow_smem(adj_expand_kernel<cf>);
   if (e != cudaSuccess) return e;
   if (precision == NEGF_FP64)
     adj_expand_kernel<cd><<<blocks, kAdjThreads, gj_smem<cd>(W), s>>>(

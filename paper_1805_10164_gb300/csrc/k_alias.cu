@@ -682,8 +682,7 @@ cudaError_t launch_two_level_split(const TaskDesc* d_tasks, int n_tasks, uint32_
       pw = p > pw ? p : pw;
     }
     const size_t smem = (size_t)kL2Warps * 32 * pw * 4;
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
+    const cudaError_t e = allow_smem(kernel);
     if (e != cudaSuccess) return e;
     kernel<<<blocks, 32 * kL2Warps, smem, s>>>(d_tasks, n_tasks, n_jobs, static_cast<R*>(d_weights),
                                                d_tab, d_err);
@@ -710,8 +709,7 @@ cudaError_t launch_energy_tables(const TaskDesc* d_tasks, int n_tasks, const Ene
   while (warps > 1 && per_warp * warps > 200 * 1024) --warps;
   const size_t smem = per_warp * warps;
   if (smem > 220 * 1024) return cudaErrorInvalidValue;     // energy grids beyond shared memory
-  cudaError_t e = cudaFuncSetAttribute(energy_alias_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(energy_alias_kernel);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
@@ -757,8 +755,7 @@ cudaError_t alias_class(const TaskDesc* d_tasks, int n_tasks, uint32_t total_job
   if (blocks > cap_blocks) blocks = cap_blocks;
   // sum-rule tolerance: FP64 weights agree with A to rounding; FP32 propagation to ~1e-5
   const double tol = sizeof(R) == 8 ? 1e-8 : 1e-3;
-  const cudaError_t e = cudaFuncSetAttribute(
-      alias_kernel<R, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(alias_kernel<R, NW>);
   if (e != cudaSuccess) return e;
   alias_kernel<R, NW><<<blocks, groups * 32 * NW, smem, s>>>(
       d_tasks, n_tasks, total_jobs, min_K, max_K, cap, tol, d_weights, d_rowsum, d_mode_w, d_tab,

@@ -226,8 +226,7 @@ __global__ void __launch_bounds__(kThreads, 1) cgemm_tc_kernel(const cf* __restr
 cudaError_t launch_cgemm_tc(const cf* A, const cf* B, cf* Y, int n, int32_t* err,
                             cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(cgemm_tc_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  const cudaError_t e = allow_smem(cgemm_tc_kernel);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((n + kTileC - 1) / kTileC), (unsigned)((n + kTileM - 1) / kTileM));
   cgemm_tc_kernel<<<grid, kThreads, kSmem, s>>>(A, B, Y, n, err);

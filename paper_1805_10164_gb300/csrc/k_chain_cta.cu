@@ -645,8 +645,7 @@ cudaError_t launch_chain_cta(const TaskDesc* d_tasks, const TcJob* d_jobs, uint3
                              uint64_t* d_tab, int32_t* d_err, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   if (n_wide) {
-    e = cudaFuncSetAttribute(chain_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kSmem);
+    e = allow_smem(chain_cta_kernel);
     if (e != cudaSuccess) return e;
     chain_cta_kernel<<<n_wide, kThreads, kSmem, s>>>(
         d_tasks, d_jobs, d_eta32, d_phi32, d_gam, static_cast<const cf*>(d_gL),
@@ -656,8 +655,7 @@ cudaError_t launch_chain_cta(const TaskDesc* d_tasks, const TcJob* d_jobs, uint3
     if (e != cudaSuccess) return e;
   }
   if (n_narrow) {
-    e = cudaFuncSetAttribute(chain_cta_narrow_kernel,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNSmem);
+    e = allow_smem(chain_cta_narrow_kernel);
     if (e != cudaSuccess) return e;
     chain_cta_narrow_kernel<<<n_narrow, kNThreads, kNSmem, s>>>(
         d_tasks, d_jobs + n_wide, d_eta32, d_phi32, d_gam, static_cast<const cf*>(d_gL),

@@ -233,8 +233,7 @@ cudaError_t launch_chain_mid(const TaskDesc* d_tasks, const TcJob* d_jobs, uint3
                              void* d_weights, cudaStream_t s) {
   if (n_jobs == 0) return cudaSuccess;
   const size_t smem = mid_smem_bytes(63);      // 94 KB: two CTAs an SM, as many as registers allow
-  const cudaError_t e = cudaFuncSetAttribute(
-      chain_mid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(chain_mid_kernel);
   if (e != cudaSuccess) return e;
   chain_mid_kernel<<<n_jobs, kMidThreads, smem, s>>>(
       d_tasks, d_jobs, d_eta32, d_phi32, d_gam, static_cast<const cf*>(d_gL),

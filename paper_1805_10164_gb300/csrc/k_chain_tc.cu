@@ -353,8 +353,7 @@ cudaError_t launch_chain_tc(const TaskDesc* d_tasks, int n_tasks, uint32_t n_col
                             const void* d_gR, const void* d_start, void* d_weights,
                             uint64_t* d_tab, void* d_edge, int32_t* d_err, cudaStream_t s) {
   if (n_jobs == 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(chain_tc_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  cudaError_t e = allow_smem(chain_tc_kernel);
   if (e != cudaSuccess) return e;
   chain_tc_kernel<<<n_jobs, kThreads, kSmem, s>>>(
       d_tasks, d_jobs, d_eta32, static_cast<const cf*>(d_gL), static_cast<const cf*>(d_gR),
@@ -363,8 +362,7 @@ cudaError_t launch_chain_tc(const TaskDesc* d_tasks, int n_tasks, uint32_t n_col
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const uint32_t lead_jobs = 2 * n_cols;
-  e = cudaFuncSetAttribute(lead_weights_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kLeadSmem);
+  e = allow_smem(lead_weights_kernel);
   if (e != cudaSuccess) return e;
   lead_weights_kernel<<<lead_jobs, 32, kLeadSmem, s>>>(
       d_tasks, n_tasks, lead_jobs, d_phi32, d_gam, static_cast<const cf*>(d_edge),

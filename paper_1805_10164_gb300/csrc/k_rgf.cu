@@ -1126,8 +1126,7 @@ cudaError_t sweep_fp64(const TaskDesc* d_tasks, int n_tasks, int max_W, const do
                        cd* d_gL, cd* d_gR, int32_t* d_err, cudaStream_t s) {
   // one CTA per sweep: each sweep is a serial chain of W x W inversions, spread one per SM
   const size_t smem = sweep_rows_bytes<cd>(max_W);
-  cudaError_t e = cudaFuncSetAttribute(rgf_sweep_rows_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(rgf_sweep_rows_kernel);
   if (e != cudaSuccess) return e;
   rgf_sweep_rows_kernel<<<2 * n_tasks, kSweepRowsThreads, smem, s>>>(d_tasks, n_tasks, d_wire,
                                                                      d_gL, d_gR, d_err);
@@ -1169,8 +1168,7 @@ cudaError_t columns_impl(const TaskDesc* d_tasks, int n_tasks, uint32_t n_cols, 
     if (e != cudaSuccess) return e;
   } else {
     const size_t smem = diag_cta_bytes(max_W);
-    cudaError_t e = cudaFuncSetAttribute(diag_cta_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(diag_cta_kernel);
     if (e != cudaSuccess) return e;
     diag_cta_kernel<<<n_cols, kSweepThreads, smem, s>>>(
         d_tasks, n_tasks, n_cols, d_wire, d_phi, d_gam, reinterpret_cast<const cd*>(d_gL),
@@ -1197,9 +1195,7 @@ cudaError_t columns_impl(const TaskDesc* d_tasks, int n_tasks, uint32_t n_cols, 
     // SMs' shares of the CTAs are the same work (eight warps a CTA 1.77 ms, two 1.67)
     if (chain_warps <= 0) warps = warps < 2 ? warps : 2;
     const size_t smem_sym = per * warps;
-    cudaError_t e = cudaFuncSetAttribute(chain_sym_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem_sym);
+    const cudaError_t e = allow_smem(chain_sym_kernel);
     if (e != cudaSuccess) return e;
     chain_sym_kernel<<<(n_cols + warps - 1) / warps, 32 * warps, smem_sym, s>>>(
         d_tasks, n_tasks, n_cols, max_W, d_wire, d_phi, d_gam, reinterpret_cast<const cd*>(d_gL),
@@ -1207,8 +1203,7 @@ cudaError_t columns_impl(const TaskDesc* d_tasks, int n_tasks, uint32_t n_cols, 
         reinterpret_cast<double*>(d_w));
     return cudaGetLastError();
   }
-  cudaError_t e = cudaFuncSetAttribute(chain_kernel<C>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(chain_kernel<C>);
   if (e != cudaSuccess) return e;
   chain_kernel<C><<<(jobs + warps - 1) / warps, 32 * warps, smem, s>>>(
       d_tasks, n_tasks, jobs, max_W, d_eta, d_phiR, d_gam, d_gL, d_gR, d_start, d_w, d_green,

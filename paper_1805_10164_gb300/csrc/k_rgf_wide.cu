@@ -270,11 +270,6 @@ __global__ void __launch_bounds__(kBgThreads<NH>, 1) diag_wide_kernel(
   }
 }
 
-template <typename K>
-cudaError_t with_smem(K kernel, size_t smem) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 }  // namespace
 
 cudaError_t launch_rgf_sweep_wide(const TaskDesc* d_tasks, int n_tasks, int max_W,
@@ -282,8 +277,8 @@ cudaError_t launch_rgf_sweep_wide(const TaskDesc* d_tasks, int n_tasks, int max_
                                   cudaStream_t s) {
   // widths 17 .. 32 and 33 .. 64 by kernels of their own; each skips the other's tasks
   const size_t smem = wide_smem_bytes(true);
-  cudaError_t e = with_smem(rgf_sweep_wide_kernel<1>, smem);
-  if (e == cudaSuccess) e = with_smem(rgf_sweep_wide_kernel<2>, smem);
+  cudaError_t e = allow_smem(rgf_sweep_wide_kernel<1>);
+  if (e == cudaSuccess) e = allow_smem(rgf_sweep_wide_kernel<2>);
   if (e != cudaSuccess) return e;
   if (max_W > 32) {
     rgf_sweep_wide_kernel<2><<<2 * n_tasks, kBgThreads<2>, smem, s>>>(d_tasks, n_tasks, d_wire,
@@ -301,8 +296,8 @@ cudaError_t launch_diag_wide(const TaskDesc* d_tasks, int n_tasks, uint32_t n_co
                              const cf* d_gL, const cf* d_gR, cf* d_start, double* d_rowsum,
                              double* d_mode_w, double* d_c, int32_t* d_err, cudaStream_t s) {
   const size_t smem = wide_smem_bytes(false);
-  cudaError_t e = with_smem(diag_wide_kernel<1>, smem);
-  if (e == cudaSuccess) e = with_smem(diag_wide_kernel<2>, smem);
+  cudaError_t e = allow_smem(diag_wide_kernel<1>);
+  if (e == cudaSuccess) e = allow_smem(diag_wide_kernel<2>);
   if (e != cudaSuccess) return e;
   if (max_W > 32) {
     diag_wide_kernel<2><<<n_cols, kBgThreads<2>, smem, s>>>(d_tasks, n_tasks, n_cols, d_wire,

@@ -165,8 +165,7 @@ cudaError_t launch_slice_modes(const TaskDesc* d_tasks, int n_tasks, int max_W, 
                                double* d_phi, float* d_phi32, int32_t* d_err, cudaStream_t s) {
   if (n_tasks == 0) return cudaSuccess;
   const size_t smem = jacobi_smem(max_W);
-  cudaError_t e = cudaFuncSetAttribute(slice_modes_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(slice_modes_kernel, 1024);
   if (e != cudaSuccess) return e;
   slice_modes_kernel<<<n_tasks, kJacobiThreads, smem, s>>>(d_tasks, n_tasks, d_wire, d_phi,
                                                            d_phi32, d_err);

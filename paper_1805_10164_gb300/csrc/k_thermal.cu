@@ -541,8 +541,7 @@ cudaError_t launch_thermal_walk(const TaskDesc* d_tasks, int task0, int M, int w
   const size_t smem = few ? tally : staged;
   auto kern = two_level ? (few ? thermal_few_kernel<true> : thermal_walk_kernel<true>)
                         : (few ? thermal_few_kernel<false> : thermal_walk_kernel<false>);
-  cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   int per_sm = 8;
   if (few || walkers < 8 * lanes) {

@@ -100,6 +100,16 @@ __host__ __device__ inline cf cdiv(cf a, cf b) {
   return cf{(a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d};
 }
 
+// Lets `kernel` take as much dynamic shared memory as a block can have (less what it holds
+// statically).  Always the same limit: the limit belongs to the function, so one set to the size
+// of the launch at hand would be lowered again by another thread's launch before this one, or
+// under the launches of a captured plan.
+template <typename K>
+inline cudaError_t allow_smem(K kernel, int static_bytes = 0) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              227 * 1024 - static_bytes);
+}
+
 // Launchers (each returns the cudaError_t of its launch).
 // Per wire: transverse modes phi (FP64 and FP32 copies, [W][W] at phi_off) and an FP32 copy of
 // eta ([n] at onsite_off / 2); per task: lead eigen self-energies.
