@@ -79,7 +79,7 @@ def tensor_peak(kind):
 # n^2 per task): x 100 per task, x 256 / 8 tasks.
 MEASURED_TRAFFIC = {
     ("walk_kernel", "wire_W10_L50_eta0.05_64E", "f2e0d58f8c278a46"): 133581824,
-    ("chain_cta_kernel", "wire_W64_L1000_eta0.005_256E", "ba6ca48a4cf00100"): 5110117606400,
+    ("chain_cta_kernel", "wire_W64_L1000_eta0.005_256E", "b304b4e2a6487b89"): 5148668288000,
 }
 TRAFFIC_SOURCES = {"walk_kernel": ["k_walk.cu", "philox.cuh"],
                    "chain_cta_kernel": ["k_chain_cta.cu", "level2.cuh"]}
