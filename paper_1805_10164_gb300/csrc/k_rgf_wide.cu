@@ -146,9 +146,12 @@ __device__ __forceinline__ int wide_task(const TaskDesc* tasks, int n_tasks, uin
   return lo;
 }
 
-// Diagonal blocks: one CTA per (task, y) as diag_cta_kernel (k_rgf.cu), same outputs.
+// Diagonal blocks: one CTA per (task, y) as diag_cta_kernel (k_rgf.cu), same outputs.  Two CTAs an SM
+// at W <= 32: with one (106 registers) batches of short narrow wires were slower than by that
+// kernel (W=17 x L=20, 64 energies 0.063 ms there, 0.090 with one, 0.062 with two; W=32 x L=100, 32
+// energies 0.246, 0.240, 0.164).
 template <int NH>
-__global__ void __launch_bounds__(kBgThreads<NH>, 1) diag_wide_kernel(
+__global__ void __launch_bounds__(kBgThreads<NH>, NH == 1 ? 2 : 1) diag_wide_kernel(
     const TaskDesc* __restrict__ tasks, int n_tasks, uint32_t n_jobs,
     const double* __restrict__ wire, const double* __restrict__ phig,
     const double* __restrict__ gam, const cf* __restrict__ gL, const cf* __restrict__ gR,
