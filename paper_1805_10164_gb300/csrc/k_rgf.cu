@@ -1027,9 +1027,7 @@ __global__ void __maxnreg__(80) chain_sym_kernel(const TaskDesc* __restrict__ ta
         wt[(uint64_t)(k * W + a) * K + n + (y - L)] = sum;
       }
       // the injection rows themselves: sum_nu Gamma_nu |(Phi^T X)_{nu b}|^2
-#pragma unroll 1
-      for (int col = 0; col < 2; ++col) {
-        if (k != (col ? L - 1 : 0)) continue;
+      if (k == 0 || k == L - 1) {
         __syncwarp();
 #pragma unroll 1
         for (int idx = lane; idx < WW; idx += 32) {
@@ -1048,7 +1046,9 @@ __global__ void __maxnreg__(80) chain_sym_kernel(const TaskDesc* __restrict__ ta
           double sum = 0.0;
 #pragma unroll 1
           for (int nu = 0; nu < W; ++nu) sum = fma(lgam[nu], sq[nu * W + b], sum);
-          wt[(uint64_t)(row0 + b) * K + n + col] = sum;
+          double* lw = wt + (uint64_t)(row0 + b) * K + n;
+          if (k == 0) lw[0] = sum;
+          if (k == L - 1) lw[1] = sum;
         }
       }
     } else if (k != m0) {
