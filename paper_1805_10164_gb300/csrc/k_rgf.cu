@@ -90,7 +90,17 @@ __global__ void lead_modes_kernel(const TaskDesc* __restrict__ tasks, int n_task
 // of slice L - 1 is never needed).  One thread per entry a >= b, mirrored.  The sum takes W
 // dependent FP64 steps per entry; formed inside every sweep and boundary diagonal block, one
 // CTA at a time on the narrow FP64 pipe, it cost 0.2 ms of latency per kernel at W = 64.
+// Wires of up to kOwnLeadW sites form it within the register sweeps (complex64), which saves the
+// smallest builds a launch: W=1 x L=1 0.099 -> 0.093 ms.
 constexpr int kLeadBlockThreads = 64;
+constexpr int kOwnLeadW = 4;
+
+// entry (a, b) of Phi diag(sigma) Phi^T
+__device__ __forceinline__ cd lead_entry(int a, int b, int W, const double* phi, const cd* sg) {
+  cd acc = mk(0.0, 0.0);
+  for (int m = 0; m < W; ++m) acc = acc + (phi[a * W + m] * phi[b * W + m]) * sg[m];
+  return acc;
+}
 
 template <typename C>
 __global__ void __launch_bounds__(kLeadBlockThreads) lead_block_kernel(
@@ -104,10 +114,7 @@ __global__ void __launch_bounds__(kLeadBlockThreads) lead_block_kernel(
   while (a * (a + 1) / 2 > e) --a;
   while ((a + 1) * (a + 2) / 2 <= e) ++a;
   const int b = e - a * (a + 1) / 2;
-  const double* phi = phig + d.phi_off;
-  const cd* sg = sig + d.lead_off;
-  cd acc = mk(0.0, 0.0);
-  for (int m = 0; m < W; ++m) acc = acc + (phi[a * W + m] * phi[b * W + m]) * sg[m];
+  const cd acc = lead_entry(a, b, W, phig + d.phi_off, sig + d.lead_off);
   C* lb = gL + d.g_off + (uint64_t)(d.L - 1) * W * W;
   lb[a * W + b] = lb[b * W + a] = to_c(acc, C{});
 }
@@ -490,7 +497,9 @@ __device__ __forceinline__ void lead_col(const cf* lb, cf (&x)[W]) {
 // One sweep (task d, direction dir) with W == MAXW known at compile time.
 template <int MAXW>
 __device__ __forceinline__ void sweep_reg_body(const TaskDesc& d, int dir,
-                                               const double* __restrict__ wire, cf* gL, cf* gR,
+                                               const double* __restrict__ wire,
+                                               const double* __restrict__ phig,
+                                               const cd* __restrict__ sig, cf* gL, cf* gR,
                                                int32_t* err, cf* srow) {
   constexpr int W = MAXW;
   const int L = d.L;
@@ -499,7 +508,21 @@ __device__ __forceinline__ void sweep_reg_body(const TaskDesc& d, int dir,
   const double* eta = onsite + d.n;
   const float ttf = (float)(d.t * d.t);     // FP32 on the serial path (FP64 is slow here)
   cf x[MAXW], a[MAXW];
-  lead_col<W>(gL + d.g_off + (uint64_t)(L - 1) * W * W, x);
+  cf* lb = gL + d.g_off + (uint64_t)(L - 1) * W * W;
+  if (W <= kOwnLeadW) {
+    // (one of the two sweeps keeps it for the diagonal blocks)
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      x[i] = cf{0.f, 0.f};
+      if (lane < W) {
+        x[i] = to_c(lead_entry(i > lane ? i : lane, i > lane ? lane : i, W, phig + d.phi_off,
+                               sig + d.lead_off), cf{});
+        if (dir == 0) lb[i * W + lane] = x[i];
+      }
+    }
+  } else {
+    lead_col<W>(lb, x);
+  }
   cf* out = dir == 0 ? gL : gR;
   const int jc = lane < W ? lane : 0;
   // the next slice's onsite energy and dephasing are fetched one step ahead
@@ -567,14 +590,15 @@ struct SweepReg {
 
 // One warp per (task, direction), tasks of width W <= kSweepRegMaxW.
 __global__ void rgf_sweep_reg_kernel(const TaskDesc* __restrict__ tasks, int n_tasks,
-                                     const double* __restrict__ wire, cf* gL, cf* gR,
-                                     int32_t* err) {
+                                     const double* __restrict__ wire,
+                                     const double* __restrict__ phig,
+                                     const cd* __restrict__ sig, cf* gL, cf* gR, int32_t* err) {
   const int job = blockIdx.x;
   if (job >= 2 * n_tasks) return;
   __shared__ __align__(16) cf s_row[34];
   const TaskDesc d = tasks[job >> 1];
-  if (d.L < 2) return;
-  by_width<SweepReg>(d.W, d, job & 1, wire, gL, gR, err, s_row);
+  if (d.L < 2 && d.W > kOwnLeadW) return;
+  by_width<SweepReg>(d.W, d, job & 1, wire, phig, sig, gL, gR, err, s_row);
 }
 
 // last task whose first job index (`first(t)`) is <= job
@@ -1134,10 +1158,12 @@ cudaError_t sweep_fp64(const TaskDesc* d_tasks, int n_tasks, int max_W, const do
 }
 
 cudaError_t sweep_fp32(const TaskDesc* d_tasks, int n_tasks, int max_W, const double* d_wire,
-                       cf* d_gL, cf* d_gR, int32_t* d_err, cudaStream_t s) {
+                       const double* d_phi, const cd* d_sig, cf* d_gL, cf* d_gR, int32_t* d_err,
+                       cudaStream_t s) {
   // one warp per sweep for the tasks of width <= 16 (it skips wider ones), a CTA per sweep for
   // the rest
-  rgf_sweep_reg_kernel<<<2 * n_tasks, 32, 0, s>>>(d_tasks, n_tasks, d_wire, d_gL, d_gR, d_err);
+  rgf_sweep_reg_kernel<<<2 * n_tasks, 32, 0, s>>>(d_tasks, n_tasks, d_wire, d_phi, d_sig, d_gL,
+                                                  d_gR, d_err);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || max_W <= kSweepRegMaxW) return e;
   return launch_rgf_sweep_wide(d_tasks, n_tasks, max_W, d_wire, d_gL, d_gR, d_err, s);
@@ -1234,10 +1260,12 @@ cudaError_t launch_rgf_sweep(const TaskDesc* d_tasks, int n_tasks, int max_W, in
                             : sweep_fp64(d_tasks, n_tasks, max_W, d_wire, static_cast<cd*>(d_gL),
                                          static_cast<cd*>(d_gR), d_err, s);
   }
-  e = lead_blocks(d_tasks, n_tasks, max_W, d_phi, d_sig, static_cast<cf*>(d_gL), s);
+  e = max_W > kOwnLeadW
+          ? lead_blocks(d_tasks, n_tasks, max_W, d_phi, d_sig, static_cast<cf*>(d_gL), s)
+          : cudaSuccess;
   return e != cudaSuccess ? e
-                          : sweep_fp32(d_tasks, n_tasks, max_W, d_wire, static_cast<cf*>(d_gL),
-                                       static_cast<cf*>(d_gR), d_err, s);
+                          : sweep_fp32(d_tasks, n_tasks, max_W, d_wire, d_phi, d_sig,
+                                       static_cast<cf*>(d_gL), static_cast<cf*>(d_gR), d_err, s);
 }
 
 cudaError_t launch_block_columns(const TaskDesc* d_tasks, int n_tasks, uint32_t n_cols,
